@@ -352,14 +352,15 @@ static int upload(const HostMech& hm, chem_mech_s* cm) {
       for (int i = 0; i < 7; ++i) gneg[((size_t)k * 2 + rg) * 8 + i] = (double)(-c[i] * kExpScale);
     }
   }
-  std::vector<double> exptab(256);
-  for (int j = 0; j < 256; ++j) exptab[j] = (double)std::exp2((long double)j / 256.0L);
-  std::vector<double> logtab(3 * 97);
+  // fixed-point tables of the kernels' exponentials and logarithm (see internal.h)
+  std::vector<unsigned long long> exptab(256);
+  for (int j = 0; j < 256; ++j)
+    exptab[j] = (unsigned long long)std::round(std::ldexp(std::exp2((long double)j / 256.0L), 63));
+  std::vector<long long> logtab(2 * 97);
   for (int j = 96; j <= 192; ++j) {
-    const long double F = (long double)j / 128.0L;
-    logtab[3 * (j - 96)] = (double)F;
-    logtab[3 * (j - 96) + 1] = (double)(1.0L / F);
-    logtab[3 * (j - 96) + 2] = (double)std::log(F);
+    const long double G = std::round(1024.0L * 128.0L / (long double)j);
+    logtab[2 * (j - 96)] = (long long)G;
+    logtab[2 * (j - 96) + 1] = (long long)std::round(std::ldexp(-std::log(G / 1024.0L), 63));
   }
   // FP32 copies for the learned step's update (its enthalpy, element sums and T(h) run in
   // FP32): NASA-7 c_p/R (5) and h/RT (6) per species and range, 1/W, composition / W
@@ -502,8 +503,8 @@ static int upload(const HostMech& hm, chem_mech_s* cm) {
   m.troe = (const double*)(b + otroe); m.sp_ptr = (const int*)(b + optr);
   m.sp_rxn = (const int*)(b + orxn); m.sp_nu = (const double*)(b + onu);
   m.gneg = (const double*)(b + ogn);
-  m.exptab = (const double*)(b + oexp);
-  m.logtab = (const double*)(b + olog);
+  m.exptab = (const unsigned long long*)(b + oexp);
+  m.logtab = (const longlong2*)(b + olog);
   m.compW = (const double*)(b + ocw);
   m.th32 = (const float*)(b + oth32);
   m.invW32 = (const float*)(b + oiw32);

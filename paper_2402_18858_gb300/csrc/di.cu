@@ -220,7 +220,7 @@ __device__ __forceinline__ CellP cell_p(double p) {
 template <bool JAC>
 __device__ __forceinline__ void troe_phase(const DevMech& m, const WarpMem& w, double invT, double ctot, int lane) {
   const int nT = m.I - m.n_tb_end;
-  const double* __restrict__ et = m.exptab;
+  const unsigned long long* __restrict__ et = m.exptab;
   const double kS = 0.4342944819032518;   // 1 / ln 10
   for (int t0 = 0; t0 < 2 * nT; t0 += 32) {
     const int t = t0 + lane, jt = t >> 1, q = t & 1;
@@ -296,7 +296,7 @@ __device__ void rhs_eval(const DevMech& m, const WarpMem& w, const CellP& cp0, c
   const int K = m.K, I = m.I;
   const double T = comp_get<NPL>(y, K);
   const double lnT = log_t(T, m.logtab), RT = kR * T;
-  const double* __restrict__ et = m.exptab;
+  const unsigned long long* __restrict__ et = m.exptab;
   // T >= T_mid on the bit patterns (both positive: they order like the values)
   const int hi = __double_as_longlong(T) >= __double_as_longlong(m.Tmid) ? 1 : 0;
   // pass 1: c_p/R per species and the two mixture sums sum Y/W and sum Y c_p/(R W)
@@ -358,9 +358,15 @@ __device__ void rhs_eval(const DevMech& m, const WarpMem& w, const CellP& cp0, c
       w.C[k] = Ck;
       w.hRT[k] = hRT;
       sp.hRT[s] = hRT;
-      const double e = exp_s256(ng, et);
+      // e and 1/e from the one fixed-point argument
+      const long long gf = fix_s256(ng);
+      double e = exp2_fix(gf, et), ie = exp2_fix(-gf, et);
+      if (s256_end(ng)) {
+        e = exp_s256_end(ng, e);
+        ie = rcp_nr(e);
+      }
       w.eg[k] = e * P0RT;
-      w.ieg[k] = rcp_nr(e) * (two ? RTP0 * Ck : RTP0);
+      w.ieg[k] = ie * (two ? RTP0 * Ck : RTP0);
     }
   }
   // exponential rounds: k_f of every non-falloff reaction (into w.q, read back by the same
@@ -1261,17 +1267,17 @@ __global__ void __launch_bounds__(128) jacobian_kernel(DevMech m, int64_t n, int
   }
 }
 
-__global__ void exp_selftest_kernel(const double* __restrict__ tab, int64_t n, const double* x, double* y) {
+__global__ void exp_selftest_kernel(const unsigned long long* __restrict__ tab, int64_t n, const double* x, double* y) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     y[i] = exp_t(x[i], tab);
 }
 
-__global__ void exp256_selftest_kernel(const double* __restrict__ tab, int64_t n, const double* x, double* y) {
+__global__ void exp256_selftest_kernel(const unsigned long long* __restrict__ tab, int64_t n, const double* x, double* y) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     y[i] = exp_s256(x[i], tab);
 }
 
-__global__ void log_selftest_kernel(const double* __restrict__ tab, int64_t n, const double* x, double* y) {
+__global__ void log_selftest_kernel(const longlong2* __restrict__ tab, int64_t n, const double* x, double* y) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     y[i] = log_t(x[i], tab);
 }

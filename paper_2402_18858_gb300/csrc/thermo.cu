@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(128) thermo_kernel(DevMech m, int64_t n, int64
       // species pair, no cancellation); mixture-averaged conductivity 0.5 (sum X lambda +
       // 1 / sum X / lambda).  Exponentials by the table-driven exp, reciprocals by Newton's
       // iteration (both within about 2 ulp).
-      const double* __restrict__ et = m.exptab;
+      const unsigned long long* __restrict__ et = m.exptab;
       double X[KC ? KC : CHEM_MAX_SPECIES], sm[KC ? KC : CHEM_MAX_SPECIES];
       double vx[KC ? KC : CHEM_MAX_SPECIES], wx[KC ? KC : CHEM_MAX_SPECIES];
       const double isYW = rcp_nr(sYW);
