@@ -330,7 +330,8 @@ static int upload(const HostMech& hm, chem_mech_s* cm) {
   // g/RT = h/RT - s/R = (a1 - a7) - a1 ln T - a2 T/2 - a3 T^2/6 - a4 T^3/12 - a5 T^4/20 + a6/T
   // of the NASA-7 fit (coefficients a1..a7), shifted by the element potentials,
   // g' = g - sum_r P[k][r] g_ref_r (formed in long double, rounded once)
-  std::vector<double> gneg((size_t)K * 2 * 8, 0.0);
+  const int KP = (K + 31) & ~31;
+  std::vector<double> gneg((size_t)2 * 7 * KP, 0.0);
   for (int rg = 0; rg < 2; ++rg) {
     auto gcoef = [&](int k, long double* c) {
       const double* a = &hm.nasa[(size_t)k * 14 + 7 * rg];
@@ -349,7 +350,7 @@ static int upload(const HostMech& hm, chem_mech_s* cm) {
         gcoef(refs[r], cr);
         for (int i = 0; i < 7; ++i) c[i] -= (long double)Pm[(size_t)k * R + r] * cr[i];
       }
-      for (int i = 0; i < 7; ++i) gneg[((size_t)k * 2 + rg) * 8 + i] = (double)(-c[i] * kExpScale);
+      for (int i = 0; i < 7; ++i) gneg[((size_t)rg * 7 + i) * KP + k] = (double)(-c[i] * kExpScale);
     }
   }
   // fixed-point tables of the kernels' exponentials and logarithm (see internal.h)
@@ -362,6 +363,10 @@ static int upload(const HostMech& hm, chem_mech_s* cm) {
     logtab[2 * (j - 96)] = (long long)G;
     logtab[2 * (j - 96) + 1] = (long long)std::round(std::ldexp(-std::log(G / 1024.0L), 63));
   }
+  std::vector<double> rth((size_t)2 * 11 * KP, 0.0);
+  for (int rg = 0; rg < 2; ++rg)
+    for (int i = 0; i < 11; ++i)
+      for (int k = 0; k < K; ++k) rth[((size_t)rg * 11 + i) * KP + k] = th[((size_t)k * 2 + rg) * kThermoStride + i];
   // FP32 copies for the learned step's update (its enthalpy, element sums and T(h) run in
   // FP32): NASA-7 c_p/R (5) and h/RT (6) per species and range, 1/W, composition / W
   std::vector<float> th32((size_t)K * 2 * 16, 0.0f), invW32(K), compW32((size_t)K * E);
@@ -378,22 +383,24 @@ static int upload(const HostMech& hm, chem_mech_s* cm) {
   // exponential items of the right-hand side (see DevMech::xarg)
   const int nT = I - n_tb_end;
   const int n_x = n_tb_end + 5 * nT;
-  std::vector<double> xarg((size_t)std::max(n_x, 1) * 4, 0.0);
-  for (int jj = 0; jj < n_tb_end; ++jj)
-    for (int c = 0; c < 3; ++c) xarg[(size_t)jj * 4 + c] = arr[(size_t)jj * 4 + c];
+  const int XP = std::max((n_x + 31) & ~31, 32);
+  std::vector<double> xarg((size_t)4 * XP, 0.0);
+  auto item = [&](int t, double x0, double x1, double x2, double x3) {
+    const double x[4] = {x0, x1, x2, x3};
+    for (int c = 0; c < 4; ++c) xarg[(size_t)c * XP + t] = (double)((long double)x[c] * kExpScale);
+  };
+  for (int jj = 0; jj < n_tb_end; ++jj) item(jj, arr[(size_t)jj * 4], arr[(size_t)jj * 4 + 1], arr[(size_t)jj * 4 + 2], 0.0);
   for (int jt = 0; jt < nT; ++jt) {
-    const int jj = n_tb_end + jt;
-    const double* a = &arr[(size_t)jj * 4];
-    const double* tp = &troe[(size_t)jj * 8];
-    double* x = &xarg[(size_t)(n_tb_end + 5 * jt) * 4];
-    x[0] = a[0]; x[1] = a[1]; x[2] = a[2];                            // k_inf
-    x[4] = tp[0] - a[0]; x[5] = tp[1] - a[1]; x[6] = tp[2] - a[2];    // k_0 / k_inf
-    x[11] = -tp[4];                                                   // exp(-T / T***)
-    x[15] = -tp[5];                                                   // exp(-T / T*)
-    if (tp[7] != 0.0) x[18] = tp[6];                                  // exp(-T** / T)
-    else x[16] = -1e300;                                              // absent term: 0
+    const double* a = &arr[(size_t)(n_tb_end + jt) * 4];
+    const double* tp = &troe[(size_t)(n_tb_end + jt) * 8];
+    const int t = n_tb_end + 5 * jt;
+    item(t, a[0], a[1], a[2], 0.0);                                    // k_inf
+    item(t + 1, tp[0] - a[0], tp[1] - a[1], tp[2] - a[2], 0.0);        // k_0 / k_inf
+    item(t + 2, 0.0, 0.0, 0.0, -tp[4]);                                // exp(-T / T***)
+    item(t + 3, 0.0, 0.0, 0.0, -tp[5]);                                // exp(-T / T*)
+    if (tp[7] != 0.0) item(t + 4, 0.0, 0.0, tp[6], 0.0);               // exp(-T** / T)
+    else item(t + 4, -1e300, 0.0, 0.0, 0.0);                           // absent term: 0
   }
-  for (auto& v : xarg) v = (double)((long double)v * kExpScale);
 
   std::vector<int> sp_ptr(K + 1, 0), sp_rxn;
   std::vector<double> sp_nu;
@@ -426,10 +433,11 @@ static int upload(const HostMech& hm, chem_mech_s* cm) {
       const int a = (int)std::fabs(nu);
       if ((double)a != std::fabs(nu) || a < 1 || a > 3) ok = false;
     }
-    if (runs > 3 * K || runs > 255) ok = false;   // the runs' slots reuse 3K dead doubles
+    if (runs > 3 * K || runs > 254) ok = false;   // the runs' slots and the padding's reuse 3K + 2 dead doubles
     if (ok) {
       for (int k = 0; k < K; ++k) run_ptr[k] = sp_ptr[k] < sp_ptr[k + 1] ? run_of_entry[sp_ptr[k]] : -1;
       run_ptr[K] = runs;
+      for (unsigned int& e : bal) e = (unsigned int)runs << 4;   // padding: nu = 0, a slot of no species
       for (int k = K - 1; k >= 0; --k) if (run_ptr[k] < 0) run_ptr[k] = run_ptr[k + 1];
       for (int e = 0; e < E_inc; ++e) {
         const int lane = e / bal_P, i = e % bal_P;
@@ -443,15 +451,13 @@ static int upload(const HostMech& hm, chem_mech_s* cm) {
     }
   }
   // two-partner reaction table (see DevMech::rsp2)
-  std::vector<int> rsp2((size_t)std::max(I, 1) * 4, K);
+  std::vector<unsigned int> rsp2((size_t)std::max(I, 1), 0u);
   int arity2 = 1;
   for (int jj = 0; jj < I; ++jj) {
     const int* s = &rsp[(size_t)jj * 8];
     if (s[3] > 2 || s[7] > 2) arity2 = 0;
-    rsp2[(size_t)jj * 4 + 0] = s[0];
-    rsp2[(size_t)jj * 4 + 1] = s[3] > 1 ? s[1] : K;
-    rsp2[(size_t)jj * 4 + 2] = s[4];
-    rsp2[(size_t)jj * 4 + 3] = s[7] > 1 ? s[5] : K;
+    rsp2[jj] = (unsigned int)s[0] | (unsigned int)(s[3] > 1 ? s[1] : K) << 8 | (unsigned int)s[4] << 16 |
+               (unsigned int)(s[7] > 1 ? s[5] : K) << 24;
   }
   const int nnz = std::max((int)sp_rxn.size(), 1);
   sp_rxn.resize(nnz, 0);
@@ -474,7 +480,7 @@ static int upload(const HostMech& hm, chem_mech_s* cm) {
   size_t oexs = add(ex_sp.data(), ex_sp.size() * 4), oexa = add(ex_a.data(), ex_a.size() * 8);
   size_t otroe = add(troe.data(), troe.size() * 8), optr = add(sp_ptr.data(), sp_ptr.size() * 4);
   size_t orxn = add(sp_rxn.data(), sp_rxn.size() * 4), onu = add(sp_nu.data(), sp_nu.size() * 8);
-  size_t ogn = add(gneg.data(), gneg.size() * 8);
+  size_t ogn = add(gneg.data(), gneg.size() * 8), orth = add(rth.data(), rth.size() * 8);
   size_t oth32 = add(th32.data(), th32.size() * 4), oiw32 = add(invW32.data(), invW32.size() * 4);
   size_t ocw32 = add(compW32.data(), compW32.size() * 4);
   size_t oexp = add(exptab.data(), exptab.size() * 8), ocw = add(compW.data(), compW.size() * 8);
@@ -503,6 +509,8 @@ static int upload(const HostMech& hm, chem_mech_s* cm) {
   m.troe = (const double*)(b + otroe); m.sp_ptr = (const int*)(b + optr);
   m.sp_rxn = (const int*)(b + orxn); m.sp_nu = (const double*)(b + onu);
   m.gneg = (const double*)(b + ogn);
+  m.KP = KP;
+  m.rth = (const double*)(b + orth);
   m.exptab = (const unsigned long long*)(b + oexp);
   m.logtab = (const longlong2*)(b + olog);
   m.compW = (const double*)(b + ocw);
@@ -510,12 +518,13 @@ static int upload(const HostMech& hm, chem_mech_s* cm) {
   m.invW32 = (const float*)(b + oiw32);
   m.compW32 = (const float*)(b + ocw32);
   m.n_x = n_x;
+  m.XP = XP;
   m.xarg = (const double*)(b + oxa);
   m.bal_P = bal_P;
   m.bal = (const unsigned int*)(b + obal);
   m.run_ptr = (const int*)(b + orun);
   m.arity2 = arity2;
-  m.rsp2 = (const int4*)(b + orsp2);
+  m.rsp2 = (const unsigned int*)(b + orsp2);
   cm->dmem = d;
   cm->K = K; cm->I = I; cm->E = m.E;
   for (int k = 0; k < K; ++k)

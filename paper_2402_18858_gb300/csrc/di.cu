@@ -12,6 +12,15 @@
 // norms, step-size factors) runs in FP32, the solution, the rates, the equilibrium
 // constants and the LU stay FP64.  Every loop is bounded and every failure becomes a
 // per-cell status code.
+//
+// Measured latencies behind the loop shapes (one warp per SM): FP64 unit 64 cycles per warp
+// instruction in each of the SM's four sub-partitions (about 105 until another unit can use the
+// result), shared-memory load 34, L1 hit 39, L2 hit 243-311.  With shared memory taking all but 28 KB
+// of L1 the mechanism tables come from L2, so they are laid out for contiguous warp loads, loops
+// over reactions and factor columns issue the loads of several iterations ahead of the FP64 chain,
+// and 12 warps per SM (3 per sub-partition) run in one block.  12,345 30-species cells: 128.2 ->
+// 125.0 ms; 150 cells (one warp per SM, tables in L1): 23.2 -> 18.7 ms; 3,001 53-species cells: 146.6
+// -> 143.8 ms.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -86,17 +95,17 @@ struct WarpMem {
   double* kre;    // I   effective reverse coefficient
   double* aux;    // I   d q / d [M] factor (third-body: q0, Troe: dk/dM (fwd - rev/Kc))
   double* qT;     // I   d q / d T at fixed C
-  double* tr;     // 14 per Troe reaction: [0..4] the exponentials of the rounds, [10] k,
-                  // [11] dk/d[M], [12] dln k/dT (the other slots are spare)
+  double* tr;     // 8 per Troe reaction: [0..4] the exponentials of the rounds, [5] k,
+                  // [6] dk/d[M], [7] dln k/dT
   double* invd;   // n   reciprocal pivots
-  double* ru;     // 64  step-size change matrix (0..24) and R(f) (32..56)
+  double* ru;     // 50  step-size change matrix (0..24) and R(f) (25..49)
   int* perm;      // n   row permutation of the LU
   int ld;
 };
 
 __host__ __device__ inline int pad_ld(int n) { return n | 1; }
 
-constexpr int kTroeSlots = 14;
+constexpr int kTroeSlots = 8;
 
 // doubles per warp: matrices (optional) + species + reactions + Troe scratch + small vectors
 // The per-reaction Jacobian terms (kfe, kre, aux, qT) are live only between rhs_eval<true> and
@@ -126,7 +135,7 @@ __host__ __device__ inline size_t warp_doubles(int K, int I, int n, int nT, bool
     alias = mats && jac && jac_terms_in_lu(I, n);
   }
   d += 5 * (size_t)K + 3 + (jac && !alias ? 5 : 1) * (size_t)(I > 0 ? I : 1) + (size_t)kTroeSlots * nT;
-  d += (size_t)n + 64 + (size_t)(n + 1) / 2 + 2;
+  d += (size_t)n + 50 + (size_t)(n + 1) / 2 + 2;
   return (d + 1) & ~size_t(1);   // keep 16-byte alignment per warp
 }
 
@@ -178,7 +187,7 @@ __device__ __forceinline__ WarpMem carve(double* base, int K, int I, int n, int 
   }
   w.tr = p; p += (size_t)kTroeSlots * nT;
   w.invd = p; p += n;
-  w.ru = p; p += 64;
+  w.ru = p; p += 50;
   w.perm = (int*)p;
   return w;
 }
@@ -215,7 +224,7 @@ __device__ __forceinline__ CellP cell_p(double p) {
 // of 1/(den^2 + x^2) (den = n - 0.14 x), lane 1 of 1/(1 + P_r).  Lane 0 then forms
 // F = exp(ln F_cent den^2 / (den^2 + x^2)) (the base-10 form of log10 F = log10 F_cent /
 // (1 + (x/den)^2) with both sides times ln 10) and k = k_inf P_r/(1 + P_r) F.
-// Results: [10] k, [11] dk/d[M], [12] d ln k/dT at fixed [M].
+// Results: [5] k, [6] dk/d[M], [7] d ln k/dT at fixed [M].
 // ------------------------------------------------------------------------------------------
 template <bool JAC>
 __device__ __forceinline__ void troe_phase(const DevMech& m, const WarpMem& w, double invT, double ctot, int lane) {
@@ -262,7 +271,7 @@ __device__ __forceinline__ void troe_phase(const DevMech& m, const WarpMem& w, d
     if (act && q == 0) {
       const double F = exp_t(lc * d2 * iS, et);
       const double kinf = r[0];
-      r[10] = kinf * Pr * ipr * F;
+      r[5] = kinf * Pr * ipr * F;
       if (JAC) {
         const double L = kS * lc;   // log10 F_cent
         const double Fc = v;
@@ -275,12 +284,12 @@ __device__ __forceinline__ void troe_phase(const DevMech& m, const WarpMem& w, d
         const double dFc = -(1.0 - aa) * iT3 * r[2] - aa * iT1 * r[3] + __ldg(tp + 6) * invT * invT * r[4];
         const double df1dx = nn / d2;
         const double gg = -L * 2.0 * f1 / (opf * opf) * df1dx;          // d log F / d log Pr
-        r[11] = k0 * F * (ipr * ipr + gg * ipr);
+        r[6] = k0 * F * (ipr * ipr + gg * ipr);
         const double df1dL = df1dx * (-0.67) + (-x / d2) * (-1.27);
         const double dlogFdL = 1.0 / opf - L * 2.0 * f1 / (opf * opf) * df1dL;
         const double dlnkinf = __ldg(ar + 1) * invT + __ldg(ar + 2) * invT * invT;
         const double dlnk0 = __ldg(tp + 1) * invT + __ldg(tp + 2) * invT * invT;
-        r[12] = dlnkinf + (ipr + gg) * (dlnk0 - dlnkinf) + dlogFdL * dFc / Fc;
+        r[7] = dlnkinf + (ipr + gg) * (dlnk0 - dlnkinf) + dlogFdL * dFc / Fc;
       }
     }
   }
@@ -301,14 +310,17 @@ __device__ void rhs_eval(const DevMech& m, const WarpMem& w, const CellP& cp0, c
   const int hi = __double_as_longlong(T) >= __double_as_longlong(m.Tmid) ? 1 : 0;
   // pass 1: c_p/R per species and the two mixture sums sum Y/W and sum Y c_p/(R W)
   double sYW = 0.0, cpp = 0.0, ywr[NPL];
+  const int KP = m.KP;
+  const double* rth = m.rth + (size_t)hi * 11 * KP;
+  const double* rgn = m.gneg + (size_t)hi * 7 * KP;
 #pragma unroll
   for (int s = 0; s < NPL; ++s) {
     const int k = lane + 32 * s;
     ywr[s] = 0.0;
     sp.cpR[s] = sp.dcpR[s] = sp.hRT[s] = 0.0;
     if (k < K) {
-      const double* a = m.th + ((size_t)k * 2 + hi) * kThermoStride;
-      const double a0 = __ldg(a + 0), a1 = __ldg(a + 1), a2 = __ldg(a + 2), a3 = __ldg(a + 3), a4 = __ldg(a + 4);
+      const double a0 = __ldg(rth + k), a1 = __ldg(rth + KP + k), a2 = __ldg(rth + 2 * KP + k);
+      const double a3 = __ldg(rth + 3 * KP + k), a4 = __ldg(rth + 4 * KP + k);
       const double cpR = a0 + T * (a1 + T * (a2 + T * (a3 + T * a4)));
       if (JAC) sp.dcpR[s] = a1 + T * (2.0 * a2 + T * (3.0 * a3 + T * 4.0 * a4));
       const double yw = y[s] * __ldg(m.invW + k);
@@ -346,14 +358,13 @@ __device__ void rhs_eval(const DevMech& m, const WarpMem& w, const CellP& cp0, c
       w.ieg[K] = 1.0;
     }
     if (k < K) {
-      const double* a = m.th + ((size_t)k * 2 + hi) * kThermoStride;
-      const double hRT = __ldg(a + 5) + T * (__ldg(a + 6) + T * (__ldg(a + 7) + T * (__ldg(a + 8) + T * __ldg(a + 9))))
-                         + __ldg(a + 10) * invT;
-      const double* gc = m.gneg + ((size_t)k * 2 + hi) * 8;
-      const double2 g01 = __ldg((const double2*)gc), g23 = __ldg((const double2*)(gc + 2));
-      const double2 g45 = __ldg((const double2*)(gc + 4));
-      const double g6 = __ldg(gc + 6);
-      const double ng = fma(T, T * fma(T, fma(T, g45.y, g45.x), g23.y) + g23.x, fma(g6, invT, fma(g01.y, lnT, g01.x)));
+      double a[6], g[7];
+#pragma unroll
+      for (int i = 0; i < 6; ++i) a[i] = __ldg(rth + (5 + i) * KP + k);
+#pragma unroll
+      for (int i = 0; i < 7; ++i) g[i] = __ldg(rgn + i * KP + k);
+      const double hRT = a[0] + T * (a[1] + T * (a[2] + T * (a[3] + T * a[4]))) + a[5] * invT;
+      const double ng = fma(T, T * fma(T, fma(T, g[5], g[4]), g[3]) + g[2], fma(g[6], invT, fma(g[1], lnT, g[0])));
       const double Ck = rho * ywr[s];
       w.C[k] = Ck;
       w.hRT[k] = hRT;
@@ -375,15 +386,15 @@ __device__ void rhs_eval(const DevMech& m, const WarpMem& w, const CellP& cp0, c
   const int nb = m.n_tb_end;
   // whole rounds before the first falloff item: k_f only, no T term in the argument
   const int n_plain = (nb / 32) * 32;
-  for (int t = lane; t < n_plain; t += 32) {
-    const double2 x01 = __ldg((const double2*)(m.xarg + 4 * (size_t)t));
-    const double x2 = __ldg(m.xarg + 4 * (size_t)t + 2);
-    w.q[t] = exp_s256(fma(-x2, invT, fma(x01.y, lnT, x01.x)), et);
-  }
+  const int XP = m.XP;
+  const double* xa = m.xarg + lane;
+#pragma unroll 2
+  for (int t = 0; t < n_plain; t += 32)
+    w.q[t + lane] = exp_s256(fma(-__ldg(xa + 2 * XP + t), invT, fma(__ldg(xa + XP + t), lnT, __ldg(xa + t))), et);
+#pragma unroll 2
   for (int t = n_plain + lane; t < m.n_x; t += 32) {
-    const double2 x01 = __ldg((const double2*)(m.xarg + 4 * (size_t)t));
-    const double2 x23 = __ldg((const double2*)(m.xarg + 4 * (size_t)t + 2));
-    const double e = exp_s256(fma(x23.y, T, fma(-x23.x, invT, fma(x01.y, lnT, x01.x))), et);
+    const double* x = m.xarg + t;
+    const double e = exp_s256(fma(__ldg(x + 3 * XP), T, fma(-__ldg(x + 2 * XP), invT, fma(__ldg(x + XP), lnT, __ldg(x)))), et);
     if (t < nb) {
       w.q[t] = e;
     } else {
@@ -397,11 +408,19 @@ __device__ void rhs_eval(const DevMech& m, const WarpMem& w, const CellP& cp0, c
     // q_j = k_f (C_a C_b - K_c^-1 C_c C_d) = k_f (C_a C_b - (e_a e_b)(u_c u_d)) with
     // e = exp(-g'/RT) p0/RT and u = exp(g'/RT) (RT/p0) C; a missing partner is the sentinel 1.
     // No predication on the reaction's arity, one rounding in the difference.
-    for (int j = lane; j < I; j += 32) {
-      const int4 rs = __ldg(m.rsp2 + j);
+    auto net = [&](unsigned int rs, double kf) {
+      const int r0 = rs & 255u, r1 = (rs >> 8) & 255u, p0 = (rs >> 16) & 255u, p1 = rs >> 24;
+      return kf * fma(-(w.eg[r0] * w.eg[r1]), w.ieg[p0] * w.ieg[p1], w.C[r0] * w.C[r1]);
+    };
+    // whole rounds of elementary reactions, then the rest
+    const int n_full = (m.n_elem / 32) * 32;
+#pragma unroll 2
+    for (int j = lane; j < n_full; j += 32) w.q[j] = net(__ldg(m.rsp2 + j), w.q[j]);
+    for (int j = n_full + lane; j < I; j += 32) {
+      const unsigned int rs = __ldg(m.rsp2 + j);
       double kf;
       if (j < nb) kf = w.q[j];
-      else kf = w.tr[kTroeSlots * (j - nb) + 10];
+      else kf = w.tr[kTroeSlots * (j - nb) + 5];
       if (j >= m.n_elem && j < nb) {
         double M = ctot;
 #pragma unroll
@@ -411,7 +430,7 @@ __device__ void rhs_eval(const DevMech& m, const WarpMem& w, const CellP& cp0, c
         }
         kf *= M;
       }
-      w.q[j] = kf * fma(-(w.eg[rs.x] * w.eg[rs.y]), w.ieg[rs.z] * w.ieg[rs.w], w.C[rs.x] * w.C[rs.y]);
+      w.q[j] = net(rs, kf);
     }
   } else
   for (int j = lane; j < I; j += 32) {
@@ -424,8 +443,8 @@ __device__ void rhs_eval(const DevMech& m, const WarpMem& w, const CellP& cp0, c
       if (JAC) dlnkf = __ldg(m.arr + 4 * (size_t)j + 1) * invT + __ldg(m.arr + 4 * (size_t)j + 2) * invT * invT;
     } else {
       const double* r = w.tr + kTroeSlots * (j - nb);
-      kf = r[10];
-      if (JAC) { dkdM = r[11]; dlnkf = r[12]; }
+      kf = r[5];
+      if (JAC) { dkdM = r[6]; dlnkf = r[7]; }
     }
     double fwd = w.C[ra.x], ratio = w.eg[ra.x], sh = 0.0;
     if (JAC) sh = -w.hRT[ra.x];
@@ -463,18 +482,27 @@ __device__ void rhs_eval(const DevMech& m, const WarpMem& w, const CellP& cp0, c
   double* part = w.g;   // g, eg and ieg are dead from here on: 3K slots for the runs
   if (P > 0) {
     double acc = 0.0;
-    for (int i = 0; i < P; ++i) {
-      const unsigned int e = __ldg(m.bal + (size_t)i * 32 + lane);
-      if (e & 3u) {
-        // nu = +-1, +-2, +-3 built from its bits (no FP64 conversion)
-        const unsigned int a = e & 3u;
-        const unsigned int hw = (a == 1u ? 0x3ff00000u : a == 2u ? 0x40000000u : 0x40080000u) | ((e & 4u) << 29);
-        acc = fma(__hiloint2double((int)hw, 0), w.q[e >> 12], acc);
-        if (e & 8u) {
-          part[(e >> 4) & 255u] = acc;
-          acc = 0.0;
-        }
-      }
+    const unsigned int* bl = m.bal + lane;
+    // one entry: nu = 0 (padding), +-1, +-2, +-3 built from its bits (no FP64 conversion); the run's
+    // slot takes the partial sum every time, its last entry leaves the whole and clears it
+    auto entry = [&](unsigned int e, double q) {
+      const unsigned int a = e & 3u;
+      const unsigned int hw = (a == 0u ? 0u : a == 1u ? 0x3ff00000u : a == 2u ? 0x40000000u : 0x40080000u) | ((e & 4u) << 29);
+      acc = fma(__hiloint2double((int)hw, 0), q, acc);
+      part[(e >> 4) & 255u] = acc;
+      if (e & 8u) acc = 0.0;
+    };
+    for (int i = 0; i < P; i += 4) {
+      // four entries' table words and net rates are loaded ahead of the chain of FMAs
+      unsigned int e[4];
+      double q[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) e[u] = i + u < P ? __ldg(bl + (i + u) * 32) : 0u;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) q[u] = w.q[e[u] >> 12];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (i + u < P) entry(e[u], q[u]);
     }
     __syncwarp();
   }
@@ -736,13 +764,23 @@ __device__ void lu_solve(const WarpMem& w, int n, double (&x)[NPL], int lane) {
     }
     b[s] = r < n ? v : 0.0;
   }
-  // L (unit lower) forward substitution
-  for (int col = 0; col < n - 1; ++col) {
-    const double xc = comp_get<NPL>(b, col);
+  // L (unit lower) forward substitution.  The factors' entries of four columns are loaded ahead of
+  // the chain of broadcasts and FMAs (0 where the lane's row takes no part)
+  const double* row[NPL];
 #pragma unroll
-    for (int s = 0; s < NPL; ++s) {
-      const int r = lane + 32 * s;
-      if (r > col && r < n) b[s] -= w.LU[(size_t)r * ld + col] * xc;
+  for (int s = 0; s < NPL; ++s) row[s] = w.LU + (size_t)min(lane + 32 * s, n - 1) * ld;
+  for (int c0 = 0; c0 < n - 1; c0 += 4) {
+    double l[4][NPL];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int s = 0; s < NPL; ++s) l[q][s] = (lane + 32 * s > c0 + q && lane + 32 * s < n) ? row[s][c0 + q] : 0.0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (c0 + q >= n - 1) break;
+      const double xc = comp_get<NPL>(b, c0 + q);
+#pragma unroll
+      for (int s = 0; s < NPL; ++s) b[s] = fma(-l[q][s], xc, b[s]);
     }
   }
   // diag(1/u_kk), then the unit upper factor backward
@@ -751,12 +789,18 @@ __device__ void lu_solve(const WarpMem& w, int n, double (&x)[NPL], int lane) {
     const int r = lane + 32 * s;
     if (r < n) b[s] *= w.invd[r];
   }
-  for (int col = n - 1; col > 0; --col) {
-    const double xc = comp_get<NPL>(b, col);
+  for (int c0 = n - 1; c0 > 0; c0 -= 4) {
+    double l[4][NPL];
 #pragma unroll
-    for (int s = 0; s < NPL; ++s) {
-      const int r = lane + 32 * s;
-      if (r < col) b[s] -= w.LU[(size_t)r * ld + col] * xc;
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int s = 0; s < NPL; ++s) l[q][s] = (lane + 32 * s < c0 - q) ? row[s][c0 - q] : 0.0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (c0 - q <= 0) break;
+      const double xc = comp_get<NPL>(b, c0 - q);
+#pragma unroll
+      for (int s = 0; s < NPL; ++s) b[s] = fma(-l[q][s], xc, b[s]);
     }
   }
 #pragma unroll
@@ -859,11 +903,11 @@ __device__ void rescale_D(double (&D)[kMaxOrd + 3][NPL], int order, double fct, 
 #pragma unroll
     for (int mm = 2; mm <= kMaxOrd; ++mm)
       if (mm <= rc.i) r *= (double)(mm - 1) - fl;
-    w.ru[32 + lane] = r * rc.inv_fact;
+    w.ru[25 + lane] = r * rc.inv_fact;
   }
   __syncwarp();
   if (lane < 25) {
-    const double* Ri = w.ru + 32 + (rc.i - 1) * 5;
+    const double* Ri = w.ru + 25 + (rc.i - 1) * 5;
     const double* Uj = kRescaleU + (rc.j - 1);
     double a = Ri[0] * __ldg(Uj);
 #pragma unroll
@@ -1173,7 +1217,7 @@ __device__ __forceinline__ void load_cell(const DevMech& m, int64_t col, int64_t
 }
 
 template <int NPL>
-__global__ void __launch_bounds__(NPL == 1 ? 160 : 128, 2) di_kernel(DevMech m, int64_t n, int64_t ld, double dt, double* T,
+__global__ void __launch_bounds__(NPL == 1 ? 384 : 256, 1) di_kernel(DevMech m, int64_t n, int64_t ld, double dt, double* T,
                                                  const double* p, double* Y, const int32_t* idx, DiOpts o,
                                                  int32_t* status, int32_t* stats, unsigned int* queue,
                                                  size_t warp_bytes, const int32_t* n_dev) {
@@ -1184,11 +1228,11 @@ __global__ void __launch_bounds__(NPL == 1 ? 160 : 128, 2) di_kernel(DevMech m, 
                           NPL > 1 && di_use_j32(m.K, m.I, m.n, nT));
   // n_dev (optional): the number of entries of idx actually filled, known only on the device
   const int64_t n_eff = n_dev ? min(n, (int64_t)max(*n_dev, 0)) : n;
-  while (true) {
-    unsigned int slot = 0;
-    if (lane == 0) slot = atomicAdd(queue, 1u);
-    slot = __shfl_sync(FULLMASK, slot, 0);
-    if ((int64_t)slot >= n_eff) break;
+  // the first cells are dealt out one per block and then round again (few cells spread over the
+  // SMs), the rest come from the queue as warps fall free
+  const unsigned int n_warps = gridDim.x * (blockDim.x >> 5);
+  unsigned int slot = wid * gridDim.x + blockIdx.x;
+  for (; (int64_t)slot < n_eff; slot = __shfl_sync(FULLMASK, slot, 0)) {
     const int64_t col = idx ? (int64_t)idx[slot] : (int64_t)slot;
     double z[NPL];
     int cnt[4];
@@ -1216,6 +1260,7 @@ __global__ void __launch_bounds__(NPL == 1 ? 160 : 128, 2) di_kernel(DevMech m, 
         stats[2 * n + slot] = cnt[2];
         stats[3 * n + slot] = cnt[3];
       }
+      slot = n_warps + atomicAdd(queue, 1u);
     }
   }
 }
@@ -1392,39 +1437,42 @@ int launch_di(const DevMech& m, int64_t n, int64_t ld, double dt, double* T, con
               int32_t* stats, unsigned int* queue, cudaStream_t s, const int32_t* n_dev) {
   const size_t wb = di_smem_per_warp(m);
   DiOpts o{opts.rtol, opts.atol_Y, opts.atol_T, opts.newton_tol, opts.max_steps, opts.jac_max_age};
-  int wpb;
-  size_t smem;
-  int rc;
   if (n > (int64_t)0x7fffffff) return set_error(CHEM_E_ARG, "chem_step_di: too many cells in one call");
-  int dev = 0, per_sm = 0, max_threads_sm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&max_threads_sm, cudaDevAttrMaxThreadsPerMultiProcessor, dev);
-  // persistent grid: the block shape (1..5 warps) that keeps the most warps resident per SM
-  auto best_shape = [&](auto kern) -> int {
-    int best_w = 0;
-    const int optin = smem_optin();
+  auto launch = [&](auto kern) -> int {
+    // block shape (warps) that keeps the most warps resident per SM, the widest of equal ones (its
+    // warps are dealt evenly to the SM's four sub-partitions, each of which has its own FP64 unit)
+    const int optin = smem_optin(), sms = sm_count();
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
     cudaFuncAttributes fa;
     if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) return cuda_check(cudaGetLastError(), "di_kernel attributes");
-    for (int cand = 5; cand >= 1; --cand) {
-      if ((size_t)cand * wb > (size_t)optin || 32 * cand > fa.maxThreadsPerBlock) continue;
+    int wpb = 0, per_sm = 0;
+    for (int cand = fa.maxThreadsPerBlock / 32; cand >= 1; --cand) {
+      if ((size_t)cand * wb > (size_t)optin) continue;
       int blocks = 0;
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kern, 32 * cand, (size_t)cand * wb);
-      if (blocks * cand > best_w) { best_w = blocks * cand; wpb = cand; per_sm = blocks; }
+      if (blocks * cand > wpb * per_sm) { wpb = cand; per_sm = blocks; }
     }
-    smem = (size_t)wpb * wb;
-    return best_w > 0 ? CHEM_OK : set_error(CHEM_E_UNSUPPORTED, "mechanism needs more shared memory per warp than the device has");
+    if (wpb == 0) return set_error(CHEM_E_UNSUPPORTED, "mechanism needs more shared memory per warp than the device has");
+    // fewer cells than resident warps: one smaller block per SM, and what shared memory it leaves
+    // goes to L1, which then holds the mechanism tables
+    if (n < (int64_t)sms * wpb * per_sm) {
+      wpb = (int)std::min<int64_t>(wpb, std::max<int64_t>(1, (n + sms - 1) / sms));
+      per_sm = std::max<int64_t>(1, (n + (int64_t)sms * wpb - 1) / ((int64_t)sms * wpb));
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)std::min<int64_t>((n + wpb - 1) / wpb, (int64_t)sms * per_sm));
+    cfg.blockDim = dim3(32 * wpb);
+    cfg.dynamicSmemBytes = (size_t)wpb * wb;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr[0].val.sharedMemCarveout = (unsigned)std::min<size_t>(100, (per_sm * (cfg.dynamicSmemBytes + 1024) * 100 + 228 * 1024 - 1) / (228 * 1024));
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cuda_check(cudaLaunchKernelEx(&cfg, kern, m, n, ld, dt, T, p, Y, idx, o, status, stats, queue, wb, n_dev),
+                      "di_kernel launch");
   };
-  if (m.n <= 32) {
-    if ((rc = best_shape(di_kernel<1>))) return rc;
-    const int64_t grid = std::min<int64_t>((n + wpb - 1) / wpb, (int64_t)sm_count() * per_sm);
-    di_kernel<1><<<(int)grid, 32 * wpb, smem, s>>>(m, n, ld, dt, T, p, Y, idx, o, status, stats, queue, wb, n_dev);
-  } else {
-    if ((rc = best_shape(di_kernel<2>))) return rc;
-    const int64_t grid = std::min<int64_t>((n + wpb - 1) / wpb, (int64_t)sm_count() * per_sm);
-    di_kernel<2><<<(int)grid, 32 * wpb, smem, s>>>(m, n, ld, dt, T, p, Y, idx, o, status, stats, queue, wb, n_dev);
-  }
-  return cuda_check(cudaGetLastError(), "di_kernel launch");
+  return m.n <= 32 ? launch(di_kernel<1>) : launch(di_kernel<2>);
 }
 
 }  // namespace chem

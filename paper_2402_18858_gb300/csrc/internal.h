@@ -41,12 +41,17 @@ struct DevMech {
   const int* sp_ptr;       // [K+1]
   const int* sp_rxn;       // [nnz]
   const double* sp_nu;     // [nnz]
+  // Species polynomials of the right-hand side, one lane per species: [2 ranges][11][KP], KP = K
+  // rounded up to 32: c_p/R (a1..a5), h/RT (a1 a2/2 .. a5/5 a6), so that a warp's load of one
+  // coefficient is contiguous.
+  int KP;
+  const double* rth;
   // -g'_k/RT for the equilibrium constants, g' = g_k - sum_r P[k][r] g_{ref_r} the free
   // energy shifted by element potentials (P = composition x pinv(reference compositions));
   // balanced reactions cancel the shift exactly, and it keeps exp(-g') products in range.
   // Per species and range one polynomial: [0] + [1] ln T + T ([2] + T ([3] + T ([4] + T [5])))
-  // + [6] / T ([7] unused), times 256/ln 2 (exp_s256's argument unit).
-  const double* gneg;      // [K][2][8]
+  // + [6] / T, times 256/ln 2 (exp_s256's argument unit).
+  const double* gneg;      // [2][7][KP]
   const unsigned long long* exptab;   // [256] 2^(j/256) 2^63, the table of the exponentials below
   const longlong2* logtab;   // [97] {G, -ln(G 2^-10) 2^63}, j = 96..192: the table of log_t below
   const double* compW;     // [K][E] element counts divided by the molar mass (mol/kg)
@@ -56,22 +61,22 @@ struct DevMech {
   const float* compW32;    // [K][E]
   // Exponentials of one right-hand side, in lane rounds: item t < n_tb_end is k_f of reaction
   // t, then 5 per falloff reaction (k_inf, k_0/k_inf, the three F_cent terms).  Item t is
-  // exp(x) with x = xarg[4t] + xarg[4t+1] ln T - xarg[4t+2] / T + xarg[4t+3] T, the
+  // exp(x) with x = xarg[0][t] + xarg[1][t] ln T - xarg[2][t] / T + xarg[3][t] T, the
   // coefficients stored times 256/ln 2 (exp_s256's argument unit).
-  int n_x;
-  const double* xarg;      // [n_x][4]
+  int n_x, XP;             // XP: n_x rounded up to 32
+  const double* xarg;      // [4][XP]
   // Lane-balanced species production rates: lane L walks entries bal[i*32 + L], i < bal_P,
   // each |nu| (bits 0-1), nu < 0 (bit 2), last entry of its run (bit 3), run slot (bits 4-11),
-  // reaction (bits 12-31); 0 = padding.  wdot_k = sum of the run slots run_ptr[k] ..
+  // reaction (bits 12-31); |nu| = 0: padding, in a slot of no species.  wdot_k = sum of the run slots run_ptr[k] ..
   // run_ptr[k+1] - 1 in order.  bal_P = 0: walk the incidence lists instead.
   int bal_P;
   const unsigned int* bal;   // [bal_P][32]
   const int* run_ptr;        // [K+1]
   // Two-partner form of the reactions, used when every reaction has at most two reactants and
-  // two products (arity2 = 1): (r0, r1, p0, p1), a missing partner pointing at the sentinel
-  // slot K of the per-species shared-memory vectors, which holds 1.
+  // two products (arity2 = 1): r0 | r1 << 8 | p0 << 16 | p1 << 24, a missing partner pointing at the
+  // sentinel slot K of the per-species shared-memory vectors, which holds 1.
   int arity2;
-  const int4* rsp2;          // [I]
+  const unsigned int* rsp2;  // [I]
 };
 
 // FP64 -> FP32 on the integer pipe for values that only steer heuristics or feed FP32 sums
