@@ -231,6 +231,29 @@ static int upload(const HostMech& hm, chem_mech_s* cm) {
       wB[(size_t)k * K + j] = std::pow(hm.W[j] / hm.W[k], 0.25);
     }
   }
+  // tables of the FP64 properties' fixed-point sums (see DevMech::fxC)
+  std::vector<int2> fxC((size_t)K * K);
+  std::vector<double> fx_tr((size_t)K * 11);
+  int fxC_e = 0;
+  {
+    const double w_min = *std::min_element(hm.W.begin(), hm.W.end());
+    const long double top = 1.0L / std::sqrt(2.0L * w_min);
+    std::frexp(top, &fxC_e);
+    fxC_e = 54 - fxC_e;   // the largest constant below 2^54
+    for (int k = 0; k < K; ++k) {
+      for (int j = 0; j < K; ++j)
+        fxC[(size_t)k * K + j] = fix_limbs(
+            (long long)std::round(std::ldexp(1.0L / std::sqrt((long double)hm.W[k] + (long double)hm.W[j]), fxC_e)));
+      double* t = &fx_tr[(size_t)k * 11];
+      for (int i = 0; i < 4; ++i) {
+        t[i] = -0.5 * hm.transport[(size_t)k * 8 + i];
+        t[4 + i] = hm.transport[(size_t)k * 8 + 4 + i];
+      }
+      t[8] = 1.0 / hm.W[k];
+      t[9] = std::sqrt(hm.W[k]);
+      t[10] = (double)std::sqrt(std::sqrt((long double)hm.W[k]));
+    }
+  }
   std::vector<int> rsp((size_t)std::max(I, 1) * 8, -1), ex_sp((size_t)std::max(I, 1) * kMaxEx, -1);
   std::vector<double> arr((size_t)std::max(I, 1) * 4, 0.0), ex_a((size_t)std::max(I, 1) * kMaxEx, 0.0);
   std::vector<double> troe((size_t)std::max(I, 1) * 8, 0.0);
@@ -481,6 +504,8 @@ static int upload(const HostMech& hm, chem_mech_s* cm) {
   size_t otroe = add(troe.data(), troe.size() * 8), optr = add(sp_ptr.data(), sp_ptr.size() * 4);
   size_t orxn = add(sp_rxn.data(), sp_rxn.size() * 4), onu = add(sp_nu.data(), sp_nu.size() * 8);
   size_t ogn = add(gneg.data(), gneg.size() * 8), orth = add(rth.data(), rth.size() * 8);
+  size_t ofxC = add(fxC.data(), fxC.size() * 8);
+  size_t ofxt = add(fx_tr.data(), fx_tr.size() * 8);
   size_t oth32 = add(th32.data(), th32.size() * 4), oiw32 = add(invW32.data(), invW32.size() * 4);
   size_t ocw32 = add(compW32.data(), compW32.size() * 4);
   size_t oexp = add(exptab.data(), exptab.size() * 8), ocw = add(compW.data(), compW.size() * 8);
@@ -510,6 +535,9 @@ static int upload(const HostMech& hm, chem_mech_s* cm) {
   m.sp_rxn = (const int*)(b + orxn); m.sp_nu = (const double*)(b + onu);
   m.gneg = (const double*)(b + ogn);
   m.KP = KP;
+  m.fxC = (const int2*)(b + ofxC);
+  m.fx_tr = (const double*)(b + ofxt);
+  m.fxC_e = fxC_e;
   m.rth = (const double*)(b + orth);
   m.exptab = (const unsigned long long*)(b + oexp);
   m.logtab = (const longlong2*)(b + olog);

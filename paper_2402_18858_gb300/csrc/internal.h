@@ -31,6 +31,12 @@ struct DevMech {
   const double* th;        // [K][2][17]: low/high range; cp/R(5), h/RT(6: a1 a2/2 a3/3 a4/4 a5/5 a6),
                            //   s/R(6: a1 a2 a3/2 a4/3 a5/4 a7)
   const double* tr;        // [K][8]: ln mu fit (4), ln lambda fit (4)
+  // FP64 properties in fixed point (thermo.cu): limbs (fix_limbs) of the Wilke constants
+  // (W_j + W_k)^(-1/2) times 2^fxC_e; per species the transport exponents -ln(mu)/2 and ln(lambda) (4 +
+  // 4 coefficients in ln T) and 1/W, W^(1/2), W^(1/4)
+  const int2* fxC;         // [K][K]
+  int fxC_e;
+  const double* fx_tr;     // [K][11]
   const double* wA;        // [K][K] 1/sqrt(8 (1 + W_k/W_j))
   const double* wB;        // [K][K] (W_j/W_k)^(1/4)
   const int* rsp;          // [I][8]: r0 r1 r2 nr p0 p1 p2 np
@@ -136,6 +142,42 @@ __device__ __forceinline__ double fix63_to_double(long long v) {
   return __longlong_as_double((long long)(r | ((unsigned long long)v & 0x8000000000000000ull)));
 }
 
+// v 2^x as a double, rounded to nearest, for results in the normal range (integer pipe)
+__device__ __forceinline__ double fix_to_double(long long v, int x) {
+  unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+  if (a == 0ull) return 0.0;
+  const int n = __clzll((long long)a);
+  a <<= n;
+  const unsigned long long r = (a >> 11) + ((a >> 10) & 1ull) + ((unsigned long long)(1085 - n + x) << 52);
+  return __longlong_as_double((long long)(r | ((unsigned long long)v & 0x8000000000000000ull)));
+}
+
+// Two limbs (h, l) of a fixed-point number f = h 2^27 + l, |f| <= 2^55, l in [-2^26, 2^26), |h| <=
+// 2^28.  Products of such numbers with table entries of |f| <= 2^54 are summed as hh += h1 h2 and
+// hl += h1 l2 + l1 h2 (32 x 32 + 64-bit multiply-adds); up to 63 terms stay within 64 bits, and the
+// omitted l1 l2 is below 2^-57 of the largest possible product.
+__host__ __device__ __forceinline__ int2 fix_limbs(long long f) {
+  const int h = (int)((f + (1ll << 26)) >> 27);
+  return make_int2(h, (int)((unsigned int)f - ((unsigned int)h << 27)));
+}
+// x as limbs of x 2^(1077 - E), E >= the biased exponent of x (the largest of its vector): 55 bits,
+// rounded (cutting off would bias a sum of K terms by K/2 units)
+__device__ __forceinline__ int2 fix_vec(double x, int E) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int e = (int)((unsigned int)(b >> 52) & 0x7ffu);
+  const long long f = (long long)((((((b & 0xfffffffffffffull) | 0x10000000000000ull) << 3) >> min(E - e, 63)) + 1ull) >> 1);
+  return fix_limbs((long long)b < 0 ? -f : f);
+}
+__device__ __forceinline__ int fix_exp(double x) {
+  return (int)((unsigned int)((unsigned long long)__double_as_longlong(x) >> 52) & 0x7ffu);
+}
+// a += x y, 64-bit (one instruction; the C expression takes two to three times its cycles)
+__device__ __forceinline__ void mad_wide(long long& a, int x, int y) {
+  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(a) : "r"(x), "r"(y));
+}
+// the sum of products hh 2^54 + hl 2^27 in units of 2^53
+__device__ __forceinline__ long long fix_fold(long long hh, long long hl) { return (hh << 1) + ((hl + (1ll << 25)) >> 26); }
+
 // 2^(f 2^-45 / 256), |f| < 2^63: f = 2^45 n + fraction, n = 256 k + j.  With v = fraction ln2/256 <
 // 2.71e-3, 2^(j/256) e^v has e^v - 1 from its degree-5 Taylor polynomial (truncation below 6e-19)
 // as P = (e^v - 1) 2^72: v in 64 bits, v^2/2 in 64, the rest (below 2^-28) in 32.  tab[j] =
@@ -161,10 +203,13 @@ __device__ __forceinline__ double exp2_fix(long long f, const unsigned long long
 
 // exp(x): the argument in units of ln2/256 is x log2(e) 256 (the integer part of log2(e) exact).
 // Arguments below -708 return 0, above 709.78 return +inf, NaN propagates.
-__device__ __forceinline__ double exp_t(double x, const unsigned long long* __restrict__ tab) {
+__device__ __forceinline__ long long fix_exp_arg(double x) {
   const unsigned long long X = fix_mag(x, 53);
   const long long F = (long long)(X + __umul64hi(X, 0x71547652B82FE177ull));   // |x| log2(e) 2^53
-  double res = exp2_fix(__double_as_longlong(x) < 0 ? -F : F, tab);
+  return __double_as_longlong(x) < 0 ? -F : F;
+}
+__device__ __forceinline__ double exp_t(double x, const unsigned long long* __restrict__ tab) {
+  double res = exp2_fix(fix_exp_arg(x), tab);
   // |x| >= 708, inf and NaN, detected on the exponent bits (rare branch)
   if (((unsigned int)((unsigned long long)__double_as_longlong(x) >> 32) & 0x7fffffffu) >= 0x40862000u) {
     if (x != x) res = x;
