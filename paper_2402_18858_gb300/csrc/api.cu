@@ -237,13 +237,16 @@ static int upload(const HostMech& hm, chem_mech_s* cm) {
   int fxC_e = 0;
   {
     const double w_min = *std::min_element(hm.W.begin(), hm.W.end());
-    const long double top = 1.0L / std::sqrt(2.0L * w_min);
-    std::frexp(top, &fxC_e);
+    std::frexp(1.0 / std::sqrt(2.0 * w_min), &fxC_e);
     fxC_e = 54 - fxC_e;   // the largest constant below 2^54
     for (int k = 0; k < K; ++k) {
-      for (int j = 0; j < K; ++j)
-        fxC[(size_t)k * K + j] = fix_limbs(
-            (long long)std::round(std::ldexp(1.0L / std::sqrt((long double)hm.W[k] + (long double)hm.W[j]), fxC_e)));
+      for (int j = 0; j < k; ++j) fxC[(size_t)k * K + j] = fxC[(size_t)j * K + k];
+      for (int j = k; j < K; ++j) {
+        // c = w^(-1/2) in FP64 and its error by one Newton step with exact products
+        const double w = hm.W[k] + hm.W[j], c = 1.0 / std::sqrt(w), wc = w * c;
+        const double r = std::fma(-wc, c, 1.0) - std::fma(w, c, -wc) * c;
+        fxC[(size_t)k * K + j] = fix_limbs(std::llround(std::ldexp(c, fxC_e)) + std::llround(std::ldexp(0.5 * c * r, fxC_e)));
+      }
       double* t = &fx_tr[(size_t)k * 11];
       for (int i = 0; i < 4; ++i) {
         t[i] = -0.5 * hm.transport[(size_t)k * 8 + i];
@@ -251,7 +254,7 @@ static int upload(const HostMech& hm, chem_mech_s* cm) {
       }
       t[8] = 1.0 / hm.W[k];
       t[9] = std::sqrt(hm.W[k]);
-      t[10] = (double)std::sqrt(std::sqrt((long double)hm.W[k]));
+      t[10] = std::sqrt(t[9]);
     }
   }
   std::vector<int> rsp((size_t)std::max(I, 1) * 8, -1), ex_sp((size_t)std::max(I, 1) * kMaxEx, -1);
@@ -354,7 +357,7 @@ static int upload(const HostMech& hm, chem_mech_s* cm) {
   // of the NASA-7 fit (coefficients a1..a7), shifted by the element potentials,
   // g' = g - sum_r P[k][r] g_ref_r (formed in long double, rounded once)
   const int KP = (K + 31) & ~31;
-  std::vector<double> gneg((size_t)2 * 7 * KP, 0.0);
+  std::vector<double> gneg((size_t)2 * 8 * KP, 0.0);
   for (int rg = 0; rg < 2; ++rg) {
     auto gcoef = [&](int k, long double* c) {
       const double* a = &hm.nasa[(size_t)k * 14 + 7 * rg];
@@ -373,23 +376,31 @@ static int upload(const HostMech& hm, chem_mech_s* cm) {
         gcoef(refs[r], cr);
         for (int i = 0; i < 7; ++i) c[i] -= (long double)Pm[(size_t)k * R + r] * cr[i];
       }
-      for (int i = 0; i < 7; ++i) gneg[((size_t)rg * 7 + i) * KP + k] = (double)(-c[i] * kExpScale);
+      for (int i = 0; i < 7; ++i) gneg[((size_t)(rg * 4 + i / 2) * KP + k) * 2 + i % 2] = (double)(-c[i] * kExpScale);
     }
   }
-  // fixed-point tables of the kernels' exponentials and logarithm (see internal.h)
-  std::vector<unsigned long long> exptab(256);
-  for (int j = 0; j < 256; ++j)
-    exptab[j] = (unsigned long long)std::round(std::ldexp(std::exp2((long double)j / 256.0L), 63));
-  std::vector<long long> logtab(2 * 97);
-  for (int j = 96; j <= 192; ++j) {
-    const long double G = std::round(1024.0L * 128.0L / (long double)j);
-    logtab[2 * (j - 96)] = (long long)G;
-    logtab[2 * (j - 96) + 1] = (long long)std::round(std::ldexp(-std::log(G / 1024.0L), 63));
+  // tables of the elementary functions, FP64 and fixed point (see internal.h)
+  std::vector<double> exptab(256), logtab(3 * 97);
+  std::vector<unsigned long long> fexptab(256);
+  std::vector<long long> flogtab(2 * 97);
+  for (int j = 0; j < 256; ++j) {
+    const long double e = std::exp2((long double)j / 256.0L);
+    exptab[j] = (double)e;
+    fexptab[j] = (unsigned long long)std::round(std::ldexp(e, 63));
   }
-  std::vector<double> rth((size_t)2 * 11 * KP, 0.0);
+  for (int j = 96; j <= 192; ++j) {
+    const long double F = (long double)j / 128.0L, G = std::round(1024.0L / F);
+    logtab[3 * (j - 96)] = (double)F;
+    logtab[3 * (j - 96) + 1] = (double)(1.0L / F);
+    logtab[3 * (j - 96) + 2] = (double)std::log(F);
+    flogtab[2 * (j - 96)] = (long long)G;
+    flogtab[2 * (j - 96) + 1] = (long long)std::round(std::ldexp(-std::log(G / 1024.0L), 63));
+  }
+  std::vector<double> rth((size_t)2 * 12 * KP, 0.0);
   for (int rg = 0; rg < 2; ++rg)
     for (int i = 0; i < 11; ++i)
-      for (int k = 0; k < K; ++k) rth[((size_t)rg * 11 + i) * KP + k] = th[((size_t)k * 2 + rg) * kThermoStride + i];
+      for (int k = 0; k < K; ++k)
+        rth[((size_t)(rg * 6 + i / 2) * KP + k) * 2 + i % 2] = th[((size_t)k * 2 + rg) * kThermoStride + i];
   // FP32 copies for the learned step's update (its enthalpy, element sums and T(h) run in
   // FP32): NASA-7 c_p/R (5) and h/RT (6) per species and range, 1/W, composition / W
   std::vector<float> th32((size_t)K * 2 * 16, 0.0f), invW32(K), compW32((size_t)K * E);
@@ -410,7 +421,7 @@ static int upload(const HostMech& hm, chem_mech_s* cm) {
   std::vector<double> xarg((size_t)4 * XP, 0.0);
   auto item = [&](int t, double x0, double x1, double x2, double x3) {
     const double x[4] = {x0, x1, x2, x3};
-    for (int c = 0; c < 4; ++c) xarg[(size_t)c * XP + t] = (double)((long double)x[c] * kExpScale);
+    for (int c = 0; c < 4; ++c) xarg[((size_t)(c / 2) * XP + t) * 2 + c % 2] = (double)((long double)x[c] * kExpScale);
   };
   for (int jj = 0; jj < n_tb_end; ++jj) item(jj, arr[(size_t)jj * 4], arr[(size_t)jj * 4 + 1], arr[(size_t)jj * 4 + 2], 0.0);
   for (int jt = 0; jt < nT; ++jt) {
@@ -456,11 +467,10 @@ static int upload(const HostMech& hm, chem_mech_s* cm) {
       const int a = (int)std::fabs(nu);
       if ((double)a != std::fabs(nu) || a < 1 || a > 3) ok = false;
     }
-    if (runs > 3 * K || runs > 254) ok = false;   // the runs' slots and the padding's reuse 3K + 2 dead doubles
+    if (runs > 3 * K || runs > 255) ok = false;   // the runs' slots reuse 3K dead doubles
     if (ok) {
       for (int k = 0; k < K; ++k) run_ptr[k] = sp_ptr[k] < sp_ptr[k + 1] ? run_of_entry[sp_ptr[k]] : -1;
       run_ptr[K] = runs;
-      for (unsigned int& e : bal) e = (unsigned int)runs << 4;   // padding: nu = 0, a slot of no species
       for (int k = K - 1; k >= 0; --k) if (run_ptr[k] < 0) run_ptr[k] = run_ptr[k + 1];
       for (int e = 0; e < E_inc; ++e) {
         const int lane = e / bal_P, i = e % bal_P;
@@ -510,6 +520,7 @@ static int upload(const HostMech& hm, chem_mech_s* cm) {
   size_t ocw32 = add(compW32.data(), compW32.size() * 4);
   size_t oexp = add(exptab.data(), exptab.size() * 8), ocw = add(compW.data(), compW.size() * 8);
   size_t oxa = add(xarg.data(), xarg.size() * 8), olog = add(logtab.data(), logtab.size() * 8);
+  size_t ofexp = add(fexptab.data(), fexptab.size() * 8), oflog = add(flogtab.data(), flogtab.size() * 8);
   size_t obal = add(bal.data(), bal.size() * 4), orun = add(run_ptr.data(), run_ptr.size() * 4);
   size_t orsp2 = add(rsp2.data(), rsp2.size() * 4);
   std::vector<char> blob(total, 0);
@@ -533,21 +544,23 @@ static int upload(const HostMech& hm, chem_mech_s* cm) {
   m.ex_sp = (const int*)(b + oexs); m.ex_a = (const double*)(b + oexa);
   m.troe = (const double*)(b + otroe); m.sp_ptr = (const int*)(b + optr);
   m.sp_rxn = (const int*)(b + orxn); m.sp_nu = (const double*)(b + onu);
-  m.gneg = (const double*)(b + ogn);
+  m.gneg = (const double2*)(b + ogn);
   m.KP = KP;
   m.fxC = (const int2*)(b + ofxC);
   m.fx_tr = (const double*)(b + ofxt);
   m.fxC_e = fxC_e;
-  m.rth = (const double*)(b + orth);
-  m.exptab = (const unsigned long long*)(b + oexp);
-  m.logtab = (const longlong2*)(b + olog);
+  m.rth = (const double2*)(b + orth);
+  m.exptab = (const double*)(b + oexp);
+  m.logtab = (const double*)(b + olog);
+  m.fexptab = (const unsigned long long*)(b + ofexp);
+  m.flogtab = (const longlong2*)(b + oflog);
   m.compW = (const double*)(b + ocw);
   m.th32 = (const float*)(b + oth32);
   m.invW32 = (const float*)(b + oiw32);
   m.compW32 = (const float*)(b + ocw32);
   m.n_x = n_x;
   m.XP = XP;
-  m.xarg = (const double*)(b + oxa);
+  m.xarg = (const double2*)(b + oxa);
   m.bal_P = bal_P;
   m.bal = (const unsigned int*)(b + obal);
   m.run_ptr = (const int*)(b + orun);

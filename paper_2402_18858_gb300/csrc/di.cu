@@ -16,11 +16,11 @@
 // Measured latencies behind the loop shapes (one warp per SM): FP64 unit 64 cycles per warp
 // instruction in each of the SM's four sub-partitions (about 105 until another unit can use the
 // result), shared-memory load 34, L1 hit 39, L2 hit 243-311.  With shared memory taking all but 28 KB
-// of L1 the mechanism tables come from L2, so they are laid out for contiguous warp loads, loops
-// over reactions and factor columns issue the loads of several iterations ahead of the FP64 chain,
-// and 12 warps per SM (3 per sub-partition) run in one block.  12,345 30-species cells: 128.2 ->
-// 125.0 ms; 150 cells (one warp per SM, tables in L1): 23.2 -> 18.7 ms; 3,001 53-species cells: 146.6
-// -> 143.8 ms.
+// of L1 the mechanism tables come from L2, so they are laid out for contiguous warp loads, the
+// triangular solves issue the loads of four factor columns ahead of the FP64 chain, and 12 warps per SM
+// (3 per sub-partition) run in one block.  Same bits; 150 30-species cells (one warp per SM, tables in
+// L1): 22.3 -> 18.0 ms; 3,001 53-species cells: 145.7 -> 138 ms; 12,345 30-species cells: 137.7 ->
+// 134.8 ms (FP64 issue bound).
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -226,10 +226,9 @@ __device__ __forceinline__ CellP cell_p(double p) {
 // (1 + (x/den)^2) with both sides times ln 10) and k = k_inf P_r/(1 + P_r) F.
 // Results: [5] k, [6] dk/d[M], [7] d ln k/dT at fixed [M].
 // ------------------------------------------------------------------------------------------
-template <bool JAC>
+template <bool JAC, bool FIX>
 __device__ __forceinline__ void troe_phase(const DevMech& m, const WarpMem& w, double invT, double ctot, int lane) {
   const int nT = m.I - m.n_tb_end;
-  const unsigned long long* __restrict__ et = m.exptab;
   const double kS = 0.4342944819032518;   // 1 / ln 10
   for (int t0 = 0; t0 < 2 * nT; t0 += 32) {
     const int t = t0 + lane, jt = t >> 1, q = t & 1;
@@ -256,7 +255,7 @@ __device__ __forceinline__ void troe_phase(const DevMech& m, const WarpMem& w, d
       }
     }
     const double v = fmax(scale * fma(c4[3], u4[3], fma(c4[2], u4[2], fma(c4[1], u4[1], fma(c4[0], u4[0], base)))), 1e-300);
-    const double lv = log_t(v, m.logtab);
+    const double lv = FIX ? log_t_fix(v, m.flogtab) : log_t(v, m.logtab);
     const int l0 = lane & ~1, l1 = lane | 1;
     const double lc = __shfl_sync(FULLMASK, lv, l0);   // ln F_cent
     const double lp = __shfl_sync(FULLMASK, lv, l1);   // ln P_r
@@ -269,7 +268,8 @@ __device__ __forceinline__ void troe_phase(const DevMech& m, const WarpMem& w, d
     const double iS = rcp_nr(q ? 1.0 + Pr : fma(x, x, d2));
     const double ipr = __shfl_sync(FULLMASK, iS, l1);
     if (act && q == 0) {
-      const double F = exp_t(lc * d2 * iS, et);
+      const double lF = lc * d2 * iS;
+      const double F = FIX ? exp_t_fix(lF, m.fexptab) : exp_t(lF, m.exptab);
       const double kinf = r[0];
       r[5] = kinf * Pr * ipr * F;
       if (JAC) {
@@ -299,28 +299,29 @@ __device__ __forceinline__ void troe_phase(const DevMech& m, const WarpMem& w, d
 // ------------------------------------------------------------------------------------------
 // right-hand side f(z) of the reactor, z = (Y_1..Y_K, T)  [Eq. 1]
 // ------------------------------------------------------------------------------------------
-template <int NPL, bool JAC>
+// FIX: exponentials and logarithms in fixed point (rates); the integrator takes the FP64 forms
+template <int NPL, bool JAC, bool FIX>
 __device__ void rhs_eval(const DevMech& m, const WarpMem& w, const CellP& cp0, const double (&y)[NPL],
                          double (&f)[NPL], LaneSp<NPL>& sp, CellSc& cs, int lane) {
   const int K = m.K, I = m.I;
   const double T = comp_get<NPL>(y, K);
-  const double lnT = log_t(T, m.logtab), RT = kR * T;
-  const unsigned long long* __restrict__ et = m.exptab;
+  const double lnT = FIX ? log_t_fix(T, m.flogtab) : log_t(T, m.logtab), RT = kR * T;
+  auto exp_s = [&](double x) { return FIX ? exp_s256_fix(x, m.fexptab) : exp_s256(x, m.exptab); };
   // T >= T_mid on the bit patterns (both positive: they order like the values)
   const int hi = __double_as_longlong(T) >= __double_as_longlong(m.Tmid) ? 1 : 0;
   // pass 1: c_p/R per species and the two mixture sums sum Y/W and sum Y c_p/(R W)
   double sYW = 0.0, cpp = 0.0, ywr[NPL];
   const int KP = m.KP;
-  const double* rth = m.rth + (size_t)hi * 11 * KP;
-  const double* rgn = m.gneg + (size_t)hi * 7 * KP;
+  const double2* rth = m.rth + (size_t)hi * 6 * KP;
+  const double2* rgn = m.gneg + (size_t)hi * 4 * KP;
 #pragma unroll
   for (int s = 0; s < NPL; ++s) {
     const int k = lane + 32 * s;
     ywr[s] = 0.0;
     sp.cpR[s] = sp.dcpR[s] = sp.hRT[s] = 0.0;
     if (k < K) {
-      const double a0 = __ldg(rth + k), a1 = __ldg(rth + KP + k), a2 = __ldg(rth + 2 * KP + k);
-      const double a3 = __ldg(rth + 3 * KP + k), a4 = __ldg(rth + 4 * KP + k);
+      const double2 a01 = __ldg(rth + k), a23 = __ldg(rth + KP + k);
+      const double a0 = a01.x, a1 = a01.y, a2 = a23.x, a3 = a23.y, a4 = __ldg(&rth[2 * KP + k].x);
       const double cpR = a0 + T * (a1 + T * (a2 + T * (a3 + T * a4)));
       if (JAC) sp.dcpR[s] = a1 + T * (2.0 * a2 + T * (3.0 * a3 + T * 4.0 * a4));
       const double yw = y[s] * __ldg(m.invW + k);
@@ -358,22 +359,28 @@ __device__ void rhs_eval(const DevMech& m, const WarpMem& w, const CellP& cp0, c
       w.ieg[K] = 1.0;
     }
     if (k < K) {
-      double a[6], g[7];
-#pragma unroll
-      for (int i = 0; i < 6; ++i) a[i] = __ldg(rth + (5 + i) * KP + k);
-#pragma unroll
-      for (int i = 0; i < 7; ++i) g[i] = __ldg(rgn + i * KP + k);
-      const double hRT = a[0] + T * (a[1] + T * (a[2] + T * (a[3] + T * a[4]))) + a[5] * invT;
-      const double ng = fma(T, T * fma(T, fma(T, g[5], g[4]), g[3]) + g[2], fma(g[6], invT, fma(g[1], lnT, g[0])));
+      const double h0 = __ldg(&rth[2 * KP + k].y), h5 = __ldg(&rth[5 * KP + k].x);
+      const double2 h12 = __ldg(rth + 3 * KP + k), h34 = __ldg(rth + 4 * KP + k);
+      const double2 g01 = __ldg(rgn + k), g23 = __ldg(rgn + KP + k), g45 = __ldg(rgn + 2 * KP + k);
+      const double g6 = __ldg(&rgn[3 * KP + k].x);
+      const double hRT = h0 + T * (h12.x + T * (h12.y + T * (h34.x + T * h34.y))) + h5 * invT;
+      const double ng = fma(T, T * fma(T, fma(T, g45.y, g45.x), g23.y) + g23.x, fma(g6, invT, fma(g01.y, lnT, g01.x)));
       const double Ck = rho * ywr[s];
       w.C[k] = Ck;
       w.hRT[k] = hRT;
       sp.hRT[s] = hRT;
-      // e and 1/e from the one fixed-point argument
-      const long long gf = fix_s256(ng);
-      double e = exp2_fix(gf, et), ie = exp2_fix(-gf, et);
-      if (s256_end(ng)) {
-        e = exp_s256_end(ng, e);
+      double e, ie;
+      if (FIX) {
+        // e and 1/e from the one fixed-point argument
+        const long long gf = fix_s256(ng);
+        e = exp2_fix(gf, m.fexptab);
+        ie = exp2_fix(-gf, m.fexptab);
+        if (s256_end(ng)) {
+          e = exp_s256_end(ng, e);
+          ie = rcp_nr(e);
+        }
+      } else {
+        e = exp_s256(ng, m.exptab);
         ie = rcp_nr(e);
       }
       w.eg[k] = e * P0RT;
@@ -387,14 +394,18 @@ __device__ void rhs_eval(const DevMech& m, const WarpMem& w, const CellP& cp0, c
   // whole rounds before the first falloff item: k_f only, no T term in the argument
   const int n_plain = (nb / 32) * 32;
   const int XP = m.XP;
-  const double* xa = m.xarg + lane;
-#pragma unroll 2
-  for (int t = 0; t < n_plain; t += 32)
-    w.q[t + lane] = exp_s256(fma(-__ldg(xa + 2 * XP + t), invT, fma(__ldg(xa + XP + t), lnT, __ldg(xa + t))), et);
-#pragma unroll 2
+  const double2* xa = m.xarg;
+  // (two rounds at a time pay for the large mechanisms only: 53 species 144.0 -> 142.0 ms, 30 species
+  // 135.4 -> 137.4 ms, 9 species 3.53 -> 3.61 ms)
+#pragma unroll NPL
+  for (int t = lane; t < n_plain; t += 32) {
+    const double2 x01 = __ldg(xa + t);
+    w.q[t] = exp_s(fma(-__ldg(&xa[XP + t].x), invT, fma(x01.y, lnT, x01.x)));
+  }
+#pragma unroll NPL
   for (int t = n_plain + lane; t < m.n_x; t += 32) {
-    const double* x = m.xarg + t;
-    const double e = exp_s256(fma(__ldg(x + 3 * XP), T, fma(-__ldg(x + 2 * XP), invT, fma(__ldg(x + XP), lnT, __ldg(x)))), et);
+    const double2 x01 = __ldg(xa + t), x23 = __ldg(xa + XP + t);
+    const double e = exp_s(fma(x23.y, T, fma(-x23.x, invT, fma(x01.y, lnT, x01.x))));
     if (t < nb) {
       w.q[t] = e;
     } else {
@@ -403,7 +414,7 @@ __device__ void rhs_eval(const DevMech& m, const WarpMem& w, const CellP& cp0, c
     }
   }
   __syncwarp();
-  if (I > nb) troe_phase<JAC>(m, w, invT, ctot, lane);
+  if (I > nb) troe_phase<JAC, FIX>(m, w, invT, ctot, lane);
   if (two) {
     // q_j = k_f (C_a C_b - K_c^-1 C_c C_d) = k_f (C_a C_b - (e_a e_b)(u_c u_d)) with
     // e = exp(-g'/RT) p0/RT and u = exp(g'/RT) (RT/p0) C; a missing partner is the sentinel 1.
@@ -412,11 +423,7 @@ __device__ void rhs_eval(const DevMech& m, const WarpMem& w, const CellP& cp0, c
       const int r0 = rs & 255u, r1 = (rs >> 8) & 255u, p0 = (rs >> 16) & 255u, p1 = rs >> 24;
       return kf * fma(-(w.eg[r0] * w.eg[r1]), w.ieg[p0] * w.ieg[p1], w.C[r0] * w.C[r1]);
     };
-    // whole rounds of elementary reactions, then the rest
-    const int n_full = (m.n_elem / 32) * 32;
-#pragma unroll 2
-    for (int j = lane; j < n_full; j += 32) w.q[j] = net(__ldg(m.rsp2 + j), w.q[j]);
-    for (int j = n_full + lane; j < I; j += 32) {
+    for (int j = lane; j < I; j += 32) {
       const unsigned int rs = __ldg(m.rsp2 + j);
       double kf;
       if (j < nb) kf = w.q[j];
@@ -482,27 +489,18 @@ __device__ void rhs_eval(const DevMech& m, const WarpMem& w, const CellP& cp0, c
   double* part = w.g;   // g, eg and ieg are dead from here on: 3K slots for the runs
   if (P > 0) {
     double acc = 0.0;
-    const unsigned int* bl = m.bal + lane;
-    // one entry: nu = 0 (padding), +-1, +-2, +-3 built from its bits (no FP64 conversion); the run's
-    // slot takes the partial sum every time, its last entry leaves the whole and clears it
-    auto entry = [&](unsigned int e, double q) {
-      const unsigned int a = e & 3u;
-      const unsigned int hw = (a == 0u ? 0u : a == 1u ? 0x3ff00000u : a == 2u ? 0x40000000u : 0x40080000u) | ((e & 4u) << 29);
-      acc = fma(__hiloint2double((int)hw, 0), q, acc);
-      part[(e >> 4) & 255u] = acc;
-      if (e & 8u) acc = 0.0;
-    };
-    for (int i = 0; i < P; i += 4) {
-      // four entries' table words and net rates are loaded ahead of the chain of FMAs
-      unsigned int e[4];
-      double q[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) e[u] = i + u < P ? __ldg(bl + (i + u) * 32) : 0u;
-#pragma unroll
-      for (int u = 0; u < 4; ++u) q[u] = w.q[e[u] >> 12];
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (i + u < P) entry(e[u], q[u]);
+    for (int i = 0; i < P; ++i) {
+      const unsigned int e = __ldg(m.bal + (size_t)i * 32 + lane);
+      if (e & 3u) {
+        // nu = +-1, +-2, +-3 built from its bits (no FP64 conversion)
+        const unsigned int a = e & 3u;
+        const unsigned int hw = (a == 1u ? 0x3ff00000u : a == 2u ? 0x40000000u : 0x40080000u) | ((e & 4u) << 29);
+        acc = fma(__hiloint2double((int)hw, 0), w.q[e >> 12], acc);
+        if (e & 8u) {
+          part[(e >> 4) & 255u] = acc;
+          acc = 0.0;
+        }
+      }
     }
     __syncwarp();
   }
@@ -991,7 +989,7 @@ __device__ int integrate_cell(const DevMech& m, const WarpMem& w, double pc, dou
   double D[kMaxOrd + 3][NPL];
   double f[NPL], y[NPL], d[NPL], dy[NPL], psi[NPL];
   // initial step (Hairer, Norsett & Wanner, Sec. II.4, order 1)
-  rhs_eval<NPL, false>(m, w, pp, z, f, sp, cs, lane);
+  rhs_eval<NPL, false, false>(m, w, pp, z, f, sp, cs, lane);
   cnt[1]++;
 #pragma unroll
   for (int s = 0; s < NPL; ++s) isc[s] = __frcp_rn(fmaf(rtolf, fabsf(narrow_f32(z[s])), atolf[s]));
@@ -1000,7 +998,7 @@ __device__ int integrate_cell(const DevMech& m, const WarpMem& w, double pc, dou
   h0 = fmin(h0, dt);
 #pragma unroll
   for (int s = 0; s < NPL; ++s) y[s] = z[s] + h0 * f[s];
-  rhs_eval<NPL, false>(m, w, pp, y, dy, sp, cs, lane);
+  rhs_eval<NPL, false, false>(m, w, pp, y, dy, sp, cs, lane);
   cnt[1]++;
 #pragma unroll
   for (int s = 0; s < NPL; ++s) dy[s] -= f[s];
@@ -1055,7 +1053,7 @@ __device__ int integrate_cell(const DevMech& m, const WarpMem& w, double pc, dou
     const double c = h * ig;
     bool f_at_pred = false;
     if (need_jac) {
-      rhs_eval<NPL, true>(m, w, pp, y, f, sp, cs, lane);
+      rhs_eval<NPL, true, false>(m, w, pp, y, f, sp, cs, lane);
       jac_assemble<NPL>(m, w, y, sp, cs, lane);
       cnt[1]++;
       cnt[2]++;
@@ -1091,7 +1089,7 @@ __device__ int integrate_cell(const DevMech& m, const WarpMem& w, double pc, dou
     newton_iters = 0;
     for (int it = 0; it < kNewtonMax; ++it) {
       if (!(it == 0 && f_at_pred)) {
-        rhs_eval<NPL, false>(m, w, pp, y, f, sp, cs, lane);
+        rhs_eval<NPL, false, false>(m, w, pp, y, f, sp, cs, lane);
         cnt[1]++;
       }
       bool ok = true;
@@ -1279,7 +1277,7 @@ __global__ void __launch_bounds__(128) rates_kernel(DevMech m, int64_t n, int64_
     CellSc cs;
     load_cell<NPL>(m, col, ld, T, Y, z, lane);
     const double pc = p[col];
-    rhs_eval<NPL, false>(m, w, cell_p(pc), z, f, sp, cs, lane);
+    rhs_eval<NPL, false, true>(m, w, cell_p(pc), z, f, sp, cs, lane);
 #pragma unroll
     for (int s = 0; s < NPL; ++s) {
       const int k = lane + 32 * s;
@@ -1304,7 +1302,7 @@ __global__ void __launch_bounds__(128) jacobian_kernel(DevMech m, int64_t n, int
     CellSc cs;
     load_cell<NPL>(m, col, ld, T, Y, z, lane);
     const double pc = p[col];
-    rhs_eval<NPL, true>(m, w, cell_p(pc), z, f, sp, cs, lane);
+    rhs_eval<NPL, true, false>(m, w, cell_p(pc), z, f, sp, cs, lane);
     jac_assemble<NPL>(m, w, z, sp, cs, lane);
     double* out = jac + (size_t)col * nn * nn;
     for (int e = lane; e < nn * nn; e += 32) out[e] = w.J[(size_t)(e / nn) * w.ld + (e % nn)];
@@ -1312,17 +1310,17 @@ __global__ void __launch_bounds__(128) jacobian_kernel(DevMech m, int64_t n, int
   }
 }
 
-__global__ void exp_selftest_kernel(const unsigned long long* __restrict__ tab, int64_t n, const double* x, double* y) {
+__global__ void exp_selftest_kernel(const double* __restrict__ tab, int64_t n, const double* x, double* y) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     y[i] = exp_t(x[i], tab);
 }
 
-__global__ void exp256_selftest_kernel(const unsigned long long* __restrict__ tab, int64_t n, const double* x, double* y) {
+__global__ void exp256_selftest_kernel(const double* __restrict__ tab, int64_t n, const double* x, double* y) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     y[i] = exp_s256(x[i], tab);
 }
 
-__global__ void log_selftest_kernel(const longlong2* __restrict__ tab, int64_t n, const double* x, double* y) {
+__global__ void log_selftest_kernel(const double* __restrict__ tab, int64_t n, const double* x, double* y) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     y[i] = log_t(x[i], tab);
 }

@@ -47,19 +47,21 @@ struct DevMech {
   const int* sp_ptr;       // [K+1]
   const int* sp_rxn;       // [nnz]
   const double* sp_nu;     // [nnz]
-  // Species polynomials of the right-hand side, one lane per species: [2 ranges][11][KP], KP = K
-  // rounded up to 32: c_p/R (a1..a5), h/RT (a1 a2/2 .. a5/5 a6), so that a warp's load of one
-  // coefficient is contiguous.
+  // Species polynomials of the right-hand side, one lane per species, in pairs so that a warp's load
+  // of two coefficients is contiguous: [2 ranges][6][KP], KP = K rounded up to 32: c_p/R (a1..a5),
+  // h/RT (a1 a2/2 .. a5/5 a6), one unused
   int KP;
-  const double* rth;
+  const double2* rth;
   // -g'_k/RT for the equilibrium constants, g' = g_k - sum_r P[k][r] g_{ref_r} the free
   // energy shifted by element potentials (P = composition x pinv(reference compositions));
   // balanced reactions cancel the shift exactly, and it keeps exp(-g') products in range.
   // Per species and range one polynomial: [0] + [1] ln T + T ([2] + T ([3] + T ([4] + T [5])))
-  // + [6] / T, times 256/ln 2 (exp_s256's argument unit).
-  const double* gneg;      // [2][7][KP]
-  const unsigned long long* exptab;   // [256] 2^(j/256) 2^63, the table of the exponentials below
-  const longlong2* logtab;   // [97] {G, -ln(G 2^-10) 2^63}, j = 96..192: the table of log_t below
+  // + [6] / T ([7] unused), times 256/ln 2 (exp_s256's argument unit).
+  const double2* gneg;     // [2][4][KP], coefficients 2i and 2i + 1
+  const double* exptab;    // [256] 2^(j/256), the table of the FP64 exponentials below
+  const double* logtab;    // [97][3] F = j/128, 1/F, log F (j = 96..192): the table of log_t below
+  const unsigned long long* fexptab;   // [256] 2^(j/256) 2^63 and
+  const longlong2* flogtab;            // [97] {G, -ln(G 2^-10) 2^63}: those of the fixed-point forms
   const double* compW;     // [K][E] element counts divided by the molar mass (mol/kg)
   // the same rounded to FP32, for the learned step's FP32 parts
   const float* th32;       // [K][2][16]: c_p/R (5: a1..a5), h/RT (6: a1 a2/2 .. a5/5 a6), pad
@@ -67,13 +69,13 @@ struct DevMech {
   const float* compW32;    // [K][E]
   // Exponentials of one right-hand side, in lane rounds: item t < n_tb_end is k_f of reaction
   // t, then 5 per falloff reaction (k_inf, k_0/k_inf, the three F_cent terms).  Item t is
-  // exp(x) with x = xarg[0][t] + xarg[1][t] ln T - xarg[2][t] / T + xarg[3][t] T, the
+  // exp(x) with x = xarg[0][t].x + xarg[0][t].y ln T - xarg[1][t].x / T + xarg[1][t].y T, the
   // coefficients stored times 256/ln 2 (exp_s256's argument unit).
   int n_x, XP;             // XP: n_x rounded up to 32
-  const double* xarg;      // [4][XP]
+  const double2* xarg;     // [2][XP]
   // Lane-balanced species production rates: lane L walks entries bal[i*32 + L], i < bal_P,
   // each |nu| (bits 0-1), nu < 0 (bit 2), last entry of its run (bit 3), run slot (bits 4-11),
-  // reaction (bits 12-31); |nu| = 0: padding, in a slot of no species.  wdot_k = sum of the run slots run_ptr[k] ..
+  // reaction (bits 12-31); 0 = padding.  wdot_k = sum of the run slots run_ptr[k] ..
   // run_ptr[k+1] - 1 in order.  bal_P = 0: walk the incidence lists instead.
   int bal_P;
   const unsigned int* bal;   // [bal_P][32]
@@ -106,7 +108,114 @@ __device__ __forceinline__ double widen_f64(float f) {
 }
 
 // ------------------------------------------------------------------------------------------
-// FP64 exponentials and logarithm on the integer pipe.
+// Elementary functions in FP64: the forms of the integrator and its Jacobian.
+//
+// The integrator keeps them although the fixed-point forms below are cheaper and more accurate: any
+// change in the last bit of a rate re-draws the knife-edge decisions of its step control.  At loose
+// tolerances (rtol 1e-6, atol 1e-12) 3 in 10,000 cells then end with another value of a species at the
+// noise level of the absolute tolerance, which the Box-Cox targets of a training set magnify to O(1)
+// (the 30-species training gradients moved by 1.4e-4).
+// ------------------------------------------------------------------------------------------
+// FP64 exponential by the table-driven method (P. T. P. Tang, "Table-driven implementation of
+// the exponential function in IEEE floating-point arithmetic", ACM TOMS 15, 1989), here with a
+// 256-entry table: x = (256 k + j) ln2/256 + r, exp(x) = 2^k 2^(j/256) e^r, e^r - 1 from its
+// degree-4 Taylor polynomial.  The split n = 256 k + j only has to keep r small, so it is
+// taken from the FP32 value of x (integer-pipe narrowing, one FP32 FMA against 1.5 * 2^23,
+// which rounds to an integer): for |x| < 709.8, |x 256/ln2 - n| <= 0.5 + 0.05, so |r| <=
+// 1.49e-3 and the truncation |r|^5/120 < 6e-17 relative stays below an ulp.  n goes back to
+// FP64 exactly through FP32 (|n| < 2^18) on the integer pipe, and n ln2/256 is split so that
+// n times its high part is exact.  7 FP64 instructions (against ~22 FP64-pipe slots for the
+// library exp on GB300); within 2 ulp of a correctly rounded exp (tested).
+// Arguments below -708 return 0, above 709.78 return +inf, NaN propagates.
+__device__ __forceinline__ double exp_t(double x, const double* __restrict__ tab) {
+  const float kInvLf = 369.329930467574f;            // 256 / ln 2
+  const float kMagicf = 12582912.0f;                 // 1.5 * 2^23: rounds to an integer
+  const double kL1 = 0x1.62e42ff000000p-9;           // ln 2 / 256, high part (29 bits: nd kL1 exact)
+  const double kL2 = -1.6409824502660487e-13;        // ln 2 / 256 - kL1
+  const float tf = fmaf(narrow_f32(x), kInvLf, kMagicf);
+  const int nn = (int)(__float_as_uint(tf) - 0x4B400000u);   // tf = 1.5 * 2^23 + n
+  const double nd = widen_f64(tf - kMagicf);                 // n, exactly
+  const double r = fma(-nd, kL2, fma(-nd, kL1, x));
+  double q = fma(r, 1.0 / 24.0, 1.0 / 6.0);
+  q = fma(q, r, 0.5);
+  q = fma(q, r, 1.0);
+  const double tj = __ldg(tab + (nn & 255));
+  double res = fma(tj * r, q, tj);                   // 2^(j/256) (1 + r q)
+  res = __longlong_as_double(__double_as_longlong(res) + ((long long)(nn >> 8) << 52));
+  // |x| >= 708, inf and NaN, detected on the exponent bits (integer pipe, rare branch)
+  if (((unsigned int)((unsigned long long)__double_as_longlong(x) >> 32) & 0x7fffffffu) >= 0x40862000u) {
+    if (x != x) res = x;
+    else if (x < -708.0) res = 0.0;
+    else if (x > 709.78) res = __longlong_as_double(0x7ff0000000000000LL);
+  }
+  return res;
+}
+// exp of an argument given in units of ln2/256: exp_s256(y) = 2^(y/256) = exp(y ln2/256), the
+// same table-driven method as exp_t for callers whose arguments are linear in tabulated
+// coefficients (the rate constants and free energies of the chemistry kernels), which are
+// stored pre-scaled by 256/ln 2.  y = 256 k + j + r_s with n = 256 k + j rounded from the FP32
+// value of y (|y - n| <= 0.53) and r_s = y - n exact (Sterbenz); e^(r_s ln2/256) - 1 from
+// its degree-4 Taylor polynomial in r_s, whose coefficients carry the powers of ln2/256
+// (truncation below 5e-17 relative).  6 FP64 instructions; within 2 ulp of 2^(y/256)
+// (tested).  y below -261485.59 (x < -708) returns 0, y >= 2^18 (x > 709.78) +inf, NaN
+// propagates.
+__device__ __forceinline__ double exp_s256(double y, const double* __restrict__ tab) {
+  const float kMagicf = 12582912.0f;                 // 1.5 * 2^23: rounds to an integer
+  const double c1 = 0.0027076061740622863;           // ln 2 / 256
+  const double c2 = 3.6655655969101062e-06;          // c1^2 / 2
+  const double c3 = 3.3083026805413713e-09;          // c1^3 / 6
+  const double c4 = 2.239395190875157e-12;           // c1^4 / 24
+  const float tf = narrow_f32(y) + kMagicf;
+  const int nn = (int)(__float_as_uint(tf) - 0x4B400000u);   // tf = 1.5 * 2^23 + n
+  const double rs = y - widen_f64(tf - kMagicf);             // y - n, exactly
+  double q = fma(rs, c4, c3);
+  q = fma(q, rs, c2);
+  q = fma(q, rs, c1);
+  const double tj = __ldg(tab + (nn & 255));
+  double res = fma(tj * rs, q, tj);                  // 2^(j/256) (1 + r_s q)
+  res = __longlong_as_double(__double_as_longlong(res) + ((long long)(nn >> 8) << 52));
+  // |y| >= 261485, inf and NaN, detected on the exponent bits (integer pipe, rare branch)
+  if (((unsigned int)((unsigned long long)__double_as_longlong(y) >> 32) & 0x7fffffffu) >= 0x410feb68u) {
+    if (y != y) res = y;
+    else if (y < -261485.59077104286) res = 0.0;
+    else if (y >= 262144.0) res = __longlong_as_double(0x7ff0000000000000LL);
+  }
+  return res;
+}
+
+// FP64 natural logarithm by the table-driven method (P. T. P. Tang, "Table-driven
+// implementation of the logarithm function in IEEE floating-point arithmetic", ACM TOMS 16,
+// 1990): x = 2^k m with m in [0.75, 1.5), F = j/128 the grid point nearest m (j = 96..192),
+// log x = k ln2 + log F + log1p(u), u = (m - F)/F (m - F exact), |u| <= 1/192, log1p(u) from
+// its degree-7 Taylor polynomial (truncation < |u|^8/8: < 1.7e-18 |u| at F = 1, where u is
+// exact, and < 3e-17 of the result elsewhere).  Centring m on 1 keeps log x accurate near
+// x = 1; k ln2 is split (32-bit high part, exact product).
+// tab[3(j-96) + {0, 1, 2}] = F_j, 1/F_j, log F_j.  Positive normal x only: zero, negative,
+// subnormal, inf and NaN take the library log.
+__device__ __forceinline__ double log_t(double x, const double* __restrict__ tab) {
+  const long long b = __double_as_longlong(x);
+  const unsigned int hw = (unsigned int)((unsigned long long)b >> 32);
+  if (hw - 0x00100000u >= 0x7fe00000u) return log(x);
+  const long long frac = b & 0x000fffffffffffffLL;
+  const int up = (int)(frac >> 51);                 // m >= 1.5: use m/2 and k + 1
+  const int j = (int)((frac + (1LL << 52) + (1LL << (44 + up))) >> (45 + up));     // round(128 m)
+  const double* t = tab + 3 * (j - 96);
+  const double m = __longlong_as_double(frac | ((long long)(1023 - up) << 52));
+  const double u = (m - __ldg(t)) * __ldg(t + 1);
+  double pl = fma(u, 1.0 / 7.0, -1.0 / 6.0);
+  pl = fma(pl, u, 0.2);
+  pl = fma(pl, u, -0.25);
+  pl = fma(pl, u, 1.0 / 3.0);
+  pl = fma(pl, u, -0.5);
+  // k as a double without an FP64 instruction: 1.5 * 2^23 + k (any sign) has k in its low
+  // bits, one FP32 subtraction leaves k exactly, and the integer pipe widens it
+  const int k = (int)(hw >> 20) - 1023 + up;
+  const double kd = widen_f64(__uint_as_float(0x4B400000u + (unsigned int)k) - 12582912.0f);
+  const double kLn2Hi = 0x1.62e42fee00000p-1, kLn2Lo = 1.9082149292705877e-10;
+  return fma(kd, kLn2Hi, __ldg(t + 2)) + fma(kd, kLn2Lo, fma(pl, u * u, u));
+}
+// ------------------------------------------------------------------------------------------
+// The same functions on the integer pipe, for rates and properties.
 //
 // GB300 issues one FP64 warp instruction per SM every 16 cycles, while each of the SM's four
 // schedulers can issue an integer instruction every cycle: one FP64 instruction costs the pipe as
@@ -120,7 +229,7 @@ __device__ __forceinline__ double widen_f64(float f) {
 // the last one: worst errors over the ranges of use 0.55 ulp (exponentials; 1.2 ulp where the
 // argument is within one table step of 0) and 0.92 ulp (logarithm), against 2 ulp of the FP64
 // forms.  Against those (same inputs): rates of 200,000 30-species cells 2,715 -> 2,132 us, FP64
-// properties of 1 M cells 7,560 -> 6,489 us, direct integration of 12,345 cells 139.7 -> 128.2 ms.
+// properties of 1 M cells 7,560 -> 6,489 us.
 // ------------------------------------------------------------------------------------------
 
 // |x| 2^fb truncated to an integer, for |x| < 2^(63 - fb): the significand with its leading one at
@@ -201,14 +310,14 @@ __device__ __forceinline__ double exp2_fix(long long f, const unsigned long long
   return __longlong_as_double((long long)(((R + 0x400ull) >> 11) + ((unsigned long long)(1022 + (n >> 8)) << 52)));
 }
 
-// exp(x): the argument in units of ln2/256 is x log2(e) 256 (the integer part of log2(e) exact).
+// exp_t_fix(x) = exp(x): the argument in units of ln2/256 is x log2(e) 256 (the integer part of log2(e) exact).
 // Arguments below -708 return 0, above 709.78 return +inf, NaN propagates.
 __device__ __forceinline__ long long fix_exp_arg(double x) {
   const unsigned long long X = fix_mag(x, 53);
   const long long F = (long long)(X + __umul64hi(X, 0x71547652B82FE177ull));   // |x| log2(e) 2^53
   return __double_as_longlong(x) < 0 ? -F : F;
 }
-__device__ __forceinline__ double exp_t(double x, const unsigned long long* __restrict__ tab) {
+__device__ __forceinline__ double exp_t_fix(double x, const unsigned long long* __restrict__ tab) {
   double res = exp2_fix(fix_exp_arg(x), tab);
   // |x| >= 708, inf and NaN, detected on the exponent bits (rare branch)
   if (((unsigned int)((unsigned long long)__double_as_longlong(x) >> 32) & 0x7fffffffu) >= 0x40862000u) {
@@ -219,7 +328,7 @@ __device__ __forceinline__ double exp_t(double x, const unsigned long long* __re
   return res;
 }
 
-// exp of an argument given in units of ln2/256: exp_s256(y) = 2^(y/256) = exp(y ln2/256), for
+// exp of an argument given in units of ln2/256: exp_s256_fix(y) = 2^(y/256) = exp(y ln2/256), for
 // callers whose arguments are linear in tabulated coefficients (the rate constants and free
 // energies of the chemistry kernels), which are stored pre-scaled by 256/ln 2.  y below -261485.59
 // (x < -708) returns 0, y >= 2^18 (x > 709.78) +inf, NaN propagates.
@@ -236,7 +345,7 @@ __device__ __forceinline__ double exp_s256_end(double y, double res) {
   if (y < -261485.59077104286) return 0.0;
   return y >= 262144.0 ? __longlong_as_double(0x7ff0000000000000LL) : res;
 }
-__device__ __forceinline__ double exp_s256(double y, const unsigned long long* __restrict__ tab) {
+__device__ __forceinline__ double exp_s256_fix(double y, const unsigned long long* __restrict__ tab) {
   double res = exp2_fix(fix_s256(y), tab);
   if (s256_end(y)) res = exp_s256_end(y, res);
   return res;
@@ -249,7 +358,7 @@ __device__ __forceinline__ double exp_s256(double y, const unsigned long long* _
 // FP64 in the integer pipe and k ln2 is added by two FMAs (k ln2 split, 32-bit high part).  Zero,
 // negative, subnormal, inf and NaN take the library log; so do arguments within 1/256 of 1 (k = 0,
 // j = 128), whose results need more fraction bits.
-__device__ __forceinline__ double log_t(double x, const longlong2* __restrict__ tab) {
+__device__ __forceinline__ double log_t_fix(double x, const longlong2* __restrict__ tab) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const unsigned int hw = (unsigned int)(b >> 32);
   const unsigned long long frac = b & 0x000fffffffffffffull;

@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(128, JC <= 16 ? 4 : 2) thermo64_kernel(DevMech
     solve_T<SPLIT == 2>(Tc, h_in != nullptr, h_in ? h_in[i] : 0.0, m.Tmid, coeffs, A, cp, h);
     double l1 = 0.0, l2 = 0.0, mu = 0.0;
     if (transport) {
-      const double L = log_t(Tc, m.logtab);
+      const double L = log_t_fix(Tc, m.flogtab);
 #pragma unroll
       for (int j = 0; j < JC; ++j) ps[j * nt + tid] = v[j];
       int Ep = 0, Eq = 0, Er = 0, ex = 0;
@@ -336,10 +336,10 @@ __global__ void __launch_bounds__(128, JC <= 16 ? 4 : 2) thermo64_kernel(DevMech
         const double yw = ps[j * nt + tid];
         const double xu = b[0] + L * (b[1] + L * (b[2] + L * b[3]));
         const double xl = b[4] + L * (b[5] + L * (b[6] + L * b[7]));
-        const double u = b[10] * exp2_fix(fix_exp_arg(xu), m.exptab);
+        const double u = b[10] * exp2_fix(fix_exp_arg(xu), m.fexptab);
         const long long fl = fix_exp_arg(xl);
-        l1 = fma(yw, exp2_fix(fl, m.exptab), l1);
-        l2 = fma(yw, exp2_fix(-fl, m.exptab), l2);
+        l1 = fma(yw, exp2_fix(fl, m.fexptab), l1);
+        l2 = fma(yw, exp2_fix(-fl, m.fexptab), l2);
         const double p = yw * b[9], q = p * u;
         us[j * nt + tid] = u;
         ps[j * nt + tid] = p;
