@@ -469,7 +469,7 @@ __global__ void scatter_status_kernel(int64_t nmax, const int32_t* n_dev, const 
 //   L = w_data * mean_{b,k}(u - u_t)^2 + w_mass * mean_b |sum_k Y*_k - 1| + w_hrr * mean_b e_b^2,
 //   Y*_k = F^-1(F(Y_k) + u_k sigma_k + mu_k),
 //   e_b = sum_k c_bk (Y*_k - Y_k) - r_b   (the step-mean heat-release error, scaled)
-// dU (BF16 [B, n_out_pad]) and its transpose dUT ([n_out_pad, B]); per-block loss partials.
+// dU (BF16 [B, n_out_pad]) and, if not null, its transpose dUT ([n_out_pad, B]); per-block loss partials.
 __global__ void loss_grad_kernel(int64_t B, int K, int n_out_pad, const float* Up, const float* Ut, const float* bcty,
                                  const float* out_mean, const float* out_sd, float w_data, float w_mass,
                                  const float* hrr_c, const float* hrr_r, float w_hrr, bf16* dU, bf16* dUT,
@@ -512,7 +512,7 @@ __global__ void loss_grad_kernel(int64_t B, int K, int n_out_pad, const float* U
       }
       const bf16 gb = __float2bfloat16_rn(g);
       dU[b * n_out_pad + k] = gb;
-      dUT[(int64_t)k * B + b] = gb;
+      if (dUT) dUT[(int64_t)k * B + b] = gb;
     }
   }
   sh[0][threadIdx.x] = ld;
@@ -620,22 +620,62 @@ __device__ __forceinline__ int64_t wt_index(int64_t i, int gh, int ldt, int cols
   return (g * cols + c) * ldt + (r - g * gh);
 }
 
-// Adam (Kingma & Ba 2015) on FP32 masters; refreshes the BF16 copy and its transpose
-__global__ void adam_kernel(int64_t n, int gh, int ldt, int cols, float* w, const float* g, float* mom, float* vel,
-                            float lr, float b1, float b2, float eps, float bc1, float bc2, bf16* wb, bf16* wt) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const float gi = g[i];
-    const float mi = b1 * mom[i] + (1.0f - b1) * gi;
-    const float vi = b2 * vel[i] + (1.0f - b2) * gi * gi;
-    mom[i] = mi;
-    vel[i] = vi;
-    const float wi = w[i] - lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
-    w[i] = wi;
-    if (wb) {
-      const bf16 q = __float2bfloat16_rn(wi);
-      wb[i] = q;
-      wt[wt_index(i, gh, ldt, cols)] = q;
+// Adam (Kingma & Ba 2015) on the FP32 masters, refreshing the BF16 copy and its transpose, for every
+// weight and bias of the network in one launch (8 launches of 3 to 19 us before, the scattered 2-byte
+// writes of the transpose among them).  Bound by memory: 7 FP32 and 2 BF16 accesses per parameter.  A
+// block takes a 32 x 32 tile of a layer's weights (of one group), transposed through shared memory so
+// that both BF16 copies are written in 64-byte rows, or 1024 biases.
+struct AdamSeg {
+  float* w;
+  const float* g;
+  float *mom, *vel;
+  bf16 *wb, *wt;                        // null for biases
+  int n, gh, cols, ldt, tr, tc, block0;   // n: biases; gh x cols weights per group in tr x tc tiles
+};
+struct AdamArgs {
+  AdamSeg seg[2 * kMaxLayers];
+  int nseg;
+  float lr, b1, b2, eps, bc1, bc2;
+};
+
+__device__ __forceinline__ float adam_step(const AdamArgs& a, const AdamSeg& s, int64_t i) {
+  const float gi = s.g[i];
+  const float mi = a.b1 * s.mom[i] + (1.0f - a.b1) * gi;
+  const float vi = a.b2 * s.vel[i] + (1.0f - a.b2) * gi * gi;
+  s.mom[i] = mi;
+  s.vel[i] = vi;
+  const float wi = s.w[i] - a.lr * (mi / a.bc1) / (sqrtf(vi / a.bc2) + a.eps);
+  s.w[i] = wi;
+  return wi;
+}
+
+__global__ void __launch_bounds__(256) adam_kernel(const __grid_constant__ AdamArgs a) {
+  __shared__ bf16 t[32][34];
+  int q = 0;
+  while (q + 1 < a.nseg && (int)blockIdx.x >= a.seg[q + 1].block0) ++q;
+  const AdamSeg& s = a.seg[q];
+  const int b = blockIdx.x - s.block0;
+  if (!s.wb) {
+    for (int i = b * 1024 + threadIdx.x; i < min(s.n, (b + 1) * 1024); i += 256) adam_step(a, s, i);
+    return;
+  }
+  const int per = s.tr * s.tc, gr = b / per, r0 = (b - gr * per) / s.tc * 32, c0 = (b - gr * per) % s.tc * 32;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+#pragma unroll
+  for (int y = ty; y < 32; y += 8) {
+    const int r = r0 + y, c = c0 + tx;
+    if (r < s.gh && c < s.cols) {
+      const int64_t i = ((int64_t)gr * s.gh + r) * s.cols + c;
+      const bf16 w = __float2bfloat16_rn(adam_step(a, s, i));
+      s.wb[i] = w;
+      t[y][tx] = w;
     }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int y = ty; y < 32; y += 8) {
+    const int c = c0 + y, r = r0 + tx;
+    if (r < s.gh && c < s.cols) s.wt[((int64_t)gr * s.cols + c) * s.ldt + r] = t[tx][y];
   }
 }
 
@@ -758,17 +798,24 @@ int ldt_of(const chem_ann_s* a, int l) { return (a->dims[l + 1] + 7) & ~7; }
 
 // training scratch for a batch of B rows
 struct TrainBufs {
-  bf16 *Z[kMaxLayers], *A[kMaxLayers], *AT[kMaxLayers], *dZ[kMaxLayers], *dZT[kMaxLayers];
+  bf16 *Z[kMaxLayers], *A[kMaxLayers], *dZ[kMaxLayers];
   float* Up;
 };
+
+// the output layer of per-species networks (one unit per group, whose columns no TMA coordinate can
+// address) forms its weight gradient from transposed operands
+bool wgrad_direct(const chem_ann_s* a, int l) { return !(a->groups > 1 && l == a->L - 1); }
 
 size_t train_bytes(const chem_ann_s* a, int64_t B) {
   size_t s = 0;
   for (int l = 0; l < a->L; ++l) {
     const size_t w = (size_t)width_of(a, l);
-    s += 5 * B * w * 2 + 5 * 256;       // Z, A, AT, dZ, dZT
+    s += 3 * B * w * 2 + 3 * 256;       // Z, A, dZ
   }
-  s += (size_t)B * kInPad * 2 + 256;   // XT
+  if (a->groups > 1) {                 // transposes of the per-species output layer's operands
+    s += (size_t)B * a->n_out_pad * 2 + 256;
+    s += (size_t)B * width_of(a, a->L - 2) * 2 + 256;
+  }
   s += (size_t)B * a->n_out_pad * 4 + 256;
   // minibatch staging of chem_ann_train_epoch: X, Ut, bcty, hrr_c, hrr_r, loss sums
   s += (size_t)B * kInPad * 2 + (size_t)B * a->n_out_pad * 4 + 2 * (size_t)B * a->K * 4 + (size_t)B * 4 + 6 * 256;
@@ -1244,11 +1291,14 @@ static int train_step_impl(chem_ann a, const bf16* X, const float* Ut, const flo
     const size_t n = (size_t)B * width_of(a, l);
     t.Z[l] = (bf16*)take(n * 2);
     t.A[l] = (bf16*)take(n * 2);
-    t.AT[l] = (bf16*)take(n * 2);
     t.dZ[l] = (bf16*)take(n * 2);
-    t.dZT[l] = (bf16*)take(n * 2);
   }
-  bf16* XT = (bf16*)take((size_t)B * kInPad * 2);
+  const int Lo = a->L - 1, G = a->groups;
+  bf16 *dUT = nullptr, *hidT = nullptr;   // per-species output layer: dU^T [n_out_pad, B], A^T [width, B]
+  if (G > 1) {
+    dUT = (bf16*)take((size_t)B * a->n_out_pad * 2);
+    hidT = (bf16*)take((size_t)B * width_of(a, Lo - 1) * 2);
+  }
   t.Up = (float*)take((size_t)B * a->n_out_pad * 4);
   // forward (pre-activations kept for GELU')
   bf16* act[kMaxLayers];
@@ -1258,47 +1308,37 @@ static int train_step_impl(chem_ann a, const bf16* X, const float* Ut, const flo
   // loss and dU
   const float* om = a->norm + 4 * a->n_in;
   const int nbl = (int)std::min<int64_t>((B + 255) / 256, 2048);
-  const int Lo = a->L - 1;
   loss_grad_kernel<<<nbl, 256, 0, s>>>(B, a->K, a->n_out_pad, t.Up, Ut, bcty, om, om + a->n_out, opts->w_data,
-                                      opts->w_mass, hrr_c, hrr_r, opts->w_hrr, t.dZ[Lo], t.dZT[Lo], a->loss_part);
+                                      opts->w_mass, hrr_c, hrr_r, opts->w_hrr, t.dZ[Lo], dUT, a->loss_part);
   if (loss_out)
     loss_final_kernel<<<1, 32, 0, s>>>(nbl, a->loss_part, opts->w_data, opts->w_mass, opts->w_hrr, loss_out);
   // backward
-  dim3 tb(32, 8);
-  const int G = a->groups;
+  WgradLayer wg[kMaxLayers];
+  int nwg = 0;
   for (int l = Lo; l >= 0; --l) {
     const int Kd = a->dims[l], wl = width_of(a, l);
     const bool grouped = G > 1 && l > 0;
     const int Ng = a->dims[l + 1];
-    // input activations of layer l, transposed: [width, B]
-    const bf16* inT;
-    if (l == 0) {
-      transpose_kernel<<<dim3((kInPad + 31) / 32, (unsigned)((B + 31) / 32)), tb, 0, s>>>(X, B, kInPad, XT);
-      inT = XT;
+    // dW_l [rows, Kd] = dZ_l^T A_{l-1}, per species for grouped layers; formed after the loop where the
+    // operands can be read in place
+    const bf16* in = l == 0 ? X : t.A[l - 1];
+    const int win = l == 0 ? kInPad : width_of(a, l - 1);
+    if (wgrad_direct(a, l)) {
+      wg[nwg++] = WgradLayer{t.dZ[l], in, wl, win, grouped ? Ng : 0, grouped ? Kd : 0, grouped ? G : 1,
+                             grouped ? Ng : rows_of(a, l), Kd, a->gW[l]};
     } else {
-      const int win = width_of(a, l - 1);
-      transpose_kernel<<<dim3((unsigned)((win + 31) / 32), (unsigned)((B + 31) / 32)), tb, 0, s>>>(t.A[l - 1], B, win,
-                                                                                                   t.AT[l - 1]);
-      inT = t.AT[l - 1];
-    }
-    if (l != Lo)
-      transpose_kernel<<<dim3((unsigned)((wl + 31) / 32), (unsigned)((B + 31) / 32)), tb, 0, s>>>(t.dZ[l], B, wl, t.dZT[l]);
-    // dW_l [rows, Kd] = dZ_l^T [rows, B] (A_{l-1}^T [Kd, B])^T, per species for grouped layers
-    GemmEpi e{};
-    e.out = a->gW[l];
-    e.ldo = Kd;
-    if (grouped) {
+      transpose_kernel<<<dim3((unsigned)((win + 31) / 32), (unsigned)((B + 31) / 32)), dim3(32, 8), 0, s>>>(in, B, win, hidT);
+      GemmEpi e{};
+      e.out = a->gW[l];
+      e.ldo = Kd;
       e.groups = G;
       e.a_row = Ng;
       e.b_row = Kd;
       e.out_goff = (int64_t)Ng * Kd;
-      if ((rc = gemm_bf16(3, t.dZT[l], B, inT, B, Ng, Kd, (int)B, e, a->err, s))) return rc;
-    } else if ((rc = gemm_bf16(3, t.dZT[l], B, inT, B, rows_of(a, l), Kd, (int)B, e, a->err, s))) {
-      return rc;
+      if ((rc = gemm_bf16(3, dUT, B, hidT, B, Ng, Kd, (int)B, e, a->err, s))) return rc;
     }
     if (l == 0) continue;
     // dZ_{l-1} = (dZ_l W_l) * GELU'(Z_{l-1}); B operand = W_l^T
-    const int win = width_of(a, l - 1);
     if (!grouped) {
       GemmEpi e2{};
       e2.out = t.dZ[l - 1];
@@ -1323,6 +1363,7 @@ static int train_step_impl(chem_ann a, const bf16* X, const float* Ut, const flo
       if ((rc = gemm_bf16(2, t.dZ[l], wl, a->WT[l], ldt_of(a, l), (int)B, Kd, Ng, e2, a->err, s))) return rc;
     }
   }
+  if ((rc = wgrad_bf16(wg, nwg, (int)B, a->err, s))) return rc;
   ColsumArgs cs{};
   int cols_max = 0;
   for (int l = 0; l < a->L; ++l) {
@@ -1335,22 +1376,27 @@ static int train_step_impl(chem_ann a, const bf16* X, const float* Ut, const flo
   colsum_kernel<<<dim3((unsigned)((cols_max + kColsumCols - 1) / kColsumCols), (unsigned)a->L), 2 * kColsumRows, 0, s>>>(cs, B);
   if ((rc = cuda_check(cudaGetLastError(), "training launches"))) return rc;
   if (!opts->apply) return CHEM_OK;
-  // Adam
+  AdamArgs aa{};
   a->step++;
+  aa.lr = opts->lr;
+  aa.b1 = opts->beta1;
+  aa.b2 = opts->beta2;
+  aa.eps = opts->eps;
   // bias corrections 1 - beta^t in FP64: in FP32, 1 - 0.999^t loses most of its digits to
   // cancellation for small t
-  const float bc1 = (float)(1.0 - std::pow((double)opts->beta1, (double)a->step));
-  const float bc2 = (float)(1.0 - std::pow((double)opts->beta2, (double)a->step));
+  aa.bc1 = (float)(1.0 - std::pow((double)opts->beta1, (double)a->step));
+  aa.bc2 = (float)(1.0 - std::pow((double)opts->beta2, (double)a->step));
+  int blocks = 0;
   for (int l = 0; l < a->L; ++l) {
-    const int rows = rows_of(a, l), cols = a->dims[l];
-    const int64_t nw = (int64_t)rows * cols;
-    adam_kernel<<<grid_for(nw, 256), 256, 0, s>>>(nw, a->dims[l + 1], ldt_of(a, l), cols, a->Wm[l], a->gW[l], a->mW[l],
-                                                   a->vW[l], opts->lr, opts->beta1, opts->beta2, opts->eps, bc1, bc2,
-                                                   a->W[l], a->WT[l]);
-    adam_kernel<<<grid_for(rows, 256), 256, 0, s>>>(rows, 1, 1, 1, a->bm[l], a->gb[l], a->mb[l], a->vb[l], opts->lr,
-                                                    opts->beta1, opts->beta2, opts->eps, bc1, bc2, nullptr, nullptr);
+    const int rows = rows_of(a, l), gh = a->dims[l + 1], cols = a->dims[l];
+    const int tr = (gh + 31) / 32, tc = (cols + 31) / 32;
+    aa.seg[aa.nseg++] = AdamSeg{a->Wm[l], a->gW[l], a->mW[l], a->vW[l], a->W[l], a->WT[l], 0, gh, cols, ldt_of(a, l), tr, tc, blocks};
+    blocks += rows / gh * tr * tc;
+    aa.seg[aa.nseg++] = AdamSeg{a->bm[l], a->gb[l], a->mb[l], a->vb[l], nullptr, nullptr, rows, 0, 0, 0, 0, 0, blocks};
+    blocks += (rows + 1023) / 1024;
   }
-  return cuda_check(cudaGetLastError(), "adam launch");
+  adam_kernel<<<blocks, 256, 0, s>>>(aa);
+  return cuda_check(cudaGetLastError(), "adam_kernel launch");
 }
 
 int chem_ann_train_step(chem_ann a, const void* Xv, const float* Ut, const float* bcty, const float* hrr_c,

@@ -110,11 +110,20 @@ __device__ __forceinline__ uint64_t sw128_desc(const void* smem_tile) {
   return addr | (sbo << 32) | (1ull << 46) | (2ull << 61);
 }
 
+// The same for MN-major 128B-swizzled tiles (the operand's M or N index contiguous, as in a transposed
+// operand read in place): rows of 128 bytes hold 64 M (or N) elements of one k, 8-row atoms of 1024
+// bytes (8 k; the stride byte offset), the next 64 M elements at the leading byte offset `lbo`.
+__device__ __forceinline__ uint64_t sw128_desc_mn(const void* smem_tile, uint32_t lbo) {
+  return sw128_desc(smem_tile) | ((uint64_t)(lbo >> 4) << 16);
+}
+
 // Instruction descriptor, kind::f16: D = F32 (bits [4,6) = 1), A = B = BF16 (bits [7,10) and
 // [10,13) = 1), both K-major (bits 15, 16 = 0), N >> 3 in [17,23), M >> 4 in [24,29).
-template <int M, int N>
+// MN: both operands MN-major (bits 15, 16 = 1).
+template <int M, int N, bool MN = false>
 __host__ __device__ constexpr uint32_t idesc_bf16_f32() {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+  return (1u << 4) | (1u << 7) | (1u << 10) | (MN ? (3u << 15) : 0u) | ((uint32_t)(N >> 3) << 17) |
+         ((uint32_t)(M >> 4) << 24);
 }
 
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,

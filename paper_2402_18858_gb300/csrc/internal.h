@@ -434,6 +434,17 @@ struct GemmEpi {
   int64_t out_goff, z_goff;
   int bias_goff;
 };
+// Weight gradients of up to kWgradMax layers over the same R rows: out_g [M, N] = A_g^T B_g, FP32, with
+// A [R, *] and B [R, *] BF16 row-major (row strides lda and ldb), group g's columns from g a_col and
+// g b_col (multiples of 8) and its result at out + g M N; M and N multiples of 4 (16-byte stores).
+constexpr int kWgradMax = 8;
+struct WgradLayer {
+  const __nv_bfloat16 *A, *B;
+  int64_t lda, ldb;
+  int a_col, b_col, groups, M, N;
+  float* out;
+};
+int wgrad_bf16(const WgradLayer* layers, int n, int R, int* err, cudaStream_t s);
 int gemm_bf16(int epi, const __nv_bfloat16* A, int64_t lda, const __nv_bfloat16* B, int64_t ldb, int M, int N,
               int K, const GemmEpi& e, int* err, cudaStream_t s);
 // output layer of per-species networks, backward to the last hidden layer: dZ[b, g h + j] =
