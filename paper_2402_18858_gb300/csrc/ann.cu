@@ -36,7 +36,7 @@ constexpr int kStatBlock = 256;
 __device__ __forceinline__ float bct_x(float x) {
   return x > 0.0f ? (exp2f(kLambda * log2f(x)) - 1.0f) * (1.0f / kLambda) : -1.0f / kLambda;
 }
-__device__ __forceinline__ float bct_f(double y) { return bct_x((float)fmax(y, 0.0)); }
+__device__ __forceinline__ float bct_f(double y) { return bct_x(narrow_rn_pos(y)); }
 // inverse: x = (lambda z + 1)^(1/lambda) = t^10, 0 where t <= 0
 __device__ __forceinline__ float ibct_f(float z) {
   const float t = fmaxf(kLambda * z + 1.0f, 0.0f);
@@ -121,33 +121,55 @@ __global__ void hrr_coeff_kernel(DevMech m, int64_t n, int64_t ld, const double*
 }
 
 
-// normalised BF16 features X[i][0..63]; range flag (bit 1) against the training min/max
-__global__ void features_kernel(int64_t n, int64_t ld, const double* T, const double* p, const double* Y, int n_in,
-                                const float* norm, float margin, bf16* X, int32_t* flags, float* bcty, int K,
-                                const int32_t* idx) {
+// normalised BF16 features X[i][0..63]; range flag (bit 1) against the training min/max.  Bound by
+// memory (8 bytes per feature in, 128 per cell out).  A block takes 32 cells, lane = cell, so that the
+// species-major loads are contiguous; its 8 warps share the 64 features in pairs (a thread per cell
+// working through all of them left small calls at one long chain: learned step of 1,536 53-species
+// cells 295 -> 268 us), and the rows go out through shared memory in 16-byte pieces.
+constexpr int kFeatCells = 32;
+
+__global__ void __launch_bounds__(256) features_kernel(int64_t n, int64_t ld, const double* T, const double* p,
+                                                       const double* Y, int n_in, const float* norm, float margin,
+                                                       bf16* X, int32_t* flags, float* bcty, int K, const int32_t* idx) {
+  __shared__ __align__(16) bf16 tile[kFeatCells][kInPad + 8];
+  __shared__ int out[kFeatCells];
   const float* mean = norm;
   const float* sd = norm + n_in;
   const float* mn = norm + 2 * n_in;
   const float* mx = norm + 3 * n_in;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    int flag = 0;
-    const int64_t col = idx ? (int64_t)idx[i] : i;
-    __align__(16) bf16 row[kInPad];
-    for (int j = 0; j < kInPad; ++j) {
-      float v = 0.0f;
-      if (j < n_in) {
-        const float r = raw_feature(j, col, ld, T, p, Y);
-        const float span = mx[j] - mn[j];
-        if (!(r >= mn[j] - margin * span && r <= mx[j] + margin * span)) flag = 1;
-        v = (r - mean[j]) / sd[j];
-        if (bcty && j >= 2) bcty[(size_t)i * K + (j - 2)] = r;
-      }
-      row[j] = __float2bfloat16_rn(v);
-    }
-    uint4* dst = (uint4*)(X + (size_t)i * kInPad);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int64_t base = (int64_t)blockIdx.x * kFeatCells; base < n; base += (int64_t)gridDim.x * kFeatCells) {
+    if (threadIdx.x < kFeatCells) out[threadIdx.x] = 0;
+    __syncthreads();
+    const int64_t i = base + lane;
+    if (i < n) {
+      const int64_t col = idx ? (int64_t)idx[i] : i;
+      int flag = 0;
 #pragma unroll
-    for (int q = 0; q < kInPad / 8; ++q) dst[q] = ((const uint4*)row)[q];
-    if (flags) flags[i] = flag;
+      for (int q = 0; q < kInPad / 16; ++q) {
+        __nv_bfloat162 pair;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int j = 2 * (warp + 8 * q) + u;
+          float v = 0.0f;
+          if (j < n_in) {
+            const float r = raw_feature(j, col, ld, T, p, Y);
+            const float span = mx[j] - mn[j];
+            if (!(r >= mn[j] - margin * span && r <= mx[j] + margin * span)) flag = 1;
+            v = (r - mean[j]) / sd[j];
+            if (bcty && j >= 2) bcty[(size_t)i * K + (j - 2)] = r;
+          }
+          (u ? pair.y : pair.x) = __float2bfloat16_rn(v);
+        }
+        *(__nv_bfloat162*)&tile[lane][2 * (warp + 8 * q)] = pair;
+      }
+      if (flag) out[lane] = 1;   // every writer stores the same value
+    }
+    __syncthreads();
+    const int row = threadIdx.x >> 3, piece = threadIdx.x & 7;
+    if (base + row < n) *(uint4*)(X + (size_t)(base + row) * kInPad + 8 * piece) = *(const uint4*)&tile[row][8 * piece];
+    if (flags && threadIdx.x < kFeatCells && base + threadIdx.x < n) flags[base + threadIdx.x] = out[threadIdx.x];
+    __syncthreads();
   }
 }
 
@@ -199,6 +221,50 @@ __global__ void stats_partial_kernel(int64_t n, int64_t ld, const double* T, con
   }
 }
 
+// fmax(x, 0.0) on the bit pattern (NaN gives 0)
+__device__ __forceinline__ double pos_or_0(double x) {
+  return (unsigned long long)__double_as_longlong(x) - 1ull < 0x7ff0000000000000ull ? x : 0.0;
+}
+
+// lam from the E x (E + 1) system Mx of the element projection
+template <int EC>
+__device__ __forceinline__ void project_solve(double (&Mx)[EC][EC + 1], int E, double (&lam)[EC]) {
+  // Gauss-Jordan with partial pivoting; elements absent from both states have a zero
+  // row and column and keep lam = 0
+  bool live[EC];
+#pragma unroll
+  for (int c = 0; c < EC; ++c) live[c] = c < E && Mx[c][c] > 0.0;
+#pragma unroll
+  for (int c = 0; c < EC; ++c) {
+    if (!live[c]) continue;
+    int piv = c;
+#pragma unroll
+    for (int r = c + 1; r < EC; ++r)
+      if (live[r] && fabs(Mx[r][c]) > fabs(Mx[piv][c])) piv = r;
+    // rows swapped through a select chain (indices stay compile-time constants)
+#pragma unroll
+    for (int r = c + 1; r < EC; ++r) {
+      if (r == piv) {
+#pragma unroll
+        for (int j = 0; j <= EC; ++j) { const double t = Mx[c][j]; Mx[c][j] = Mx[r][j]; Mx[r][j] = t; }
+      }
+    }
+    if (!(fabs(Mx[c][c]) > 0.0)) continue;
+    const double d = 1.0 / Mx[c][c];
+#pragma unroll
+    for (int j = 0; j <= EC; ++j) Mx[c][j] *= d;
+#pragma unroll
+    for (int r = 0; r < EC; ++r) {
+      if (r == c) continue;
+      const double f = Mx[r][c];
+#pragma unroll
+      for (int j = 0; j <= EC; ++j) Mx[r][j] = fma(-f, Mx[c][j], Mx[r][j]);
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < EC; ++c) lam[c] = (live[c] && fabs(Mx[c][c] - 1.0) < 1e-9) ? Mx[c][EC] : 0.0;
+}
+
 // network output -> new state; flags: 1 range, 2 non-finite, 4 element residual, 8 T range, 16 |dT|
 // FP32 work of the update (the enthalpy and element sums of the old and predicted states, T
 // from h by Newton) reads FP32 copies of the NASA-7 and composition tables, so that no
@@ -219,6 +285,7 @@ __global__ void update_kernel(DevMech m, int64_t n, int64_t ld, double* T, const
     if (flag == 0) {
       float yn[CHEM_MAX_SPECIES];    // prediction (inverse Box-Cox, renormalised)
       float yp[CHEM_MAX_SPECIES];    // the state T' is solved for: projected, or yn when flagged
+      double pd[CHEM_MAX_SPECIES];   // the projected state in FP64 (unflagged cells)
       float eo[EC], en[EC];
       double eod[EC], lam[EC];
 #pragma unroll
@@ -247,7 +314,7 @@ __global__ void update_kernel(DevMech m, int64_t n, int64_t ld, double* T, const
             }
           }
         }
-        const float z = bct_x((float)fmax(y, 0.0)) + U[(size_t)slot * n_out_pad + k] * out_sd[k] + out_mean[k];
+        const float z = bct_f(y) + U[(size_t)slot * n_out_pad + k] * out_sd[k] + out_mean[k];
         finite = finite && isfinite(z);   // ibct_f would map a NaN to 0 (fmaxf)
         const float v = ibct_f(z);
         yn[k] = v;
@@ -283,7 +350,7 @@ __global__ void update_kernel(DevMech m, int64_t n, int64_t ld, double* T, const
             Mx[a1][EC] = eod[a1];
           }
           for (int k = 0; k < K; ++k) {
-            const double wk = (double)yn[k];
+            const double wk = widen_exact(yn[k]);
 #pragma unroll
             for (int a1 = 0; a1 < EC; ++a1) {
               if (a1 < E && m.compW32[(size_t)k * E + a1] != 0.0f) {
@@ -300,47 +367,15 @@ __global__ void update_kernel(DevMech m, int64_t n, int64_t ld, double* T, const
           for (int a1 = 0; a1 < EC; ++a1)
 #pragma unroll
             for (int a2 = 0; a2 < a1; ++a2) Mx[a1][a2] = Mx[a2][a1];
-          // Gauss-Jordan with partial pivoting; elements absent from both states have a zero
-          // row and column and keep lam = 0
-          bool live[EC];
-#pragma unroll
-          for (int c = 0; c < EC; ++c) live[c] = c < E && Mx[c][c] > 0.0;
-#pragma unroll
-          for (int c = 0; c < EC; ++c) {
-            if (!live[c]) continue;
-            int piv = c;
-#pragma unroll
-            for (int r = c + 1; r < EC; ++r)
-              if (live[r] && fabs(Mx[r][c]) > fabs(Mx[piv][c])) piv = r;
-            // rows swapped through a select chain (indices stay compile-time constants)
-#pragma unroll
-            for (int r = c + 1; r < EC; ++r) {
-              if (r == piv) {
-#pragma unroll
-                for (int j = 0; j <= EC; ++j) { const double t = Mx[c][j]; Mx[c][j] = Mx[r][j]; Mx[r][j] = t; }
-              }
-            }
-            if (!(fabs(Mx[c][c]) > 0.0)) continue;
-            const double d = 1.0 / Mx[c][c];
-#pragma unroll
-            for (int j = 0; j <= EC; ++j) Mx[c][j] *= d;
-#pragma unroll
-            for (int r = 0; r < EC; ++r) {
-              if (r == c) continue;
-              const double f = Mx[r][c];
-#pragma unroll
-              for (int j = 0; j <= EC; ++j) Mx[r][j] = fma(-f, Mx[c][j], Mx[r][j]);
-            }
-          }
-#pragma unroll
-          for (int c = 0; c < EC; ++c) lam[c] = (live[c] && fabs(Mx[c][c] - 1.0) < 1e-9) ? Mx[c][EC] : 0.0;
+          project_solve<EC>(Mx, E, lam);
           for (int k = 0; k < K; ++k) {
             double cl = 0.0;
 #pragma unroll
             for (int e = 0; e < EC; ++e)
               if (e < E && m.compW32[(size_t)k * E + e] != 0.0f) cl = fma(m.compW[(size_t)k * E + e], lam[e], cl);
-            const double yd = (double)yn[k];
-            yp[k] = (float)fmax(fma(yd, cl, yd), 0.0);
+            const double yd = widen_exact(yn[k]);
+            pd[k] = fma(yd, cl, yd);
+            yp[k] = narrow_rn_pos(pd[k]);
           }
         } else {
           for (int k = 0; k < K; ++k) yp[k] = yn[k];
@@ -366,21 +401,198 @@ __global__ void update_kernel(DevMech m, int64_t n, int64_t ld, double* T, const
         else if (Tn < Tmin || Tn > Tmax) flag |= 8;
         else if (dTmax > 0.0f && fabsf(Tn - T0) > dTmax) flag |= 16;
         if (!flag) {
-          // the projected state in FP64 (accepted cells were projected)
-          for (int k = 0; k < K; ++k) {
-            double cl = 0.0;
-#pragma unroll
-            for (int e = 0; e < EC; ++e)
-              if (e < E && m.compW32[(size_t)k * E + e] != 0.0f) cl = fma(m.compW[(size_t)k * E + e], lam[e], cl);
-            const double yd = (double)yn[k];
-            Y[(size_t)k * ld + i] = fmax(fma(yd, cl, yd), 0.0);
-          }
+          for (int k = 0; k < K; ++k) Y[(size_t)k * ld + i] = pos_or_0(pd[k]);
           T[i] = (double)Tn;
         }
       }
     }
     flags[slot] = flag;
     status[slot] = flag ? CHEM_CELL_ANN_FALLBACK : CHEM_CELL_OK;
+  }
+}
+
+// The same update with one warp per cell, for calls with few cells.  A thread per cell is a chain of
+// several hundred FP64 operations (64 cycles each) and as many memory latencies, 174 us for any
+// number of cells up to 78,000; a warp spreads the species over its lanes and the sums over
+// species over its lanes too (every sum runs in species order in one lane: the same bits), at 19
+// thousand FP64 cycles per cell instead of 1.4.  Learned step of 1,536 53-species cells: 268 -> 157 us;
+// by these rates the two forms meet near 10,000 cells (kUpdateWarpCells).
+constexpr int kUpdateWarps = 4;
+constexpr int64_t kUpdateWarpCells = 8192;
+
+template <int EC>
+struct UpdateSmem {
+  double comp[EC][CHEM_MAX_SPECIES + 1];     // composition / W, [element][species]
+  float comp32[EC][CHEM_MAX_SPECIES + 1];
+  float one[CHEM_MAX_SPECIES + 1];
+  struct Warp {
+    double y[CHEM_MAX_SPECIES + 1];          // Y, then the prediction
+    float p[CHEM_MAX_SPECIES + 1], q[CHEM_MAX_SPECIES + 1], v[CHEM_MAX_SPECIES + 1], yf[CHEM_MAX_SPECIES + 1];
+  } w[kUpdateWarps];
+};
+
+template <int EC>
+__global__ void __launch_bounds__(32 * kUpdateWarps) update_warp_kernel(
+    DevMech m, int64_t n, int64_t ld, double* T, double* Y, const float* U, int n_out_pad, const float* out_mean,
+    const float* out_sd, int32_t* flags, int32_t* status, float elem_tol, float Tmin, float Tmax, float dTmax,
+    const int32_t* idx) {
+  constexpr unsigned int full = 0xffffffffu;
+  constexpr int NS = EC * (EC + 1) / 2 + EC;   // sums of the projection: upper triangle, then right-hand sides
+  __shared__ UpdateSmem<EC> sm;
+  const int K = m.K, E = m.E, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int q = threadIdx.x; q < EC * K; q += blockDim.x) {
+    const int e = q / K, k = q % K;
+    sm.comp[e][k] = e < E ? m.compW[(size_t)k * E + e] : 0.0;
+    sm.comp32[e][k] = e < E ? m.compW32[(size_t)k * E + e] : 0.0f;
+  }
+  for (int k = threadIdx.x; k < K; k += blockDim.x) sm.one[k] = 1.0f;
+  __syncthreads();
+  auto& w = sm.w[warp];
+  const float Tmidf = (float)m.Tmid;
+  for (int64_t slot = (int64_t)blockIdx.x * kUpdateWarps + warp; slot < n; slot += (int64_t)gridDim.x * kUpdateWarps) {
+    const int64_t i = idx ? (int64_t)idx[slot] : slot;
+    int flag = flags[slot];
+    if (flag == 0) {
+      const float T0 = (float)T[i];
+      const int hi0 = T0 >= Tmidf ? 1 : 0;
+      bool fin = true;
+      for (int k = lane; k < K; k += 32) {
+        const double y = Y[(size_t)k * ld + i];
+        const float yf = narrow_f32(y);
+        const float* a = m.th32 + ((size_t)k * 2 + hi0) * 16;
+        const float hRT = a[5] + T0 * (a[6] + T0 * (a[7] + T0 * (a[8] + T0 * a[9]))) + a[10] / T0;
+        const float z = bct_f(y) + U[(size_t)slot * n_out_pad + k] * out_sd[k] + out_mean[k];
+        fin = fin && isfinite(z);
+        w.y[k] = y;
+        w.yf[k] = yf;
+        w.p[k] = yf * m.invW32[k];
+        w.q[k] = hRT;
+        w.v[k] = ibct_f(z);
+      }
+      fin = __all_sync(full, fin);
+      __syncwarp();
+      // sums in species order: lane 0 the old enthalpy, lane 1 the predictions, lanes 2 .. the old
+      // element moles; then in FP64 lanes 0 .. the old element moles
+      float s32 = 0.0f;
+      {
+        const float* P = lane == 0 ? w.p : lane == 1 ? w.v : w.yf;
+        const float* Q = lane == 0 ? w.q : lane == 1 ? sm.one : sm.comp32[max(0, min(lane - 2, EC - 1))];
+#pragma unroll 4
+        for (int k = 0; k < K; ++k) s32 = fmaf(P[k], Q[k], s32);
+      }
+      double eod = 0.0;
+      {
+        const double* Q = sm.comp[min(lane, EC - 1)];
+#pragma unroll 4
+        for (int k = 0; k < K; ++k)
+          if (Q[k] != 0.0) eod = fma(w.y[k], Q[k], eod);
+      }
+      const float h0 = __shfl_sync(full, s32, 0) * T0, ysum = __shfl_sync(full, s32, 1);
+      if (!fin || !(ysum > 0.0f) || !isfinite(ysum)) flag |= 2;
+      if (!flag) {
+        const float is = 1.0f / ysum;
+        __syncwarp();
+        for (int k = lane; k < K; k += 32) {
+          const float yn = w.v[k] * is;
+          w.v[k] = yn;
+          w.y[k] = widen_exact(yn);
+        }
+        __syncwarp();
+        float en = 0.0f;
+        {
+          const float* Q = sm.comp32[min(lane, EC - 1)];
+#pragma unroll 4
+          for (int k = 0; k < K; ++k) en = fmaf(w.v[k], Q[k], en);
+        }
+        float res = 0.0f;
+#pragma unroll
+        for (int e = 0; e < EC; ++e) {
+          const float eo = __shfl_sync(full, s32, 2 + e), ene = __shfl_sync(full, en, e);
+          if (e < E && eo > 0.0f) res = fmaxf(res, fabsf(ene - eo) / eo);
+        }
+        if (!(res <= elem_tol)) flag |= 4;
+        double lam[EC];
+#pragma unroll
+        for (int e = 0; e < EC; ++e) lam[e] = 0.0;
+        if (!flag) {
+          double Mx[EC][EC + 1];
+#pragma unroll
+          for (int r0 = 0; r0 < NS; r0 += 32) {
+            // this lane's sum: pair (a1, a2) of the upper triangle, or right-hand side a1
+            int a1 = 0, a2 = -1, q = r0 + lane;
+            if (q < EC * (EC + 1) / 2) {
+              while (q >= EC - a1) { q -= EC - a1; ++a1; }
+              a2 = a1 + q;
+            } else {
+              a1 = min(q - EC * (EC + 1) / 2, EC - 1);
+            }
+            const double e0 = __shfl_sync(full, eod, a1);
+            double acc = a2 < 0 ? e0 : 0.0;
+            const double *C1 = sm.comp[a1], *C2 = sm.comp[a2 < 0 ? 0 : a2];
+#pragma unroll 2
+            for (int k = 0; k < K; ++k) acc = fma(C1[k] * w.y[k], a2 < 0 ? -1.0 : C2[k], acc);
+            int at = 0;
+#pragma unroll
+            for (int b1 = 0; b1 < EC; ++b1)
+#pragma unroll
+              for (int b2 = b1; b2 < EC; ++b2, ++at)
+                if (at / 32 == r0 / 32) Mx[b1][b2] = Mx[b2][b1] = __shfl_sync(full, acc, at & 31);
+#pragma unroll
+            for (int b1 = 0; b1 < EC; ++b1, ++at)
+              if (at / 32 == r0 / 32) Mx[b1][EC] = __shfl_sync(full, acc, at & 31);
+          }
+          project_solve<EC>(Mx, E, lam);
+        }
+        // the state T' is solved for: projected (w.y in FP64, w.v), or the prediction when flagged
+        for (int k = lane; k < K; k += 32) {
+          if (!flag) {
+            double cl = 0.0;
+#pragma unroll
+            for (int e = 0; e < EC; ++e)
+              if (sm.comp32[e][k] != 0.0f) cl = fma(sm.comp[e][k], lam[e], cl);
+            const double yd = w.y[k], pd = fma(yd, cl, yd);
+            w.y[k] = pd;
+            w.v[k] = narrow_rn_pos(pd);
+          }
+          w.yf[k] = w.v[k] * m.invW32[k];
+        }
+        __syncwarp();
+        float Tn = T0;
+        for (int it = 0; it < 8; ++it) {
+          const int hi = Tn >= Tmidf ? 1 : 0;
+          for (int k = lane; k < K; k += 32) {
+            const float* a = m.th32 + ((size_t)k * 2 + hi) * 16;
+            const float cpR = a[0] + Tn * (a[1] + Tn * (a[2] + Tn * (a[3] + Tn * a[4])));
+            const float hRT = a[5] + Tn * (a[6] + Tn * (a[7] + Tn * (a[8] + Tn * a[9]))) + a[10] / Tn;
+            w.p[k] = w.yf[k] * hRT;
+            w.q[k] = cpR;
+          }
+          __syncwarp();
+          float s = 0.0f;   // lane 0: h, lane 1: c_p
+          const float *P = lane == 0 ? w.p : w.yf, *Q = lane == 0 ? sm.one : w.q;
+          const float f = lane == 0 ? Tn : 1.0f;
+#pragma unroll 4
+          for (int k = 0; k < K; ++k) s = fmaf(P[k], Q[k] * f, s);
+          __syncwarp();
+          const float h = __shfl_sync(full, s, 0), cp = __shfl_sync(full, s, 1);
+          const float dT = (h - h0) / cp;
+          Tn = fminf(fmaxf(Tn - dT, 200.0f), 6000.0f);
+          if (fabsf(dT) < 1e-4f * Tn) break;
+        }
+        if (!isfinite(Tn)) flag |= 2;
+        else if (Tn < Tmin || Tn > Tmax) flag |= 8;
+        else if (dTmax > 0.0f && fabsf(Tn - T0) > dTmax) flag |= 16;
+        if (!flag) {
+          for (int k = lane; k < K; k += 32) Y[(size_t)k * ld + i] = pos_or_0(w.y[k]);
+          if (lane == 0) T[i] = (double)Tn;
+        }
+      }
+      __syncwarp();
+    }
+    if (lane == 0) {
+      flags[slot] = flag;
+      status[slot] = flag ? CHEM_CELL_ANN_FALLBACK : CHEM_CELL_OK;
+    }
   }
 }
 
@@ -391,13 +603,21 @@ static int launch_update(const DevMech& m, int64_t n, int64_t ld, double* T, con
                          const float* U, int n_out_pad, const float* out_mean, const float* out_sd,
                          int32_t* flags, int32_t* status, float elem_tol, float Tmin, float Tmax, float dTmax,
                          const int32_t* idx, cudaStream_t s) {
-  const unsigned grid = grid_for(n, 128);
+  const unsigned grid = grid_for(n, 128), wgrid = (unsigned)((n + kUpdateWarps - 1) / kUpdateWarps);
 #define CHEM_UPDATE_CASE(EC)                                                                                  \
-  update_kernel<EC><<<grid, 128, 0, s>>>(m, n, ld, T, p, Y, U, n_out_pad, out_mean, out_sd, flags, status,  \
+  if (n <= kUpdateWarpCells)                                                                                \
+    update_warp_kernel<EC><<<wgrid, 32 * kUpdateWarps, 0, s>>>(m, n, ld, T, Y, U, n_out_pad, out_mean, out_sd, flags, \
+                                                               status, elem_tol, Tmin, Tmax, dTmax, idx);    \
+  else                                                                                                      \
+    update_kernel<EC><<<grid, 128, 0, s>>>(m, n, ld, T, p, Y, U, n_out_pad, out_mean, out_sd, flags, status,  \
                                          elem_tol, Tmin, Tmax, dTmax, idx)
-  if (m.E <= 3) CHEM_UPDATE_CASE(3);
-  else if (m.E <= 4) CHEM_UPDATE_CASE(4);
-  else CHEM_UPDATE_CASE(kMaxElem);
+  if (m.E <= 3) {
+    CHEM_UPDATE_CASE(3);
+  } else if (m.E <= 4) {
+    CHEM_UPDATE_CASE(4);
+  } else {
+    CHEM_UPDATE_CASE(kMaxElem);
+  }
 #undef CHEM_UPDATE_CASE
   return cuda_check(cudaGetLastError(), "update_kernel launch");
 }
@@ -1052,7 +1272,7 @@ int chem_ann_features(chem_ann a, int64_t n, int64_t ld, const double* T, const 
   if (n < 0 || ld < n || (n > 0 && (!T || !p || !Y || !X))) return set_error(CHEM_E_ARG, "chem_ann_features: bad arguments");
   if (flags && !(range_margin >= 0.0)) return set_error(CHEM_E_ARG, "chem_ann_features: range_margin must be >= 0");
   if (n == 0) return CHEM_OK;
-  features_kernel<<<grid_for(n, 256), 256, 0, (cudaStream_t)stream>>>(n, ld, T, p, Y, a->n_in, a->norm,
+  features_kernel<<<grid_for(n, kFeatCells), 256, 0, (cudaStream_t)stream>>>(n, ld, T, p, Y, a->n_in, a->norm,
                                                                      (float)range_margin, (bf16*)X, flags, bcty,
                                                                      a->K, nullptr);
   return cuda_check(cudaGetLastError(), "features_kernel launch");
@@ -1239,7 +1459,7 @@ int chem_step_ann(chem_mech mech, chem_ann a, int64_t n, int64_t ld, double dt, 
   unsigned int* queue = (unsigned int*)(w + off);
 
   // 1. features and range flags
-  features_kernel<<<grid_for(n, 256), 256, 0, s>>>(n, ld, T, p, Y, a->n_in, a->norm, (float)o.range_margin, X, flags,
+  features_kernel<<<grid_for(n, kFeatCells), 256, 0, s>>>(n, ld, T, p, Y, a->n_in, a->norm, (float)o.range_margin, X, flags,
                                                   nullptr, a->K, idx_in);
   if ((rc = cuda_check(cudaGetLastError(), "features_kernel launch"))) return rc;
   // 2. MLP on the tensor cores, chunk by chunk

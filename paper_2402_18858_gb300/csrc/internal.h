@@ -116,6 +116,21 @@ __device__ __forceinline__ double widen_f64(float f) {
 // noise level of the absolute tolerance, which the Box-Cox targets of a training set magnify to O(1)
 // (the 30-species training gradients moved by 1.4e-4).
 // ------------------------------------------------------------------------------------------
+// the float nearest to max(y, 0) (NaN gives 0), as (float)fmax(y, 0.0), on the integer pipe for results
+// in the middle of FP32's range: the FP64 maximum and conversion hold the FP64 pipe 64 cycles each
+__device__ __forceinline__ float narrow_rn_pos(double y) {
+  const unsigned int hi = (unsigned int)__double2hiint(y), lo = (unsigned int)__double2loint(y);
+  if (hi - 0x38100000u >= 0x0fc00000u) return (float)fmax(y, 0.0);   // zero, negative, tiny, huge, NaN
+  const unsigned int f = __funnelshift_l(lo, hi, 3) - (384u << 23);
+  return __uint_as_float(f + (((lo >> 28) & 1u) & (unsigned int)(((lo & 0x0fffffffu) | (f & 1u)) != 0u)));
+}
+
+// float to double, exact (FP32 subnormals by the conversion unit)
+__device__ __forceinline__ double widen_exact(float f) {
+  const unsigned int mag = __float_as_uint(f) & 0x7fffffffu;
+  return mag - 0x00800000u < 0x7f000000u ? widen_f64(f) : (double)f;
+}
+
 // FP64 exponential by the table-driven method (P. T. P. Tang, "Table-driven implementation of
 // the exponential function in IEEE floating-point arithmetic", ACM TOMS 15, 1989), here with a
 // 256-entry table: x = (256 k + j) ln2/256 + r, exp(x) = 2^k 2^(j/256) e^r, e^r - 1 from its
