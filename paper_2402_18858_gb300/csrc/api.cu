@@ -483,6 +483,31 @@ static int upload(const HostMech& hm, chem_mech_s* cm) {
       bal_P = 0;
     }
   }
+  // the runs dealt to the lanes of teams of two and four warps (see TeamBal)
+  std::vector<unsigned int> tb_e[2] = {{0u}, {0u}};
+  TeamBal tb[2] = {};
+  if (bal_P > 0) {
+    std::vector<std::vector<unsigned int>> runs((size_t)run_ptr[K]);
+    for (int e = 0; e < E_inc; ++e) {
+      const unsigned int v = bal[(size_t)(e % bal_P) * 32 + e / bal_P];
+      runs[(v >> 4) & 255u].push_back(v);
+    }
+    std::stable_sort(runs.begin(), runs.end(), [](const auto& a, const auto& b) { return a.size() > b.size(); });
+    for (int q = 0; q < 2; ++q) {
+      const int warps = 2 << q, lanes = 32 * warps;
+      std::vector<std::vector<unsigned int>> list(lanes);
+      for (size_t r = 0; r < runs.size(); ++r) list[r % lanes].insert(list[r % lanes].end(), runs[r].begin(), runs[r].end());
+      tb[q].single = (int)runs.size() <= lanes;
+      for (int h = 0; h < warps; ++h) {
+        size_t len = 0;
+        for (int l = 0; l < 32; ++l) len = std::max(len, list[32 * h + l].size());
+        tb[q].off[h] = (int)tb_e[q].size();
+        tb[q].len[h] = (int)len;
+        for (size_t i = 0; i < len; ++i)
+          for (int l = 0; l < 32; ++l) tb_e[q].push_back(i < list[32 * h + l].size() ? list[32 * h + l][i] : 0u);
+      }
+    }
+  }
   // two-partner reaction table (see DevMech::rsp2)
   std::vector<unsigned int> rsp2((size_t)std::max(I, 1), 0u);
   int arity2 = 1;
@@ -523,6 +548,7 @@ static int upload(const HostMech& hm, chem_mech_s* cm) {
   size_t ofexp = add(fexptab.data(), fexptab.size() * 8), oflog = add(flogtab.data(), flogtab.size() * 8);
   size_t obal = add(bal.data(), bal.size() * 4), orun = add(run_ptr.data(), run_ptr.size() * 4);
   size_t orsp2 = add(rsp2.data(), rsp2.size() * 4);
+  size_t otb[2] = {add(tb_e[0].data(), tb_e[0].size() * 4), add(tb_e[1].data(), tb_e[1].size() * 4)};
   std::vector<char> blob(total, 0);
   for (auto& p : pieces) std::memcpy(blob.data() + p.off, p.src, p.bytes);
   void* d = nullptr;
@@ -564,6 +590,9 @@ static int upload(const HostMech& hm, chem_mech_s* cm) {
   m.bal_P = bal_P;
   m.bal = (const unsigned int*)(b + obal);
   m.run_ptr = (const int*)(b + orun);
+  for (int q = 0; q < 2; ++q) tb[q].e = (const unsigned int*)(b + otb[q]);
+  m.tb2 = tb[0];
+  m.tb4 = tb[1];
   m.arity2 = arity2;
   m.rsp2 = (const unsigned int*)(b + orsp2);
   cm->dmem = d;

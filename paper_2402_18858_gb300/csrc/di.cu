@@ -24,6 +24,7 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <algorithm>
 #include <cstdint>
 
 #include "internal.h"
@@ -63,6 +64,10 @@ __device__ __forceinline__ bool finite_bits(double x) {
   return ((unsigned int)((unsigned long long)__double_as_longlong(x) >> 32) & 0x7ff00000u) != 0x7ff00000u;
 }
 
+// named barriers of a block: n threads (whole warps) arrive and wait, or arrive only
+__device__ __forceinline__ void bar_wait(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+
 __device__ __forceinline__ float wsumf(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(FULLMASK, v, o);
@@ -100,6 +105,8 @@ struct WarpMem {
   double* invd;   // n   reciprocal pivots
   double* ru;     // 50  step-size change matrix (0..24) and R(f) (25..49)
   int* perm;      // n   row permutation of the LU
+  double* tc;     // 5   teams only: T, ln T, 1/T, sum of concentrations, and the call (1: right-hand
+                  //     side, 0: leave)
   int ld;
 };
 
@@ -189,6 +196,7 @@ __device__ __forceinline__ WarpMem carve(double* base, int K, int I, int n, int 
   w.invd = p; p += n;
   w.ru = p; p += 50;
   w.perm = (int*)p;
+  w.tc = nullptr;
   return w;
 }
 
@@ -297,16 +305,168 @@ __device__ __forceinline__ void troe_phase(const DevMech& m, const WarpMem& w, d
 }
 
 // ------------------------------------------------------------------------------------------
+// pieces of the right-hand side that a team of warps shares (below); with one warp, its loops
+// ------------------------------------------------------------------------------------------
+template <bool FIX>
+__device__ __forceinline__ double exp_sel(const DevMech& m, double x) {
+  return FIX ? exp_s256_fix(x, m.fexptab) : exp_s256(x, m.exptab);
+}
+// exponential rounds: k_f of every non-falloff reaction (into w.q) and the five exponentials of each
+// falloff reaction (into w.tr), all items packed over the lanes.  Whole rounds before the first
+// falloff item (k_f only, no T term in the argument), every step / 32th:
+__device__ __forceinline__ int plain_rounds(const DevMech& m) { return m.n_tb_end / 32; }
+template <int NPL, bool FIX>
+__device__ __forceinline__ void kf_plain(const DevMech& m, const WarpMem& w, double lnT, double invT, int t0,
+                                         int step) {
+  const int end = 32 * plain_rounds(m), XP = m.XP;
+  const double2* xa = m.xarg;
+  // (two rounds at a time pay for the large mechanisms only: 53 species 144.0 -> 142.0 ms, 30 species
+  // 135.4 -> 137.4 ms, 9 species 3.53 -> 3.61 ms)
+#pragma unroll NPL
+  for (int t = t0; t < end; t += step) {
+    const double2 x01 = __ldg(xa + t);
+    w.q[t] = exp_sel<FIX>(m, fma(-__ldg(&xa[XP + t].x), invT, fma(x01.y, lnT, x01.x)));
+  }
+}
+// the other items
+template <int NPL, bool FIX>
+__device__ __forceinline__ void kf_rest(const DevMech& m, const WarpMem& w, double T, double lnT, double invT, int lane) {
+  const int nb = m.n_tb_end, XP = m.XP;
+  const double2* xa = m.xarg;
+#pragma unroll NPL
+  for (int t = 32 * plain_rounds(m) + lane; t < m.n_x; t += 32) {
+    const double2 x01 = __ldg(xa + t), x23 = __ldg(xa + XP + t);
+    const double e = exp_sel<FIX>(m, fma(x23.y, T, fma(-x23.x, invT, fma(x01.y, lnT, x01.x))));
+    if (t < nb) {
+      w.q[t] = e;
+    } else {
+      const int u = t - nb, jt = u / 5;
+      w.tr[kTroeSlots * jt + (u - 5 * jt)] = e;
+    }
+  }
+}
+// net rate of a reaction, two-partner form:
+// q_j = k_f (C_a C_b - K_c^-1 C_c C_d) = k_f (C_a C_b - (e_a e_b)(u_c u_d)) with
+// e = exp(-g'/RT) p0/RT and u = exp(g'/RT) (RT/p0) C; a missing partner is the sentinel 1.
+// No predication on the reaction's arity, one rounding in the difference.
+__device__ __forceinline__ double net_rate(const DevMech& m, const WarpMem& w, double ctot, int j) {
+  const int nb = m.n_tb_end;
+  const unsigned int rs = __ldg(m.rsp2 + j);
+  double kf;
+  if (j < nb) kf = w.q[j];
+  else kf = w.tr[kTroeSlots * (j - nb) + 5];
+  if (j >= m.n_elem && j < nb) {
+    double M = ctot;
+#pragma unroll
+    for (int e = 0; e < kMaxEx; ++e) {
+      const int se = __ldg(m.ex_sp + (size_t)j * kMaxEx + e);
+      if (se >= 0) M += __ldg(m.ex_a + (size_t)j * kMaxEx + e) * w.C[se];
+    }
+    kf *= M;
+  }
+  const int r0 = rs & 255u, r1 = (rs >> 8) & 255u, p0 = (rs >> 16) & 255u, p1 = rs >> 24;
+  return kf * fma(-(w.eg[r0] * w.eg[r1]), w.ieg[p0] * w.ieg[p1], w.C[r0] * w.C[r1]);
+}
+// of reactions j0, j0 + step, .. below end
+__device__ __forceinline__ void net_rates(const DevMech& m, const WarpMem& w, double ctot, int j0, int end, int step) {
+  for (int j = j0; j < end; j += step) w.q[j] = net_rate(m, w, ctot, j);
+}
+// nu = +-1, +-2, +-3 of a production entry, built from its bits (no FP64 conversion)
+__device__ __forceinline__ double entry_nu(unsigned int e) {
+  const unsigned int a = e & 3u;
+  const unsigned int hw = (a == 1u ? 0x3ff00000u : a == 2u ? 0x40000000u : 0x40080000u) | ((e & 4u) << 29);
+  return __hiloint2double((int)hw, 0);
+}
+
+// ------------------------------------------------------------------------------------------
+// Teams: TW warps on one cell, for launches with few cells (one warp alone keeps one of the SM's four
+// FP64 units busy, and that half of the time: 48 thousand cycles per BDF step, of which 27 in the
+// right-hand side) and for mechanisms whose shared memory leaves few warps per SM.  Warp 0 integrates;
+// the others wait for its right-hand sides and take: warp 1 the falloff reactions with the
+// exponential rounds they are in, warps 2 .. the other exponential rounds, all of them their share of
+// the net rates and of the production rates' runs.  Every item is computed as by one warp, in the
+// same order within every sum: the same bits.  Barriers per right-hand side: 1 start (T, ln T, 1/T,
+// concentrations are there), 2 the plain rounds' k_f (all but warp 1), 3 the species' terms (for
+// warp 1), 4 net rates, 5 production runs.  Every wait is met in the same right-hand side, and warp 0
+// ends with a start whose call is 0.
+// ------------------------------------------------------------------------------------------
+// production runs, one (or more, `single` = 0) per lane of the team: lane L of warp h walks its list
+template <int TW>
+__device__ __forceinline__ void team_production(const DevMech& m, const WarpMem& w, int h, int lane) {
+  const TeamBal& b = TW == 2 ? m.tb2 : m.tb4;
+  const unsigned int* el = b.e + b.off[h] + lane;
+  const int n = b.len[h];
+  double* part = w.g;
+  double acc = 0.0;
+  if (b.single) {
+    // one run: nothing to clear (the padding comes after the run's end), so the sum is one chain of
+    // FMAs, its entries loaded ahead
+    for (int i = 0; i < n; i += 4) {
+      unsigned int e[4];
+      double q[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) e[u] = i + u < n ? __ldg(el + (i + u) * 32) : 0u;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) q[u] = w.q[e[u] >> 12];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (i + u < n) acc = fma(entry_nu(e[u]), q[u], acc);
+        if (e[u] & 8u) part[(e[u] >> 4) & 255u] = acc;
+      }
+    }
+  } else {
+    for (int i = 0; i < n; ++i) {
+      const unsigned int e = __ldg(el + i * 32);
+      if (e & 3u) {
+        acc = fma(entry_nu(e), w.q[e >> 12], acc);
+        if (e & 8u) {
+          part[(e >> 4) & 255u] = acc;
+          acc = 0.0;
+        }
+      }
+    }
+  }
+}
+
+// warps 1 .. TW - 1
+template <int NPL, int TW>
+__device__ void team_helper(const DevMech& m, const WarpMem& w, int wid, int lane) {
+  const int np = plain_rounds(m);
+  while (true) {
+    bar_wait(1, 32 * TW);
+    if (w.tc[4] == 0.0) return;
+    const double T = w.tc[0], lnT = w.tc[1], invT = w.tc[2], ctot = w.tc[3];
+    if (wid == 1) {
+      kf_rest<NPL, false>(m, w, T, lnT, invT, lane);
+      __syncwarp();
+      if (m.I > m.n_tb_end) troe_phase<false, false>(m, w, invT, ctot, lane);
+      bar_wait(3, 64);
+      net_rates(m, w, ctot, 32 * np + lane, m.I, 32);
+    } else {
+      kf_plain<NPL, false>(m, w, lnT, invT, 32 * (wid - 2) + lane, 32 * (TW - 2));
+      __syncwarp();
+      bar_wait(2, 32 * (TW - 1));
+      net_rates(m, w, ctot, 32 * (wid - 1) + lane, 32 * np, 32 * (TW - 1));
+    }
+    __syncwarp();
+    bar_wait(4, 32 * TW);
+    team_production<TW>(m, w, wid, lane);
+    __syncwarp();
+    bar_wait(5, 32 * TW);
+  }
+}
+
+// ------------------------------------------------------------------------------------------
 // right-hand side f(z) of the reactor, z = (Y_1..Y_K, T)  [Eq. 1]
 // ------------------------------------------------------------------------------------------
 // FIX: exponentials and logarithms in fixed point (rates); the integrator takes the FP64 forms
-template <int NPL, bool JAC, bool FIX>
+// TW > 1: warp 0 of a team
+template <int NPL, bool JAC, bool FIX, int TW = 1>
 __device__ void rhs_eval(const DevMech& m, const WarpMem& w, const CellP& cp0, const double (&y)[NPL],
                          double (&f)[NPL], LaneSp<NPL>& sp, CellSc& cs, int lane) {
   const int K = m.K, I = m.I;
   const double T = comp_get<NPL>(y, K);
   const double lnT = FIX ? log_t_fix(T, m.flogtab) : log_t(T, m.logtab), RT = kR * T;
-  auto exp_s = [&](double x) { return FIX ? exp_s256_fix(x, m.fexptab) : exp_s256(x, m.exptab); };
   // T >= T_mid on the bit patterns (both positive: they order like the values)
   const int hi = __double_as_longlong(T) >= __double_as_longlong(m.Tmid) ? 1 : 0;
   // pass 1: c_p/R per species and the two mixture sums sum Y/W and sum Y c_p/(R W)
@@ -349,7 +509,21 @@ __device__ void rhs_eval(const DevMech& m, const WarpMem& w, const CellP& cp0, c
   // kr / kf = 1/K_c = prod_r e_r prod_p (1/e_p) (RT/p0)^(sum nu): the pressure factor goes
   // into the per-species values, p0/RT with every reactant and RT/p0 with every product
   const double P0RT = (kP0 / kR) * invT, RTP0 = RT * (1.0 / kP0);
-  const bool two = !JAC && m.arity2;   // warp-uniform
+  const bool two = TW > 1 || (!JAC && m.arity2);   // warp-uniform
+  if (TW > 1) {
+#pragma unroll
+    for (int s = 0; s < NPL; ++s)
+      if (lane + 32 * s < K) w.C[lane + 32 * s] = rho * ywr[s];
+    if (lane == 0) {
+      w.tc[0] = T;
+      w.tc[1] = lnT;
+      w.tc[2] = invT;
+      w.tc[3] = ctot;
+      w.tc[4] = 1.0;
+    }
+    __syncwarp();
+    bar_wait(1, 32 * TW);
+  }
 #pragma unroll
   for (int s = 0; s < NPL; ++s) {
     const int k = lane + 32 * s;
@@ -366,7 +540,7 @@ __device__ void rhs_eval(const DevMech& m, const WarpMem& w, const CellP& cp0, c
       const double hRT = h0 + T * (h12.x + T * (h12.y + T * (h34.x + T * h34.y))) + h5 * invT;
       const double ng = fma(T, T * fma(T, fma(T, g45.y, g45.x), g23.y) + g23.x, fma(g6, invT, fma(g01.y, lnT, g01.x)));
       const double Ck = rho * ywr[s];
-      w.C[k] = Ck;
+      if (TW == 1) w.C[k] = Ck;
       w.hRT[k] = hRT;
       sp.hRT[s] = hRT;
       double e, ie;
@@ -387,58 +561,28 @@ __device__ void rhs_eval(const DevMech& m, const WarpMem& w, const CellP& cp0, c
       w.ieg[k] = ie * (two ? RTP0 * Ck : RTP0);
     }
   }
-  // exponential rounds: k_f of every non-falloff reaction (into w.q, read back by the same
-  // lane below) and the five exponentials of each falloff reaction (into w.tr), all items
-  // packed over the lanes
   const int nb = m.n_tb_end;
-  // whole rounds before the first falloff item: k_f only, no T term in the argument
-  const int n_plain = (nb / 32) * 32;
-  const int XP = m.XP;
-  const double2* xa = m.xarg;
-  // (two rounds at a time pay for the large mechanisms only: 53 species 144.0 -> 142.0 ms, 30 species
-  // 135.4 -> 137.4 ms, 9 species 3.53 -> 3.61 ms)
-#pragma unroll NPL
-  for (int t = lane; t < n_plain; t += 32) {
-    const double2 x01 = __ldg(xa + t);
-    w.q[t] = exp_s(fma(-__ldg(&xa[XP + t].x), invT, fma(x01.y, lnT, x01.x)));
-  }
-#pragma unroll NPL
-  for (int t = n_plain + lane; t < m.n_x; t += 32) {
-    const double2 x01 = __ldg(xa + t), x23 = __ldg(xa + XP + t);
-    const double e = exp_s(fma(x23.y, T, fma(-x23.x, invT, fma(x01.y, lnT, x01.x))));
-    if (t < nb) {
-      w.q[t] = e;
+  if (TW > 1) {
+    __syncwarp();
+    bar_arrive(3, 64);
+    if (TW == 2) {
+      kf_plain<NPL, FIX>(m, w, lnT, invT, lane, 32);
+      __syncwarp();
     } else {
-      const int u = t - nb, jt = u / 5;
-      w.tr[kTroeSlots * jt + (u - 5 * jt)] = e;
+      bar_wait(2, 32 * (TW - 1));
     }
+    net_rates(m, w, ctot, lane, 32 * plain_rounds(m), 32 * (TW - 1));
+    __syncwarp();
+    bar_wait(4, 32 * TW);
+  } else {
+    kf_plain<NPL, FIX>(m, w, lnT, invT, lane, 32);
+    kf_rest<NPL, FIX>(m, w, T, lnT, invT, lane);
+    __syncwarp();
+    if (I > nb) troe_phase<JAC, FIX>(m, w, invT, ctot, lane);
   }
-  __syncwarp();
-  if (I > nb) troe_phase<JAC, FIX>(m, w, invT, ctot, lane);
-  if (two) {
-    // q_j = k_f (C_a C_b - K_c^-1 C_c C_d) = k_f (C_a C_b - (e_a e_b)(u_c u_d)) with
-    // e = exp(-g'/RT) p0/RT and u = exp(g'/RT) (RT/p0) C; a missing partner is the sentinel 1.
-    // No predication on the reaction's arity, one rounding in the difference.
-    auto net = [&](unsigned int rs, double kf) {
-      const int r0 = rs & 255u, r1 = (rs >> 8) & 255u, p0 = (rs >> 16) & 255u, p1 = rs >> 24;
-      return kf * fma(-(w.eg[r0] * w.eg[r1]), w.ieg[p0] * w.ieg[p1], w.C[r0] * w.C[r1]);
-    };
-    for (int j = lane; j < I; j += 32) {
-      const unsigned int rs = __ldg(m.rsp2 + j);
-      double kf;
-      if (j < nb) kf = w.q[j];
-      else kf = w.tr[kTroeSlots * (j - nb) + 5];
-      if (j >= m.n_elem && j < nb) {
-        double M = ctot;
-#pragma unroll
-        for (int e = 0; e < kMaxEx; ++e) {
-          const int se = __ldg(m.ex_sp + (size_t)j * kMaxEx + e);
-          if (se >= 0) M += __ldg(m.ex_a + (size_t)j * kMaxEx + e) * w.C[se];
-        }
-        kf *= M;
-      }
-      w.q[j] = net(rs, kf);
-    }
+  if (TW > 1) {
+  } else if (two) {
+    net_rates(m, w, ctot, lane, I, 32);
   } else
   for (int j = lane; j < I; j += 32) {
     const int4 ra = __ldg((const int4*)(m.rsp + 8 * (size_t)j));
@@ -487,15 +631,16 @@ __device__ void rhs_eval(const DevMech& m, const WarpMem& w, const CellP& cp0, c
   // production rates wdot_k = sum_j nu_kj q_j
   const int P = m.bal_P;
   double* part = w.g;   // g, eg and ieg are dead from here on: 3K slots for the runs
-  if (P > 0) {
+  if (TW > 1) {
+    team_production<TW>(m, w, 0, lane);
+    __syncwarp();
+    bar_wait(5, 32 * TW);
+  } else if (P > 0) {
     double acc = 0.0;
     for (int i = 0; i < P; ++i) {
       const unsigned int e = __ldg(m.bal + (size_t)i * 32 + lane);
       if (e & 3u) {
-        // nu = +-1, +-2, +-3 built from its bits (no FP64 conversion)
-        const unsigned int a = e & 3u;
-        const unsigned int hw = (a == 1u ? 0x3ff00000u : a == 2u ? 0x40000000u : 0x40080000u) | ((e & 4u) << 29);
-        acc = fma(__hiloint2double((int)hw, 0), w.q[e >> 12], acc);
+        acc = fma(entry_nu(e), w.q[e >> 12], acc);
         if (e & 8u) {
           part[(e >> 4) & 255u] = acc;
           acc = 0.0;
@@ -957,7 +1102,7 @@ struct DiOpts {
   int max_steps, jac_max_age;   // Jacobian reuse: a Newton failure with a stale one refreshes it
 };
 
-template <int NPL>
+template <int NPL, int TW>
 __device__ int integrate_cell(const DevMech& m, const WarpMem& w, double pc, double (&z)[NPL],
                               double dt, const DiOpts& o, int lane, int (&cnt)[4]) {
   const int n = m.n, K = m.K;
@@ -989,7 +1134,7 @@ __device__ int integrate_cell(const DevMech& m, const WarpMem& w, double pc, dou
   double D[kMaxOrd + 3][NPL];
   double f[NPL], y[NPL], d[NPL], dy[NPL], psi[NPL];
   // initial step (Hairer, Norsett & Wanner, Sec. II.4, order 1)
-  rhs_eval<NPL, false, false>(m, w, pp, z, f, sp, cs, lane);
+  rhs_eval<NPL, false, false, TW>(m, w, pp, z, f, sp, cs, lane);
   cnt[1]++;
 #pragma unroll
   for (int s = 0; s < NPL; ++s) isc[s] = __frcp_rn(fmaf(rtolf, fabsf(narrow_f32(z[s])), atolf[s]));
@@ -998,7 +1143,7 @@ __device__ int integrate_cell(const DevMech& m, const WarpMem& w, double pc, dou
   h0 = fmin(h0, dt);
 #pragma unroll
   for (int s = 0; s < NPL; ++s) y[s] = z[s] + h0 * f[s];
-  rhs_eval<NPL, false, false>(m, w, pp, y, dy, sp, cs, lane);
+  rhs_eval<NPL, false, false, TW>(m, w, pp, y, dy, sp, cs, lane);
   cnt[1]++;
 #pragma unroll
   for (int s = 0; s < NPL; ++s) dy[s] -= f[s];
@@ -1089,7 +1234,7 @@ __device__ int integrate_cell(const DevMech& m, const WarpMem& w, double pc, dou
     newton_iters = 0;
     for (int it = 0; it < kNewtonMax; ++it) {
       if (!(it == 0 && f_at_pred)) {
-        rhs_eval<NPL, false, false>(m, w, pp, y, f, sp, cs, lane);
+        rhs_eval<NPL, false, false, TW>(m, w, pp, y, f, sp, cs, lane);
         cnt[1]++;
       }
       bool ok = true;
@@ -1214,21 +1359,35 @@ __device__ __forceinline__ void load_cell(const DevMech& m, int64_t col, int64_t
   }
 }
 
-template <int NPL>
-__global__ void __launch_bounds__(NPL == 1 ? 384 : 256, 1) di_kernel(DevMech m, int64_t n, int64_t ld, double dt, double* T,
-                                                 const double* p, double* Y, const int32_t* idx, DiOpts o,
-                                                 int32_t* status, int32_t* stats, unsigned int* queue,
-                                                 size_t warp_bytes, const int32_t* n_dev) {
+// With n_dev, a launch works n_lo < *n_dev <= n_hi cells and otherwise none: the fallback of the learned
+// step, whose cell count only the device knows, launches the team form for few cells and another for many.
+template <int NPL, int TW>
+__global__ void __launch_bounds__(TW > 1 ? 32 * TW : NPL == 1 ? 384 : 256, TW > 1 ? (NPL == 1 ? 3 : 10 / TW) : 1)
+di_kernel(
+    DevMech m, int64_t n, int64_t ld, double dt, double* T, const double* p, double* Y, const int32_t* idx, DiOpts o,
+    int32_t* status, int32_t* stats, unsigned int* queue, size_t warp_bytes, const int32_t* n_dev, int64_t n_lo,
+    int64_t n_hi) {
   extern __shared__ double smem[];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int nT = m.I - m.n_tb_end;
-  const WarpMem w = carve((double*)((char*)smem + wid * warp_bytes), m.K, m.I, m.n, nT, true, true,
-                          NPL > 1 && di_use_j32(m.K, m.I, m.n, nT));
   // n_dev (optional): the number of entries of idx actually filled, known only on the device
-  const int64_t n_eff = n_dev ? min(n, (int64_t)max(*n_dev, 0)) : n;
+  int64_t n_eff = n;
+  if (n_dev) {
+    n_eff = min(n, (int64_t)max(*n_dev, 0));
+    if (n_eff <= n_lo || n_eff > n_hi) n_eff = 0;
+  }
+  WarpMem w = carve((double*)((char*)smem + (TW > 1 ? 0 : wid) * warp_bytes), m.K, m.I, m.n, nT, true, true,
+                    NPL > 1 && di_use_j32(m.K, m.I, m.n, nT));
+  if (TW > 1) {
+    w.tc = (double*)((char*)smem + warp_bytes);
+    if (wid > 0) {
+      team_helper<NPL, TW>(m, w, wid, lane);
+      return;
+    }
+  }
   // the first cells are dealt out one per block and then round again (few cells spread over the
   // SMs), the rest come from the queue as warps fall free
-  const unsigned int n_warps = gridDim.x * (blockDim.x >> 5);
+  const unsigned int n_warps = gridDim.x * (TW > 1 ? 1 : blockDim.x >> 5);
   unsigned int slot = wid * gridDim.x + blockIdx.x;
   for (; (int64_t)slot < n_eff; slot = __shfl_sync(FULLMASK, slot, 0)) {
     const int64_t col = idx ? (int64_t)idx[slot] : (int64_t)slot;
@@ -1240,7 +1399,7 @@ __global__ void __launch_bounds__(NPL == 1 ? 384 : 256, 1) di_kernel(DevMech m, 
       cnt[0] = cnt[1] = cnt[2] = cnt[3] = 0;
     } else {
       load_cell<NPL>(m, col, ld, T, Y, z, lane);
-      st = integrate_cell<NPL>(m, w, p[col], z, dt, o, lane, cnt);
+      st = integrate_cell<NPL, TW>(m, w, p[col], z, dt, o, lane, cnt);
       if (st == CHEM_CELL_OK) {
 #pragma unroll
         for (int s = 0; s < NPL; ++s) {
@@ -1260,6 +1419,11 @@ __global__ void __launch_bounds__(NPL == 1 ? 384 : 256, 1) di_kernel(DevMech m, 
       }
       slot = n_warps + atomicAdd(queue, 1u);
     }
+  }
+  if (TW > 1) {
+    if (lane == 0) w.tc[4] = 0.0;
+    __syncwarp();
+    bar_wait(1, 32 * TW);
   }
 }
 
@@ -1436,10 +1600,26 @@ int launch_di(const DevMech& m, int64_t n, int64_t ld, double dt, double* T, con
   const size_t wb = di_smem_per_warp(m);
   DiOpts o{opts.rtol, opts.atol_Y, opts.atol_T, opts.newton_tol, opts.max_steps, opts.jac_max_age};
   if (n > (int64_t)0x7fffffff) return set_error(CHEM_E_ARG, "chem_step_di: too many cells in one call");
-  auto launch = [&](auto kern) -> int {
+  const int sms = sm_count();
+  auto go = [&](auto kern, int wpb, int per_sm, size_t smem, int64_t blocks, int64_t lo, int64_t hi) -> int {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)std::min<int64_t>(blocks, (int64_t)sms * per_sm));
+    cfg.blockDim = dim3(32 * wpb);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    // what shared memory the resident blocks leave goes to L1, for the mechanism tables
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr[0].val.sharedMemCarveout = (unsigned)std::min<size_t>(100, (per_sm * (smem + 1024) * 100 + 228 * 1024 - 1) / (228 * 1024));
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cuda_check(cudaLaunchKernelEx(&cfg, kern, m, n, ld, dt, T, p, Y, idx, o, status, stats, queue, wb, n_dev, lo, hi),
+                      "di_kernel launch");
+  };
+  auto launch = [&](auto kern, int64_t lo, int64_t hi) -> int {
     // block shape (warps) that keeps the most warps resident per SM, the widest of equal ones (its
     // warps are dealt evenly to the SM's four sub-partitions, each of which has its own FP64 unit)
-    const int optin = smem_optin(), sms = sm_count();
+    const int optin = smem_optin();
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
     cudaFuncAttributes fa;
     if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) return cuda_check(cudaGetLastError(), "di_kernel attributes");
@@ -1451,26 +1631,45 @@ int launch_di(const DevMech& m, int64_t n, int64_t ld, double dt, double* T, con
       if (blocks * cand > wpb * per_sm) { wpb = cand; per_sm = blocks; }
     }
     if (wpb == 0) return set_error(CHEM_E_UNSUPPORTED, "mechanism needs more shared memory per warp than the device has");
-    // fewer cells than resident warps: one smaller block per SM, and what shared memory it leaves
-    // goes to L1, which then holds the mechanism tables
+    // fewer cells than resident warps: one smaller block per SM
     if (n < (int64_t)sms * wpb * per_sm) {
       wpb = (int)std::min<int64_t>(wpb, std::max<int64_t>(1, (n + sms - 1) / sms));
-      per_sm = std::max<int64_t>(1, (n + (int64_t)sms * wpb - 1) / ((int64_t)sms * wpb));
+      per_sm = (int)std::max<int64_t>(1, (n + (int64_t)sms * wpb - 1) / ((int64_t)sms * wpb));
     }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)std::min<int64_t>((n + wpb - 1) / wpb, (int64_t)sms * per_sm));
-    cfg.blockDim = dim3(32 * wpb);
-    cfg.dynamicSmemBytes = (size_t)wpb * wb;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
-    attr[0].val.sharedMemCarveout = (unsigned)std::min<size_t>(100, (per_sm * (cfg.dynamicSmemBytes + 1024) * 100 + 228 * 1024 - 1) / (228 * 1024));
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cuda_check(cudaLaunchKernelEx(&cfg, kern, m, n, ld, dt, T, p, Y, idx, o, status, stats, queue, wb, n_dev),
-                      "di_kernel launch");
+    return go(kern, wpb, per_sm, (size_t)wpb * wb, (n + wpb - 1) / wpb, lo, hi);
   };
-  return m.n <= 32 ? launch(di_kernel<1>) : launch(di_kernel<2>);
+  // a team's blocks per SM (0: they do not fit), at most enough for n cells
+  auto team_blocks = [&](auto kern, int tw) -> int {
+    const size_t smem = wb + 64;
+    int blocks = 0;
+    if (smem > (size_t)smem_optin()) return 0;
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin());
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kern, 32 * tw, smem);
+    return (int)std::min<int64_t>(blocks, (n + sms - 1) / sms);
+  };
+  const bool teams = m.arity2 && m.bal_P > 0;
+  // Cells up to one round of teams of four (three per SM up to 32 unknowns, two above: registers) go by
+  // teams of four, more by `many`.  One warp per cell -> teams (5 us
+  // at rtol 1e-6), 30 species: 11 cells 5.43 -> 4.20 ms,
+  // 152 7.15 -> 5.65, 456 9.07 -> 7.25; in a second round teams lose (608 cells 7.53 -> 7.73, 912 9.10 ->
+  // 10.18 ms).  53 species: 11 cells 11.8 -> 9.9 ms, 304 13.2 -> 11.1; teams of two, which take the same
+  // shared memory per cell as one warp, beyond (456 cells 13.1 -> 12.5 ms, 912 20.0 -> 18.9, 1824 29.8 ->
+  // 28.5; 3001 cells over 10 us at the default tolerances 142 -> 136 ms): 45 KB per cell leave five
+  // warps per SM, and teams make them ten.  Up to 32 unknowns twelve warps are resident without.  (9
+  // species: one round of everything, no difference.)
+  auto by_count = [&](auto four, auto many) -> int {
+    const int per_sm = teams ? team_blocks(four, 4) : 0;
+    const int64_t few = (int64_t)sms * per_sm;
+    int rc = CHEM_OK;
+    if (per_sm > 0 && (n <= few || n_dev)) rc = go(four, 4, per_sm, wb + 64, n, -1, few);
+    if (!rc && n > few) rc = many(n_dev ? few : -1);
+    return rc;
+  };
+  if (m.n <= 32) return by_count(di_kernel<1, 4>, [&](int64_t lo) { return launch(di_kernel<1, 1>, lo, INT64_MAX); });
+  return by_count(di_kernel<2, 4>, [&](int64_t lo) {
+    const int per_sm = teams ? team_blocks(di_kernel<2, 2>, 2) : 0;
+    return per_sm > 0 ? go(di_kernel<2, 2>, 2, per_sm, wb + 64, n, lo, INT64_MAX) : launch(di_kernel<2, 1>, lo, INT64_MAX);
+  });
 }
 
 }  // namespace chem

@@ -19,6 +19,13 @@ constexpr double kDefaultNewtonTol = 0.2;   // Newton stop, in units of the loca
 // 0.2, 100 steps cost 2.9 % less time on the 30-species workload at unchanged parity)
 constexpr int kDefaultJacMaxAge = 100;
 
+// Production runs dealt to the lanes of a team of warps (longest first): warp h walks e[off[h] + 32 i +
+// lane], i < len[h], entries as DevMech::bal; single: no lane has more than one run
+struct TeamBal {
+  const unsigned int* e;
+  int off[4], len[4], single;
+};
+
 // Device-resident mechanism tables.  Reactions are stored sorted by kind:
 // [0, n_elem) elementary, [n_elem, n_tb_end) third-body, [n_tb_end, I) Troe falloff.
 struct DevMech {
@@ -80,6 +87,7 @@ struct DevMech {
   int bal_P;
   const unsigned int* bal;   // [bal_P][32]
   const int* run_ptr;        // [K+1]
+  TeamBal tb2, tb4;          // the same runs for teams of two and four warps
   // Two-partner form of the reactions, used when every reaction has at most two reactants and
   // two products (arity2 = 1): r0 | r1 << 8 | p0 << 16 | p1 << 24, a missing partner pointing at the
   // sentinel slot K of the per-species shared-memory vectors, which holds 1.
