@@ -104,7 +104,8 @@ def di_flop_model(m: wl.Mechanism) -> dict:
 
 
 def thermo_fp64_flops(K: int, mixed: bool) -> int:
-    """FP64 flops per cell of the property kernel.  Both modes: sum Y_k/W_k (K FMAs), the six
+    """FP64 flops per cell of the properties as FP64 sums (the FP64 mode's kernel takes Wilke's sums and
+    the exponentials to 64-bit fixed point on the integer pipe instead).  Both modes: sum Y_k/W_k (K FMAs), the six
     mixture coefficients A_i = sum_k Y_k a_ik/W_k (6K FMAs), c_p and h from them (~20).  FP64
     mode also: ln T and the reciprocals (~40); per species the mole fraction (2), the ln mu and
     ln lambda cubics (12), four exponentials (4 (EXP + 1)), the conductivity sums (4) and
@@ -731,7 +732,7 @@ def main():
     th_bytes = N * (m.n_species + 1) * 8 + N * 4 * 8
     th_gbs = th_bytes / (th_ms * 1e-3) / 1e9
     th_flops_cell = thermo_fp64_flops(m.n_species, mixed=False)
-    th_tf = th_flops_cell * N / (th_ms * 1e-3) / 1e12
+    th_fp64_floor_ms = th_flops_cell * N / (peak_gf * 1e9) * 1e3
 
     # the properties in the mixed mode (FP32 transport sums) beside the step's FP64 mode
     thm = []
@@ -810,11 +811,12 @@ def main():
                          "unit": "TFLOP/s", "frac": achieved_tf / (peak_gf / 1e3),
                          "traffic": DI_DRAM_BYTES_PER_CELL * N, "kernel": "di_kernel (FP64 DFMA pipe)",
                          "peak_source": "measured live: chem_fp64_peak_gflops DFMA probe"},
-            "thermo_roofline": {"bound": "alu", "achieved": th_tf, "peak": peak_gf / 1e3, "unit": "TFLOP/s",
-                                "frac": th_tf / (peak_gf / 1e3), "kernel": "thermo_kernel (FP64)",
-                                "flops_per_cell": th_flops_cell,
-                                "note": "FP64 Wilke sums (3 FMAs per species pair) bound it; HBM side: "
-                                        f"{th_gbs:.0f} GB/s = {th_gbs / hbm:.3f} of {hbm:.0f} (hbm_gbs {PEAKS['source']})",
+            "thermo_roofline": {"bound": "issue", "achieved": th_gbs, "peak": hbm, "unit": "GB/s",
+                                "frac": th_gbs / hbm, "kernel": "thermo64_kernel", "ms": th_ms,
+                                "fp64_flops_per_cell": th_flops_cell, "fp64_floor_ms": th_fp64_floor_ms,
+                                "note": "Wilke's sums in 64-bit fixed point on the integer pipe bound it (instruction "
+                                        "issue); fp64_floor_ms is what the same sums would take at the FP64 peak; "
+                                        f"hbm_gbs {PEAKS['source']}",
                                 "hbm_gbs": th_gbs, "hbm_frac": th_gbs / hbm},
             "thermo_mixed": {"ms": thm_ms, "cells_per_s": N / (thm_ms * 1e-3),
                              "fp64_flops_per_cell": thermo_fp64_flops(m.n_species, mixed=True),

@@ -102,7 +102,8 @@ typedef struct {
  * reactor (Eq. 1 with dT/dt = -sum_k h_k wdot_k / (rho c_p)), in place: T[i] and Y[:, i]
  * are overwritten with the state at t + dt; p[i] is constant.  Variable-order (1..5) BDF
  * with a modified Newton iteration (analytic Jacobian, dense LU with partial pivoting, all
- * FP64), one warp per cell.
+ * FP64), one warp or, for few cells or many unknowns, a team of two or four warps per cell
+ * (the same bits either way).
  *   idx      NULL to integrate cells 0..n-1, else int32 idx[n] lists the cell columns to
  *            integrate (indices into the ld-strided arrays, each < ld).
  *   opts     NULL for defaults.
@@ -369,9 +370,10 @@ void chem_server_free(chem_server server);
  * If h_in is not NULL, T is first solved from h(T, Y) = h_in[i] by Newton's method starting
  * at T[i] (|dT| < 1e-9 K, at most 50 iterations, clamped to [200, 6000] K), written to T_out
  * (which may alias T), and the properties are evaluated there.
- * All FP64 when mixed_precision == 0; with mixed_precision == 1 the O(K^2) Wilke and the
- * conductivity sums run in FP32 (relative error below 1e-5) while c_p, h and the Newton
- * solve stay FP64. */
+ * When mixed_precision == 0, c_p, h and the Newton solve run in FP64 and the transport sums in
+ * 64-bit fixed point (errors no larger than FP64 sums'); with mixed_precision == 1 the O(K^2)
+ * Wilke and the conductivity sums run in FP32 (relative error below 1e-5) while c_p, h and the
+ * Newton solve stay FP64. */
 int thermo_props(chem_mech mech, int64_t n, int64_t ld, const double* T, const double* Y,
                  double* cp, double* h, double* mu, double* kappa, const double* h_in,
                  double* T_out, int mixed_precision, chem_stream stream);
