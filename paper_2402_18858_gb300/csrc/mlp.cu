@@ -136,27 +136,28 @@ struct TileCfg {
 // row per lane and for four lanes per row.
 __device__ __forceinline__ uint32_t stage_slot(int r, int c) { return (uint32_t)(r * 64 + 16 * ((c + (r >> 1)) & 3)); }
 
-// rows 0 .. nrows - 1 of `dst` (row stride ld elements, 32 columns) from the staging buffer,
-// which holds this lane's row (lane = row) at stage_slot(lane, 0..3)
-__device__ __forceinline__ void flush_rows_bf16(const uint8_t* wbuf, bf16* dst, int64_t ld, int nrows, int lane) {
+// rows 0 .. nrows - 1 of `dst` (row stride ld elements, 8 nq columns) from the staging buffer,
+// which holds this lane's row (lane = row) at stage_slot(lane, 0 .. nq - 1)
+__device__ __forceinline__ void flush_rows_bf16(const uint8_t* wbuf, bf16* dst, int64_t ld, int nrows, int nq, int lane) {
   __syncwarp();
   const int c = lane & 3;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int r = (lane >> 2) + 8 * i;
-    if (r < nrows) *(uint4*)(dst + (size_t)r * ld + 8 * c) = *(const uint4*)(wbuf + stage_slot(r, c));
+    if (r < nrows && c < nq) *(uint4*)(dst + (size_t)r * ld + 8 * c) = *(const uint4*)(wbuf + stage_slot(r, c));
   }
   __syncwarp();
 }
 
-// the reverse: this lane's row (lane = row - row0) of src into pk; rows past nrows read zero
+// the reverse: this lane's row (lane = row - row0) of src into pk; rows past nrows and columns past
+// 8 nq read zero
 __device__ __forceinline__ void load_rows_bf16(uint4 (&pk)[4], uint8_t* wbuf, const bf16* src, int64_t ld,
-                                               int nrows, int lane) {
+                                               int nrows, int nq, int lane) {
   const int c = lane & 3;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int r = (lane >> 2) + 8 * i;
-    const uint4 v = r < nrows ? __ldg((const uint4*)(src + (size_t)r * ld + 8 * c)) : make_uint4(0u, 0u, 0u, 0u);
+    const uint4 v = r < nrows && c < nq ? __ldg((const uint4*)(src + (size_t)r * ld + 8 * c)) : make_uint4(0u, 0u, 0u, 0u);
     *(uint4*)(wbuf + stage_slot(r, c)) = v;
   }
   __syncwarp();
@@ -165,58 +166,75 @@ __device__ __forceinline__ void load_rows_bf16(uint4 (&pk)[4], uint8_t* wbuf, co
   __syncwarp();
 }
 
+// hidden-layer epilogues (0, 2) of 8 nq whole columns through the staging buffer (FULL: nq = 4)
+template <int EPI, bool FULL>
+__device__ __forceinline__ void epi_staged(float (&v)[32], int col0, int nq_, const GemmEpi& e, uint8_t* wbuf, int row0,
+                                           int nrows, int lane) {
+  const int nq = FULL ? 4 : nq_;
+  if (EPI == 0) {
+    // hidden layer forward: out = bf16(GELU(acc + b)); optional pre-activation copy.  Each
+    // group of 8 columns goes to the staging buffer as soon as it is made (few live registers)
+    if (e.bias) {
+      // the chunk's 32 biases as eight 16-byte broadcast loads (col0 is a multiple of 32)
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        if (q >= 2 * nq) break;
+        const ulonglong2 b4 = __ldg((const ulonglong2*)(e.bias + col0) + q);
+        upk2(add2(pk2(v[4 * q], v[4 * q + 1]), b4.x), v[4 * q], v[4 * q + 1]);
+        upk2(add2(pk2(v[4 * q + 2], v[4 * q + 3]), b4.y), v[4 * q + 2], v[4 * q + 3]);
+      }
+    }
+    if (e.zout) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        __align__(16) bf16 u[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) u[i] = __float2bfloat16_rn(v[8 * q + i]);
+        *(uint4*)(wbuf + stage_slot(lane, q)) = *(const uint4*)u;
+      }
+      flush_rows_bf16(wbuf, e.zout + (size_t)row0 * e.ldo + col0, e.ldo, nrows, nq, lane);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (q >= nq) break;
+      __align__(16) bf16 t[8];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) ((__nv_bfloat162*)t)[i] = gelu2_bf16(pk2(v[8 * q + 2 * i], v[8 * q + 2 * i + 1]));
+      *(uint4*)(wbuf + stage_slot(lane, q)) = *(const uint4*)t;
+    }
+    flush_rows_bf16(wbuf, (bf16*)e.out + (size_t)row0 * e.ldo + col0, e.ldo, nrows, nq, lane);
+  } else {
+    // hidden-layer backward: dZ = acc * GELU'(z)
+    uint4 zk[4];
+    load_rows_bf16(zk, wbuf, e.z + (size_t)row0 * e.ldz + col0, e.ldz, nrows, nq, lane);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const bf16* zin = (const bf16*)&zk[q];
+      __align__(16) bf16 t[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) t[i] = __float2bfloat16_rn(v[8 * q + i] * dgelu_f(__bfloat162float(zin[i])));
+      *(uint4*)(wbuf + stage_slot(lane, q)) = *(const uint4*)t;
+    }
+    flush_rows_bf16(wbuf, (bf16*)e.out + (size_t)row0 * e.ldo + col0, e.ldo, nrows, nq, lane);
+  }
+}
+
 // epilogue of one 32-column chunk of the accumulator rows of a warp: this lane's row is
 // row = row0 + lane, columns col0 .. col0 + nv - 1; rows row0 .. row0 + nrows - 1 exist.
 // Called by the whole warp (the staged BF16 paths synchronise it).
 template <int EPI>
 __device__ __forceinline__ void epi_chunk(float (&v)[32], int row, int col0, int nv, const GemmEpi& e,
                                           uint8_t* wbuf, int row0, int nrows, int lane) {
-  if ((EPI == 0 || EPI == 2) && nv == 32) {
-    if (EPI == 0) {
-      // hidden layer forward: out = bf16(GELU(acc + b)); optional pre-activation copy.  Each
-      // group of 8 columns goes to the staging buffer as soon as it is made (few live registers)
-      if (e.bias) {
-        // the chunk's 32 biases as eight 16-byte broadcast loads (col0 is a multiple of 32)
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const ulonglong2 b4 = __ldg((const ulonglong2*)(e.bias + col0) + q);
-          upk2(add2(pk2(v[4 * q], v[4 * q + 1]), b4.x), v[4 * q], v[4 * q + 1]);
-          upk2(add2(pk2(v[4 * q + 2], v[4 * q + 3]), b4.y), v[4 * q + 2], v[4 * q + 3]);
-        }
-      }
-      if (e.zout) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          __align__(16) bf16 u[8];
-#pragma unroll
-          for (int i = 0; i < 8; ++i) u[i] = __float2bfloat16_rn(v[8 * q + i]);
-          *(uint4*)(wbuf + stage_slot(lane, q)) = *(const uint4*)u;
-        }
-        flush_rows_bf16(wbuf, e.zout + (size_t)row0 * e.ldo + col0, e.ldo, nrows, lane);
-      }
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        __align__(16) bf16 t[8];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) ((__nv_bfloat162*)t)[i] = gelu2_bf16(pk2(v[8 * q + 2 * i], v[8 * q + 2 * i + 1]));
-        *(uint4*)(wbuf + stage_slot(lane, q)) = *(const uint4*)t;
-      }
-      flush_rows_bf16(wbuf, (bf16*)e.out + (size_t)row0 * e.ldo + col0, e.ldo, nrows, lane);
-    } else {
-      // hidden-layer backward: dZ = acc * GELU'(z)
-      uint4 zk[4];
-      load_rows_bf16(zk, wbuf, e.z + (size_t)row0 * e.ldz + col0, e.ldz, nrows, lane);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const bf16* zin = (const bf16*)&zk[q];
-        __align__(16) bf16 t[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) t[i] = __float2bfloat16_rn(v[8 * q + i] * dgelu_f(__bfloat162float(zin[i])));
-        *(uint4*)(wbuf + stage_slot(lane, q)) = *(const uint4*)t;
-      }
-      flush_rows_bf16(wbuf, (bf16*)e.out + (size_t)row0 * e.ldo + col0, e.ldo, nrows, lane);
-    }
-    return;
+  if (EPI == 0 || EPI == 2) {
+    // Whole groups of 8 columns go through the staging buffer, 16 bytes at a time (a last chunk of 8, 16 or
+    // 24 columns, as in layers 400, 504, 1000 or 2000 wide, once took 2-byte stores of a lane per row: forward
+    // of 30,001 cells through 64-2000-1000-504-53 232 -> 213 us, training step of 16,384 rows through
+    // 64-1600-800-400-30 536 -> 525 us).  Other remainders, or rows that do not start on 16
+    // bytes, element by element.
+    if (nv == 32) return epi_staged<EPI, true>(v, col0, 4, e, wbuf, row0, nrows, lane);
+    if ((nv & 7) == 0 && (((uintptr_t)e.out | (uintptr_t)e.zout | (uintptr_t)e.z | (uintptr_t)e.bias |
+                           (2 * e.ldo) | (EPI == 2 ? 2 * e.ldz : 0)) & 15) == 0)
+      return epi_staged<EPI, false>(v, col0, nv >> 3, e, wbuf, row0, nrows, lane);
   }
   if (row - row0 >= nrows) return;
   // every loop below is unrolled over the 32 columns with the ragged bound as a predicate: an
@@ -274,13 +292,14 @@ __device__ __forceinline__ void epi_chunk(float (&v)[32], int row, int col0, int
 }
 
 // Epilogue 4 (short-K kernel only): the hidden-layer forward of epilogue 0 without the
-// pre-activation copy, N a multiple of 32.  Each 32-column chunk is read from TMEM in four
+// pre-activation copy, N a multiple of 8 (a last chunk of 8 nq columns).  Each 32-column chunk is read from TMEM in four
 // 8-column pieces: with a whole 32-float chunk plus the GELU temporaries live, the short-K
 // kernel's 64 registers per thread spill.
-__device__ __forceinline__ void epi_gelu_x8(uint32_t taddr, int col0, const GemmEpi& e, uint8_t* wbuf,
+__device__ __forceinline__ void epi_gelu_x8(uint32_t taddr, int col0, int nq, const GemmEpi& e, uint8_t* wbuf,
                                             int row0, int nrows, int lane) {
 #pragma unroll
   for (int h = 0; h < 4; ++h) {
+    if (h >= nq) break;
     float v[8];
     tc::tmem_ld8(taddr + 8 * h, v);
     if (e.bias) {
@@ -298,7 +317,7 @@ __device__ __forceinline__ void epi_gelu_x8(uint32_t taddr, int col0, const Gemm
     for (int i = 0; i < 4; ++i) ((__nv_bfloat162*)t)[i] = gelu2_bf16(pk2(v[2 * i], v[2 * i + 1]));
     *(uint4*)(wbuf + stage_slot(lane, h)) = *(const uint4*)t;
   }
-  flush_rows_bf16(wbuf, (bf16*)e.out + (size_t)row0 * e.ldo + col0, e.ldo, nrows, lane);
+  flush_rows_bf16(wbuf, (bf16*)e.out + (size_t)row0 * e.ldo + col0, e.ldo, nrows, nq, lane);
 }
 
 // S (1..STAGES, a launch argument) stages in the ring: min(STAGES, K slabs), so that a
@@ -380,7 +399,7 @@ __global__ void __launch_bounds__(256, 4) gemm_bf16_kernel(const __grid_constant
       // the whole warp takes part (no early exit): the next tcgen05.ld and the staged stores
       // need every lane
       if constexpr (EPI == 4) {
-        epi_gelu_x8(taddr, n0 + c0, e, wbuf, row0, nrows, lane);
+        epi_gelu_x8(taddr, n0 + c0, min(4, (N - (n0 + c0)) >> 3), e, wbuf, row0, nrows, lane);
       } else {
         float v[32];
         tc::tmem_ld32(taddr, v);
@@ -940,7 +959,7 @@ static int launch_gemm_t(const bf16* A, int64_t lda, const bf16* B, int64_t ldb,
   if ((rc = make_map(&tb, B, N + (int64_t)(G - 1) * e.b_row, K + (int64_t)(G - 1) * e.b_col, ldb, BN))) return rc;
   const int nkb_all = (K + tc::BK - 1) / tc::BK;
   if constexpr (EPI == 4) {
-    if (nkb_all > 2 || G > 1 || N % 32) return set_error(CHEM_E_ARG, "gemm: epilogue 4 needs K <= 128, N % 32 == 0");
+    if (nkb_all > 2 || G > 1 || N % 8) return set_error(CHEM_E_ARG, "gemm: epilogue 4 needs K <= 128, N % 8 == 0");
   } else if (nkb_all > 2 || G > 1) {
     if constexpr (BN >= 128) {
       // long K, wide tiles, at least one 256-row block: CTA pairs (cta_group::2)
@@ -1026,7 +1045,8 @@ int gemm_bf16(int epi, const bf16* A, int64_t lda, const bf16* B, int64_t ldb, i
     }
   }
   // the first layer's forward without a pre-activation copy: the short-K kernel's lean GELU epilogue
-  const bool gelu_x8 = epi == 0 && !e.zout && e.groups <= 1 && K <= 2 * tc::BK && N % 32 == 0;
+  const bool gelu_x8 = epi == 0 && !e.zout && e.groups <= 1 && K <= 2 * tc::BK && N % 8 == 0 && e.ldo % 8 == 0 &&
+                       (((uintptr_t)e.out | (uintptr_t)e.bias) & 15) == 0;
 #define CHEM_GEMM_CASE(BNV)                                                                    \
   if (bn == BNV) {                                                                             \
     switch (epi) {                                                                             \
