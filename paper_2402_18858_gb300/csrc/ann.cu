@@ -477,8 +477,12 @@ __global__ void __launch_bounds__(32 * kUpdateWarps) update_warp_kernel(
       {
         const float* P = lane == 0 ? w.p : lane == 1 ? w.v : w.yf;
         const float* Q = lane == 0 ? w.q : lane == 1 ? sm.one : sm.comp32[max(0, min(lane - 2, EC - 1))];
+        // element sums leave out the species without the element: an infinite fraction there must not
+        // meet the zero coefficient
+        const bool all = lane < 2;
 #pragma unroll 4
-        for (int k = 0; k < K; ++k) s32 = fmaf(P[k], Q[k], s32);
+        for (int k = 0; k < K; ++k)
+          if (all || Q[k] != 0.0f) s32 = fmaf(P[k], Q[k], s32);
       }
       double eod = 0.0;
       {
