@@ -265,6 +265,19 @@ __device__ __forceinline__ void project_solve(double (&Mx)[EC][EC + 1], int E, d
   for (int c = 0; c < EC; ++c) lam[c] = (live[c] && fabs(Mx[c][c] - 1.0) < 1e-9) ? Mx[c][EC] : 0.0;
 }
 
+// What both forms of the update compute per species, with the roundings written out: a contraction that
+// the compiler chose in one form only would give a cell other bits in a small call than in a large one
+// (the projection's ill-conditioned system magnifies a last bit).
+__device__ __forceinline__ float cpR_of(const float* a, float T) {
+  return fmaf(T, fmaf(T, fmaf(T, fmaf(T, a[4], a[3]), a[2]), a[1]), a[0]);
+}
+__device__ __forceinline__ float hRT_of(const float* a, float T) {
+  return __fadd_rn(fmaf(T, fmaf(T, fmaf(T, fmaf(T, a[9], a[8]), a[7]), a[6]), a[5]), __fdiv_rn(a[10], T));
+}
+__device__ __forceinline__ float predict_z(double y, float u, float sd, float mean) {
+  return __fadd_rn(fmaf(u, sd, bct_f(y)), mean);
+}
+
 // network output -> new state; flags: 1 range, 2 non-finite, 4 element residual, 8 T range, 16 |dT|
 // FP32 work of the update (the enthalpy and element sums of the old and predicted states, T
 // from h by Newton) reads FP32 copies of the NASA-7 and composition tables, so that no
@@ -302,8 +315,7 @@ __global__ void update_kernel(DevMech m, int64_t n, int64_t ld, double* T, const
         const double y = Y[(size_t)k * ld + i];
         const float yf = narrow_f32(y);
         const float* a = m.th32 + ((size_t)k * 2 + hi0) * 16;
-        const float hRT = a[5] + T0 * (a[6] + T0 * (a[7] + T0 * (a[8] + T0 * a[9]))) + a[10] / T0;
-        h0 += yf * m.invW32[k] * hRT;
+        h0 = fmaf(__fmul_rn(yf, m.invW32[k]), hRT_of(a, T0), h0);
 #pragma unroll
         for (int e = 0; e < EC; ++e) {
           if (e < E) {
@@ -314,7 +326,7 @@ __global__ void update_kernel(DevMech m, int64_t n, int64_t ld, double* T, const
             }
           }
         }
-        const float z = bct_f(y) + U[(size_t)slot * n_out_pad + k] * out_sd[k] + out_mean[k];
+        const float z = predict_z(y, U[(size_t)slot * n_out_pad + k], out_sd[k], out_mean[k]);
         finite = finite && isfinite(z);   // ibct_f would map a NaN to 0 (fmaxf)
         const float v = ibct_f(z);
         yn[k] = v;
@@ -354,8 +366,8 @@ __global__ void update_kernel(DevMech m, int64_t n, int64_t ld, double* T, const
 #pragma unroll
             for (int a1 = 0; a1 < EC; ++a1) {
               if (a1 < E && m.compW32[(size_t)k * E + a1] != 0.0f) {
-                const double c1 = m.compW[(size_t)k * E + a1] * wk;
-                Mx[a1][EC] -= c1;
+                const double c1 = __dmul_rn(m.compW[(size_t)k * E + a1], wk);
+                Mx[a1][EC] = __dsub_rn(Mx[a1][EC], c1);
 #pragma unroll
                 for (int a2 = a1; a2 < EC; ++a2)
                   if (a2 < E && m.compW32[(size_t)k * E + a2] != 0.0f)
@@ -387,11 +399,9 @@ __global__ void update_kernel(DevMech m, int64_t n, int64_t ld, double* T, const
           float h = 0.0f, cp = 0.0f;
           for (int k = 0; k < K; ++k) {
             const float* a = m.th32 + ((size_t)k * 2 + hi) * 16;
-            const float yw = yp[k] * m.invW32[k];
-            const float cpR = a[0] + Tn * (a[1] + Tn * (a[2] + Tn * (a[3] + Tn * a[4])));
-            const float hRT = a[5] + Tn * (a[6] + Tn * (a[7] + Tn * (a[8] + Tn * a[9]))) + a[10] / Tn;
-            h += yw * hRT * Tn;
-            cp += yw * cpR;
+            const float yw = __fmul_rn(yp[k], m.invW32[k]);
+            h = fmaf(__fmul_rn(yw, hRT_of(a, Tn)), Tn, h);
+            cp = fmaf(yw, cpR_of(a, Tn), cp);
           }
           const float dT = (h - h0) / cp;
           Tn = fminf(fmaxf(Tn - dT, 200.0f), 6000.0f);
@@ -460,13 +470,12 @@ __global__ void __launch_bounds__(32 * kUpdateWarps) update_warp_kernel(
         const double y = Y[(size_t)k * ld + i];
         const float yf = narrow_f32(y);
         const float* a = m.th32 + ((size_t)k * 2 + hi0) * 16;
-        const float hRT = a[5] + T0 * (a[6] + T0 * (a[7] + T0 * (a[8] + T0 * a[9]))) + a[10] / T0;
-        const float z = bct_f(y) + U[(size_t)slot * n_out_pad + k] * out_sd[k] + out_mean[k];
+        const float z = predict_z(y, U[(size_t)slot * n_out_pad + k], out_sd[k], out_mean[k]);
         fin = fin && isfinite(z);
         w.y[k] = y;
         w.yf[k] = yf;
-        w.p[k] = yf * m.invW32[k];
-        w.q[k] = hRT;
+        w.p[k] = __fmul_rn(yf, m.invW32[k]);
+        w.q[k] = hRT_of(a, T0);
         w.v[k] = ibct_f(z);
       }
       fin = __all_sync(full, fin);
@@ -534,7 +543,7 @@ __global__ void __launch_bounds__(32 * kUpdateWarps) update_warp_kernel(
             double acc = a2 < 0 ? e0 : 0.0;
             const double *C1 = sm.comp[a1], *C2 = sm.comp[a2 < 0 ? 0 : a2];
 #pragma unroll 2
-            for (int k = 0; k < K; ++k) acc = fma(C1[k] * w.y[k], a2 < 0 ? -1.0 : C2[k], acc);
+            for (int k = 0; k < K; ++k) acc = fma(__dmul_rn(C1[k], w.y[k]), a2 < 0 ? -1.0 : C2[k], acc);
             int at = 0;
 #pragma unroll
             for (int b1 = 0; b1 < EC; ++b1)
@@ -558,7 +567,7 @@ __global__ void __launch_bounds__(32 * kUpdateWarps) update_warp_kernel(
             w.y[k] = pd;
             w.v[k] = narrow_rn_pos(pd);
           }
-          w.yf[k] = w.v[k] * m.invW32[k];
+          w.yf[k] = __fmul_rn(w.v[k], m.invW32[k]);
         }
         __syncwarp();
         float Tn = T0;
@@ -566,10 +575,8 @@ __global__ void __launch_bounds__(32 * kUpdateWarps) update_warp_kernel(
           const int hi = Tn >= Tmidf ? 1 : 0;
           for (int k = lane; k < K; k += 32) {
             const float* a = m.th32 + ((size_t)k * 2 + hi) * 16;
-            const float cpR = a[0] + Tn * (a[1] + Tn * (a[2] + Tn * (a[3] + Tn * a[4])));
-            const float hRT = a[5] + Tn * (a[6] + Tn * (a[7] + Tn * (a[8] + Tn * a[9]))) + a[10] / Tn;
-            w.p[k] = w.yf[k] * hRT;
-            w.q[k] = cpR;
+            w.p[k] = __fmul_rn(w.yf[k], hRT_of(a, Tn));
+            w.q[k] = cpR_of(a, Tn);
           }
           __syncwarp();
           float s = 0.0f;   // lane 0: h, lane 1: c_p
