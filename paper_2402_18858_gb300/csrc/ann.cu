@@ -422,13 +422,17 @@ __global__ void update_kernel(DevMech m, int64_t n, int64_t ld, double* T, const
 }
 
 // The same update with one warp per cell, for calls with few cells.  A thread per cell is a chain of
-// several hundred FP64 operations (64 cycles each) and as many memory latencies, 174 us for any
-// number of cells up to 78,000; a warp spreads the species over its lanes and the sums over
-// species over its lanes too (every sum runs in species order in one lane: the same bits), at 19
-// thousand FP64 cycles per cell instead of 1.4.  Learned step of 1,536 53-species cells: 268 -> 157 us;
-// by these rates the two forms meet near 10,000 cells (kUpdateWarpCells).
+// several hundred FP64 operations (64 cycles each) and as many memory latencies (40 to 150 us for 9 to 53
+// species, whatever the call's size); a warp spreads the species over its lanes and the sums over
+// species over its lanes too (every sum runs in species order in one lane: the same bits), at many
+// times the thread form's FP64 cycles per cell.  Learned step of 1,536 53-species cells: 268 -> 157 us.
 constexpr int kUpdateWarps = 4;
-constexpr int64_t kUpdateWarpCells = 8192;
+// Up to how many cells per SM the warp form is taken: one round of resident warps (20, 16 with up to eight
+// elements: registers; the second round costs as much again), fewer for small mechanisms, whose thread
+// form is short.  Thread form -> warp form, us: 9 species 1,500 cells 39 -> 36, 2,000 40 -> 40, 3,000 39 ->
+// 44; 20 species 2,500 67 -> 64, 3,000 66 -> 64, 3,500 68 -> 83; 30 species 3,000 91 -> 74, 3,500 91 -> 106;
+// 53 species 3,000 150 -> 107, 3,500 150 -> 156.
+__host__ inline int update_warp_cells(int EC, int K) { return std::min(EC <= 4 ? 20 : 16, 4 + K); }
 
 template <int EC>
 struct UpdateSmem {
@@ -614,9 +618,12 @@ static int launch_update(const DevMech& m, int64_t n, int64_t ld, double* T, con
                          const float* U, int n_out_pad, const float* out_mean, const float* out_sd,
                          int32_t* flags, int32_t* status, float elem_tol, float Tmin, float Tmax, float dTmax,
                          const int32_t* idx, cudaStream_t s) {
+  int dev = 0, sms = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const unsigned grid = grid_for(n, 128), wgrid = (unsigned)((n + kUpdateWarps - 1) / kUpdateWarps);
 #define CHEM_UPDATE_CASE(EC)                                                                                  \
-  if (n <= kUpdateWarpCells)                                                                                \
+  if (n <= (int64_t)sms * update_warp_cells(EC, m.K))                                                       \
     update_warp_kernel<EC><<<wgrid, 32 * kUpdateWarps, 0, s>>>(m, n, ld, T, Y, U, n_out_pad, out_mean, out_sd, flags, \
                                                                status, elem_tol, Tmin, Tmax, dTmax, idx);    \
   else                                                                                                      \
