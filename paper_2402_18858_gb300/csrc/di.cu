@@ -18,7 +18,7 @@
 // result), shared-memory load 34, L1 hit 39, L2 hit 243-311.  With shared memory taking all but 28 KB
 // of L1 the mechanism tables come from L2, so they are laid out for contiguous warp loads, the
 // triangular solves issue the loads of four factor columns ahead of the FP64 chain, and 12 warps per SM
-// (3 per sub-partition) run in one block.  Same bits; 150 30-species cells (one warp per SM, tables in
+// (3 per sub-partition) are resident.  Same bits; 150 30-species cells (one warp per SM, tables in
 // L1): 22.3 -> 18.0 ms; 3,001 53-species cells: 145.7 -> 138 ms; 12,345 30-species cells: 137.7 ->
 // 134.8 ms (FP64 issue bound).
 #include <cuda_runtime.h>
@@ -1602,41 +1602,48 @@ int launch_di(const DevMech& m, int64_t n, int64_t ld, double dt, double* T, con
   if (n > (int64_t)0x7fffffff) return set_error(CHEM_E_ARG, "chem_step_di: too many cells in one call");
   const int sms = sm_count();
   auto go = [&](auto kern, int wpb, int per_sm, size_t smem, int64_t blocks, int64_t lo, int64_t hi) -> int {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)std::min<int64_t>(blocks, (int64_t)sms * per_sm));
-    cfg.blockDim = dim3(32 * wpb);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    // what shared memory the resident blocks leave goes to L1, for the mechanism tables
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
-    attr[0].val.sharedMemCarveout = (unsigned)std::min<size_t>(100, (per_sm * (smem + 1024) * 100 + 228 * 1024 - 1) / (228 * 1024));
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cuda_check(cudaLaunchKernelEx(&cfg, kern, m, n, ld, dt, T, p, Y, idx, o, status, stats, queue, wb, n_dev, lo, hi),
-                      "di_kernel launch");
+    // No shared-memory carve-out is asked for: the driver's own choice gives single calls the same times
+    // (53 species, 457 to 608 cells excepted: 36.5 -> 41 ms), and with one the SMs had to drain before a
+    // call on another stream got any (50 30-species cells beside 600: 24.0 -> 15.8 ms).
+    const unsigned grid = (unsigned)std::min<int64_t>(blocks, (int64_t)sms * per_sm);
+    kern<<<grid, 32 * wpb, smem, s>>>(m, n, ld, dt, T, p, Y, idx, o, status, stats, queue, wb, n_dev, lo, hi);
+    return cuda_check(cudaGetLastError(), "di_kernel launch");
   };
   auto launch = [&](auto kern, int64_t lo, int64_t hi) -> int {
-    // block shape (warps) that keeps the most warps resident per SM, the widest of equal ones (its
-    // warps are dealt evenly to the SM's four sub-partitions, each of which has its own FP64 unit)
+    // The block shape that keeps the most warps resident per SM (30 species: 12 warps fit in wide blocks
+    // only), but blocks of two warps where these hold as many, or all the cells of a call below one round:
+    // a block keeps its shared memory until its slowest cell ends, and what small blocks leave or return
+    // goes to calls on other streams.  Two calls at once, blocks of an SM's share of cells -> of two warps:
+    // 2 x 1,000 cells of 9 species 5.5 -> 4.4 ms, of 30 species 37.1 -> 32.2 ms, 2 x 4,000 of 9 species 13.1
+    // -> 12.6 ms; single calls within +-4 % (1,500 cells of 30 species 25.7 -> 26.7 ms, 1,800 of 9 species
+    // 3.94 -> 3.72 ms).
     const int optin = smem_optin();
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
     cudaFuncAttributes fa;
     if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) return cuda_check(cudaGetLastError(), "di_kernel attributes");
+    auto resident = [&](int warps) -> int {   // blocks of so many warps per SM
+      int blocks = 0;
+      if ((size_t)warps * wb <= (size_t)optin)
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kern, 32 * warps, (size_t)warps * wb);
+      return blocks;
+    };
     int wpb = 0, per_sm = 0;
     for (int cand = fa.maxThreadsPerBlock / 32; cand >= 1; --cand) {
-      if ((size_t)cand * wb > (size_t)optin) continue;
-      int blocks = 0;
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kern, 32 * cand, (size_t)cand * wb);
+      const int blocks = resident(cand);
       if (blocks * cand > wpb * per_sm) { wpb = cand; per_sm = blocks; }
     }
     if (wpb == 0) return set_error(CHEM_E_UNSUPPORTED, "mechanism needs more shared memory per warp than the device has");
-    // fewer cells than resident warps: one smaller block per SM
-    if (n < (int64_t)sms * wpb * per_sm) {
-      wpb = (int)std::min<int64_t>(wpb, std::max<int64_t>(1, (n + sms - 1) / sms));
-      per_sm = (int)std::max<int64_t>(1, (n + (int64_t)sms * wpb - 1) / ((int64_t)sms * wpb));
+    const int need = (int)std::min<int64_t>(wpb * per_sm, std::max<int64_t>(1, (n + sms - 1) / sms));
+    if (need == 1) {
+      wpb = per_sm = 1;
+    } else if (2 * resident(2) >= need) {
+      wpb = 2;
+      per_sm = (need + 1) / 2;
+    } else if (need < wpb * per_sm) {   // below one round, but more than blocks of two hold
+      wpb = std::min(wpb, need);
+      per_sm = (need + wpb - 1) / wpb;
     }
-    return go(kern, wpb, per_sm, (size_t)wpb * wb, (n + wpb - 1) / wpb, lo, hi);
+    return go(kern, wpb, per_sm, (size_t)wpb * wb, std::max<int64_t>((n + wpb - 1) / wpb, std::min<int64_t>(n, sms)), lo, hi);
   };
   // a team's blocks per SM (0: they do not fit), at most enough for n cells
   auto team_blocks = [&](auto kern, int tw) -> int {
