@@ -427,6 +427,14 @@ int chem_pasr_source(chem_mech mech, int64_t n, int64_t ld, double dt, const dou
                      const double* nu, double y_min, double r_min, double* omega, double* kappa,
                      chem_stream stream);
 
+/* Testing hook: chem_step_di with the number of warps per cell given (1, 2 or 4) instead of chosen by the
+ * mechanism and the number of cells.  CHEM_E_UNSUPPORTED where the mechanism has no such form (two warps
+ * below 33 unknowns; any team for a mechanism with three partners on a side of a reaction or with more
+ * production runs than fit). */
+int chem_selftest_di_form(chem_mech mech, int warps, int64_t n, int64_t ld, double dt, double* T, const double* p,
+                          double* Y, const int32_t* idx, const chem_di_opts* opts, int32_t* status,
+                          int32_t* stats, void* workspace, size_t ws_bytes, chem_stream stream);
+
 /* Testing hook: y[i] = exp(x[i]) by the library's own FP64 exponential (the table-driven
  * method the kernels use), for comparison with CUDA's exp.  Device pointers, n >= 0. */
 int chem_selftest_exp(chem_mech mech, int64_t n, const double* x, double* y, chem_stream stream);

@@ -58,6 +58,8 @@ def lib(auto_build: bool = False):
                                    vp, C.c_size_t, vp]
         L.chem_step_di_noalloc.argtypes = [vp, i64, i64, dbl, vp, vp, vp, vp, C.POINTER(DiOpts),
                                            vp, vp, vp]
+        L.chem_selftest_di_form.argtypes = [vp, i32, i64, i64, dbl, vp, vp, vp, vp, C.POINTER(DiOpts), vp, vp,
+                                            vp, C.c_size_t, vp]
         L.chem_workspace_bytes.argtypes = [vp, i64]
         L.chem_workspace_bytes.restype = C.c_size_t
         L.thermo_props.argtypes = [vp, i64, i64, vp, vp, vp, vp, vp, vp, vp, vp, i32, vp]
@@ -234,6 +236,17 @@ def chem_fp64_peak_gflops(stream=None) -> float:
     v = C.c_double()
     _check(lib().chem_fp64_peak_gflops(C.byref(v), _stream(stream)))
     return v.value
+
+
+def chem_selftest_di_form(m: Mech, warps: int, dt: float, T, p, Y, status, workspace, stats=None, rtol=0.0,
+                          atol_Y=0.0, stream=None) -> None:
+    """chem_step_di of every cell with the number of warps per cell given."""
+    n = _ld(Y, m)
+    o = DiOpts(rtol, atol_Y, 0.0, 0.0, 0, 0)
+    _check(lib().chem_selftest_di_form(m.handle, int(warps), n, n, float(dt), _ptr(T, torch.float64),
+                                       _ptr(p, torch.float64), _ptr(Y, torch.float64), None, C.byref(o),
+                                       _ptr(status, torch.int32), _ptr(stats, torch.int32), _ptr(workspace),
+                                       workspace.numel() * workspace.element_size(), _stream(stream)))
 
 
 def chem_selftest_exp(m: Mech, x, y, stream=None) -> None:

@@ -688,9 +688,9 @@ size_t chem_workspace_bytes(chem_mech m, int64_t n) {
   return 256;   // the cell work-queue counter, padded to one 256-byte line
 }
 
-int chem_step_di(chem_mech m, int64_t n, int64_t ld, double dt, double* T, const double* p,
-                 double* Y, const int32_t* idx, const chem_di_opts* opts, int32_t* status,
-                 int32_t* stats, void* workspace, size_t ws_bytes, chem_stream stream) {
+static int step_di(chem_mech m, int form, int64_t n, int64_t ld, double dt, double* T, const double* p, double* Y,
+                   const int32_t* idx, const chem_di_opts* opts, int32_t* status, int32_t* stats, void* workspace,
+                   size_t ws_bytes, chem_stream stream) {
   int rc = check_mech(m);
   if (rc) return rc;
   if (n < 0 || ld < n) return set_error(CHEM_E_ARG, "chem_step_di: need 0 <= n <= ld");
@@ -708,7 +708,20 @@ int chem_step_di(chem_mech m, int64_t n, int64_t ld, double dt, double* T, const
                        "chem_step_di: queue reset")))
     return rc;
   return launch_di(m->dev, n, ld, dt, T, p, Y, idx, o, status, stats, (unsigned int*)workspace,
-                   (cudaStream_t)stream);
+                   (cudaStream_t)stream, nullptr, form);
+}
+
+int chem_step_di(chem_mech m, int64_t n, int64_t ld, double dt, double* T, const double* p,
+                 double* Y, const int32_t* idx, const chem_di_opts* opts, int32_t* status,
+                 int32_t* stats, void* workspace, size_t ws_bytes, chem_stream stream) {
+  return step_di(m, 0, n, ld, dt, T, p, Y, idx, opts, status, stats, workspace, ws_bytes, stream);
+}
+
+int chem_selftest_di_form(chem_mech m, int warps, int64_t n, int64_t ld, double dt, double* T, const double* p,
+                          double* Y, const int32_t* idx, const chem_di_opts* opts, int32_t* status,
+                          int32_t* stats, void* workspace, size_t ws_bytes, chem_stream stream) {
+  if (warps != 1 && warps != 2 && warps != 4) return set_error(CHEM_E_ARG, "chem_selftest_di_form: warps must be 1, 2 or 4");
+  return step_di(m, warps, n, ld, dt, T, p, Y, idx, opts, status, stats, workspace, ws_bytes, stream);
 }
 
 int thermo_props(chem_mech m, int64_t n, int64_t ld, const double* T, const double* Y,

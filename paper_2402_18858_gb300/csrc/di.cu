@@ -1596,7 +1596,7 @@ int launch_jacobian(const DevMech& m, int64_t n, int64_t ld, const double* T, co
 
 int launch_di(const DevMech& m, int64_t n, int64_t ld, double dt, double* T, const double* p,
               double* Y, const int32_t* idx, const chem_di_opts& opts, int32_t* status,
-              int32_t* stats, unsigned int* queue, cudaStream_t s, const int32_t* n_dev) {
+              int32_t* stats, unsigned int* queue, cudaStream_t s, const int32_t* n_dev, int form) {
   const size_t wb = di_smem_per_warp(m);
   DiOpts o{opts.rtol, opts.atol_Y, opts.atol_T, opts.newton_tol, opts.max_steps, opts.jac_max_age};
   if (n > (int64_t)0x7fffffff) return set_error(CHEM_E_ARG, "chem_step_di: too many cells in one call");
@@ -1672,6 +1672,14 @@ int launch_di(const DevMech& m, int64_t n, int64_t ld, double dt, double* T, con
     if (!rc && n > few) rc = many(n_dev ? few : -1);
     return rc;
   };
+  if (form) {   // a test asks for so many warps per cell
+    const int per_sm = !teams ? 0 : m.n <= 32 ? (form == 4 ? team_blocks(di_kernel<1, 4>, 4) : 0)
+                       : form == 4 ? team_blocks(di_kernel<2, 4>, 4) : form == 2 ? team_blocks(di_kernel<2, 2>, 2) : 0;
+    if (form != 1 && per_sm == 0) return set_error(CHEM_E_UNSUPPORTED, "the mechanism has no such team form");
+    if (m.n <= 32) return form == 1 ? launch(di_kernel<1, 1>, -1, INT64_MAX) : go(di_kernel<1, 4>, 4, per_sm, wb + 64, n, -1, INT64_MAX);
+    if (form == 1) return launch(di_kernel<2, 1>, -1, INT64_MAX);
+    return form == 2 ? go(di_kernel<2, 2>, 2, per_sm, wb + 64, n, -1, INT64_MAX) : go(di_kernel<2, 4>, 4, per_sm, wb + 64, n, -1, INT64_MAX);
+  }
   if (m.n <= 32) return by_count(di_kernel<1, 4>, [&](int64_t lo) { return launch(di_kernel<1, 1>, lo, INT64_MAX); });
   return by_count(di_kernel<2, 4>, [&](int64_t lo) {
     const int per_sm = teams ? team_blocks(di_kernel<2, 2>, 2) : 0;

@@ -437,7 +437,8 @@ int launch_jacobian(const DevMech& m, int64_t n, int64_t ld, const double* T, co
                     const double* Y, double* jac, cudaStream_t s);
 int launch_di(const DevMech& m, int64_t n, int64_t ld, double dt, double* T, const double* p,
               double* Y, const int32_t* idx, const chem_di_opts& o, int32_t* status,
-              int32_t* stats, unsigned int* queue, cudaStream_t s, const int32_t* n_dev = nullptr);
+              int32_t* stats, unsigned int* queue, cudaStream_t s, const int32_t* n_dev = nullptr,
+              int form = 0);   // form: warps per cell, 0 by the rule of launch_di
 void di_fill_defaults(chem_di_opts& o);
 
 // mlp.cu: C = A B^T on the tensor cores with a fused epilogue
