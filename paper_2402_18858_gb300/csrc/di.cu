@@ -1609,34 +1609,39 @@ int launch_di(const DevMech& m, int64_t n, int64_t ld, double dt, double* T, con
     kern<<<grid, 32 * wpb, smem, s>>>(m, n, ld, dt, T, p, Y, idx, o, status, stats, queue, wb, n_dev, lo, hi);
     return cuda_check(cudaGetLastError(), "di_kernel launch");
   };
-  auto launch = [&](auto kern, int64_t lo, int64_t hi) -> int {
-    // The block shape that keeps the most warps resident per SM (30 species: 12 warps fit in wide blocks
-    // only), but blocks of two warps where these hold as many, or all the cells of a call below one round:
-    // a block keeps its shared memory until its slowest cell ends, and what small blocks leave or return
-    // goes to calls on other streams.  Two calls at once, blocks of an SM's share of cells -> of two warps:
-    // 2 x 1,000 cells of 9 species 5.5 -> 4.4 ms, of 30 species 37.1 -> 32.2 ms, 2 x 4,000 of 9 species 13.1
-    // -> 12.6 ms; single calls within +-4 % (1,500 cells of 30 species 25.7 -> 26.7 ms, 1,800 of 9 species
-    // 3.94 -> 3.72 ms).
-    const int optin = smem_optin();
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
+  auto resident = [&](auto kern, int warps, size_t smem) -> int {   // blocks of so many warps per SM
+    int blocks = 0;
+    if (smem <= (size_t)smem_optin()) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kern, 32 * warps, smem);
+    return blocks;
+  };
+  auto allow_smem = [&](auto kern) { cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin()); };
+  // one warp per cell: the block shape that keeps the most warps resident per SM
+  auto most_warps = [&](auto kern, int& wpb, int& per_sm) -> int {
+    allow_smem(kern);
     cudaFuncAttributes fa;
     if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) return cuda_check(cudaGetLastError(), "di_kernel attributes");
-    auto resident = [&](int warps) -> int {   // blocks of so many warps per SM
-      int blocks = 0;
-      if ((size_t)warps * wb <= (size_t)optin)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kern, 32 * warps, (size_t)warps * wb);
-      return blocks;
-    };
-    int wpb = 0, per_sm = 0;
+    wpb = per_sm = 0;
     for (int cand = fa.maxThreadsPerBlock / 32; cand >= 1; --cand) {
-      const int blocks = resident(cand);
+      const int blocks = resident(kern, cand, (size_t)cand * wb);
       if (blocks * cand > wpb * per_sm) { wpb = cand; per_sm = blocks; }
     }
-    if (wpb == 0) return set_error(CHEM_E_UNSUPPORTED, "mechanism needs more shared memory per warp than the device has");
+    return wpb ? CHEM_OK : set_error(CHEM_E_UNSUPPORTED, "mechanism needs more shared memory per warp than the device has");
+  };
+  auto launch = [&](auto kern, int64_t lo, int64_t hi) -> int {
+    // Up to 32 unknowns in blocks of two warps where these hold as many warps as the widest (30 species:
+    // twelve only in wide blocks), or all the cells of a call below one round: a block keeps its shared
+    // memory until its slowest cell ends, and what small blocks leave or return goes to calls on other
+    // streams.  Two calls at once, blocks of an SM's share of cells -> of two warps: 2 x 1,000 cells of 9
+    // species 5.5 -> 4.4 ms, of 30 species 37.1 -> 32.2 ms, 2 x 4,000 of 9 species 13.1 -> 12.6 ms; single
+    // calls within +-4 % (1,500 cells of 30 species 25.7 -> 26.7 ms, 1,800 of 9 species 3.94 -> 3.72 ms).
+    // Above 32 unknowns a warp takes 28 KB and more, and rounding up to pairs costs L1 (44 species, 700
+    // cells 34 -> 39 ms).
+    int wpb, per_sm;
+    if (const int rc = most_warps(kern, wpb, per_sm)) return rc;
     const int need = (int)std::min<int64_t>(wpb * per_sm, std::max<int64_t>(1, (n + sms - 1) / sms));
     if (need == 1) {
       wpb = per_sm = 1;
-    } else if (2 * resident(2) >= need) {
+    } else if (m.n <= 32 && 2 * resident(kern, 2, 2 * wb) >= need) {
       wpb = 2;
       per_sm = (need + 1) / 2;
     } else if (need < wpb * per_sm) {   // below one round, but more than blocks of two hold
@@ -1645,45 +1650,52 @@ int launch_di(const DevMech& m, int64_t n, int64_t ld, double dt, double* T, con
     }
     return go(kern, wpb, per_sm, (size_t)wpb * wb, std::max<int64_t>((n + wpb - 1) / wpb, std::min<int64_t>(n, sms)), lo, hi);
   };
-  // a team's blocks per SM (0: they do not fit), at most enough for n cells
-  auto team_blocks = [&](auto kern, int tw) -> int {
-    const size_t smem = wb + 64;
-    int blocks = 0;
-    if (smem > (size_t)smem_optin()) return 0;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin());
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kern, 32 * tw, smem);
-    return (int)std::min<int64_t>(blocks, (n + sms - 1) / sms);
-  };
   const bool teams = m.arity2 && m.bal_P > 0;
-  // Cells up to one round of teams of four (three per SM up to 32 unknowns, two above: registers) go by
-  // teams of four, more by `many`.  One warp per cell -> teams (5 us
-  // at rtol 1e-6), 30 species: 11 cells 5.43 -> 4.20 ms,
-  // 152 7.15 -> 5.65, 456 9.07 -> 7.25; in a second round teams lose (608 cells 7.53 -> 7.73, 912 9.10 ->
-  // 10.18 ms).  53 species: 11 cells 11.8 -> 9.9 ms, 304 13.2 -> 11.1; teams of two, which take the same
-  // shared memory per cell as one warp, beyond (456 cells 13.1 -> 12.5 ms, 912 20.0 -> 18.9, 1824 29.8 ->
-  // 28.5; 3001 cells over 10 us at the default tolerances 142 -> 136 ms): 45 KB per cell leave five
-  // warps per SM, and teams make them ten.  Up to 32 unknowns twelve warps are resident without.  (9
-  // species: one round of everything, no difference.)
-  auto by_count = [&](auto four, auto many) -> int {
-    const int per_sm = teams ? team_blocks(four, 4) : 0;
-    const int64_t few = (int64_t)sms * per_sm;
-    int rc = CHEM_OK;
-    if (per_sm > 0 && (n <= few || n_dev)) rc = go(four, 4, per_sm, wb + 64, n, -1, few);
-    if (!rc && n > few) rc = many(n_dev ? few : -1);
-    return rc;
+  auto team_blocks = [&](auto kern, int tw) -> int {   // a team's blocks per SM (0: no teams, or they do not fit)
+    if (!teams) return 0;
+    allow_smem(kern);
+    return resident(kern, tw, wb + 64);
+  };
+  auto go_team = [&](auto kern, int tw, int per_sm, int64_t lo, int64_t hi) -> int {
+    return go(kern, tw, (int)std::min<int64_t>(per_sm, (n + sms - 1) / sms), wb + 64, n, lo, hi);
   };
   if (form) {   // a test asks for so many warps per cell
-    const int per_sm = !teams ? 0 : m.n <= 32 ? (form == 4 ? team_blocks(di_kernel<1, 4>, 4) : 0)
-                       : form == 4 ? team_blocks(di_kernel<2, 4>, 4) : form == 2 ? team_blocks(di_kernel<2, 2>, 2) : 0;
-    if (form != 1 && per_sm == 0) return set_error(CHEM_E_UNSUPPORTED, "the mechanism has no such team form");
-    if (m.n <= 32) return form == 1 ? launch(di_kernel<1, 1>, -1, INT64_MAX) : go(di_kernel<1, 4>, 4, per_sm, wb + 64, n, -1, INT64_MAX);
-    if (form == 1) return launch(di_kernel<2, 1>, -1, INT64_MAX);
-    return form == 2 ? go(di_kernel<2, 2>, 2, per_sm, wb + 64, n, -1, INT64_MAX) : go(di_kernel<2, 4>, 4, per_sm, wb + 64, n, -1, INT64_MAX);
+    if (form == 1) return m.n <= 32 ? launch(di_kernel<1, 1>, -1, INT64_MAX) : launch(di_kernel<2, 1>, -1, INT64_MAX);
+    const int b = form == 4 ? (m.n <= 32 ? team_blocks(di_kernel<1, 4>, 4) : team_blocks(di_kernel<2, 4>, 4))
+                            : (m.n <= 32 ? 0 : team_blocks(di_kernel<2, 2>, 2));
+    if (b == 0) return set_error(CHEM_E_UNSUPPORTED, "the mechanism has no such team form");
+    if (form == 2) return go_team(di_kernel<2, 2>, 2, b, -1, INT64_MAX);
+    return m.n <= 32 ? go_team(di_kernel<1, 4>, 4, b, -1, INT64_MAX) : go_team(di_kernel<2, 4>, 4, b, -1, INT64_MAX);
   }
-  if (m.n <= 32) return by_count(di_kernel<1, 4>, [&](int64_t lo) { return launch(di_kernel<1, 1>, lo, INT64_MAX); });
-  return by_count(di_kernel<2, 4>, [&](int64_t lo) {
-    const int per_sm = teams ? team_blocks(di_kernel<2, 2>, 2) : 0;
-    return per_sm > 0 ? go(di_kernel<2, 2>, 2, per_sm, wb + 64, n, lo, INT64_MAX) : launch(di_kernel<2, 1>, lo, INT64_MAX);
+  // Teams of four for up to one round of them (three per SM up to 32 unknowns, two above: registers).  One
+  // warp per cell -> teams (5 us at rtol 1e-6), 30 species: 11 cells 5.43 -> 4.20 ms, 152 7.15 -> 5.65, 456
+  // 9.07 -> 7.25; in a second round teams lose (608 cells 7.53 -> 7.73, 912 9.10 -> 10.18 ms).  53
+  // species: 11 cells 11.8 -> 9.9 ms, 304 13.2 -> 11.1.  Mechanisms without the tables for it (9 species: more
+  // production runs than fit) have no teams.
+  // Above 32 unknowns then teams of two, which take the same shared memory per cell as one warp, but
+  // registers for six cells per SM at most where single warps go to eight.  Always where as many cells are
+  // resident (53 species: five of either, 45 KB each); up to three rounds where it is one less; up to what
+  // surely is one round where it is two less (32 to 40 species).  One warp -> teams of two, ms (5 us,
+  // default tolerances): 34 species 700 cells 32.1 -> 30.6, 1,200 38.4 -> 47.7, 5,000 131 -> 150; 38 species 700
+  // 61.8 -> 58.3, 1,200 67 -> 73, 2,400 114 -> 116, 5,000 202 -> 216; 44 species 700 45 -> 36, 1,200 51 -> 45, 2,400
+  // 73 -> 69, 5,000 126 -> 128; 53 species 1,200 69 -> 66, 2,400 107 -> 102, 5,000 200 -> 192.
+  // (With n_dev each form is launched for its range of counts, and those whose range the count is not in
+  // find no cells.)
+  auto four_then = [&](auto four, auto rest) -> int {
+    const int b = team_blocks(four, 4);
+    const int64_t few = (int64_t)sms * b;
+    int rc = CHEM_OK;
+    if (b > 0 && (n <= few || n_dev)) rc = go_team(four, 4, b, -1, few);
+    return rc || n <= few ? rc : rest(n_dev ? few : -1);
+  };
+  if (m.n <= 32) return four_then(di_kernel<1, 4>, [&](int64_t lo) { return launch(di_kernel<1, 1>, lo, INT64_MAX); });
+  return four_then(di_kernel<2, 4>, [&](int64_t lo) -> int {
+    const int b = team_blocks(di_kernel<2, 2>, 2);
+    const int single = (int)std::min<size_t>(8, (size_t)smem_optin() / wb);   // di_kernel<2, 1> has at most 8 warps
+    const int64_t mid = b == 0 ? -1 : b >= single ? INT64_MAX : (int64_t)sms * (b + 1 == single ? 3 * b : b - 1);
+    int rc = CHEM_OK;
+    if (mid > lo && (n <= mid || n_dev)) rc = go_team(di_kernel<2, 2>, 2, b, lo, mid);
+    return rc || n <= mid ? rc : launch(di_kernel<2, 1>, n_dev ? std::max(lo, mid) : -1, INT64_MAX);
   });
 }
 

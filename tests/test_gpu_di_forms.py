@@ -60,6 +60,35 @@ def test_forms_agree(kind, forms, n, tmp_path, monkeypatch):
         assert torch.equal(a, b)
 
 
+@pytest.mark.parametrize("n", [1, 400, 900, 2000])
+def test_fallback(n, tmp_path, monkeypatch):
+    """The learned step's fallback, whose count only the device knows, in a mechanism where each range of
+    counts has its own form: n of 2,000 cells are too hot for the learned step."""
+    m = _mechanism("c_36", monkeypatch)
+    lc, gm, _ = _load(m, tmp_path)
+    N = 2000
+    st = w.make_states(m, N, 31)
+    ann = lc.chem_ann_create(gm, [16], seed=1)
+    T, p, Y = (torch.as_tensor(np.ascontiguousarray(a), device="cuda") for a in (st.T, st.p, st.Y))
+    Yd = Y.clone()
+    status, sd = (torch.full((N,), -1, dtype=torch.int32, device="cuda") for _ in range(2))
+    ws = torch.empty(lc.chem_ann_workspace_bytes(ann, N), dtype=torch.uint8, device="cuda")
+    ref = torch.empty(lc.chem_workspace_bytes(gm, N), dtype=torch.uint8, device="cuda")
+    norm = lc.chem_ann_get_norm(ann)
+    norm[4 * ann.n_in + m.n_species:] = 1e-12     # no change predicted: cells are accepted by their temperature
+    lc.chem_ann_set_norm(ann, norm)
+    flagged = torch.arange(N, device="cuda") < n
+    T = torch.where(flagged, T + 1000.0, torch.full_like(T, 1000.0))
+    Td = T.clone()
+    lc.chem_step_ann(gm, ann, 1e-9, T, p, Y, status, ws, T_max=1100.0, elem_tol=1e9, di_rtol=1e-6,
+                     di_atol_Y=1e-12)
+    lc.chem_selftest_di_form(gm, 1, 1e-9, Td, p, Yd, sd, ref, rtol=1e-6, atol_Y=1e-12)
+    assert torch.equal(status != 0, flagged)
+    assert torch.equal(status[flagged] == 5, sd[flagged] == 0)
+    assert torch.equal(T.view(torch.int64)[flagged], Td.view(torch.int64)[flagged])
+    assert torch.equal(Y[:, flagged].contiguous().view(torch.int64), Yd[:, flagged].contiguous().view(torch.int64))
+
+
 @pytest.mark.parametrize("kind", ["h2_9", "c_30", "c_36"])
 def test_without_teams(kind, tmp_path, monkeypatch):
     from oracle import Oracle
