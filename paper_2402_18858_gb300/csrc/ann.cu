@@ -469,13 +469,14 @@ __global__ void __launch_bounds__(32 * kUpdateWarps) update_warp_kernel(
     if (flag == 0) {
       const float T0 = (float)T[i];
       const int hi0 = T0 >= Tmidf ? 1 : 0;
-      bool fin = true;
+      bool fin = true, odd = false;   // odd: a fraction that is not finite
       for (int k = lane; k < K; k += 32) {
         const double y = Y[(size_t)k * ld + i];
         const float yf = narrow_f32(y);
         const float* a = m.th32 + ((size_t)k * 2 + hi0) * 16;
         const float z = predict_z(y, U[(size_t)slot * n_out_pad + k], out_sd[k], out_mean[k]);
         fin = fin && isfinite(z);
+        odd = odd || !isfinite(yf);
         w.y[k] = y;
         w.yf[k] = yf;
         w.p[k] = __fmul_rn(yf, m.invW32[k]);
@@ -483,6 +484,7 @@ __global__ void __launch_bounds__(32 * kUpdateWarps) update_warp_kernel(
         w.v[k] = ibct_f(z);
       }
       fin = __all_sync(full, fin);
+      odd = __any_sync(full, odd);
       __syncwarp();
       // sums in species order: lane 0 the old enthalpy, lane 1 the predictions, lanes 2 .. the old
       // element moles; then in FP64 lanes 0 .. the old element moles
@@ -490,12 +492,13 @@ __global__ void __launch_bounds__(32 * kUpdateWarps) update_warp_kernel(
       {
         const float* P = lane == 0 ? w.p : lane == 1 ? w.v : w.yf;
         const float* Q = lane == 0 ? w.q : lane == 1 ? sm.one : sm.comp32[max(0, min(lane - 2, EC - 1))];
-        // element sums leave out the species without the element: an infinite fraction there must not
-        // meet the zero coefficient
-        const bool all = lane < 2;
+        if (!odd) {
 #pragma unroll 4
-        for (int k = 0; k < K; ++k)
-          if (all || Q[k] != 0.0f) s32 = fmaf(P[k], Q[k], s32);
+          for (int k = 0; k < K; ++k) s32 = fmaf(P[k], Q[k], s32);
+        } else {   // an infinite fraction must not meet the zero coefficient of an element it lacks
+          for (int k = 0; k < K; ++k)
+            if (lane < 2 || Q[k] != 0.0f) s32 = fmaf(P[k], Q[k], s32);
+        }
       }
       double eod = 0.0;
       {
