@@ -457,6 +457,9 @@ struct GemmEpi {
   int a_row, a_col, b_row, b_col;
   int64_t out_goff, z_goff;
   int bias_goff;
+  // every row of out, zout and z and every bias block starts on 16 bytes (set by gemm_bf16): whole chunks
+  // of columns may move 16 bytes at a time
+  bool vec;
 };
 // Weight gradients of up to kWgradMax layers over the same R rows: out_g [M, N] = A_g^T B_g, FP32, with
 // A [R, *] and B [R, *] BF16 row-major (row strides lda and ldb), group g's columns from g a_col and

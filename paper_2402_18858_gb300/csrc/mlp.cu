@@ -229,12 +229,10 @@ __device__ __forceinline__ void epi_chunk(float (&v)[32], int row, int col0, int
     // Whole groups of 8 columns go through the staging buffer, 16 bytes at a time (a last chunk of 8, 16 or
     // 24 columns, as in layers 400, 504, 1000 or 2000 wide, once took 2-byte stores of a lane per row: forward
     // of 30,001 cells through 64-2000-1000-504-53 232 -> 213 us, training step of 16,384 rows through
-    // 64-1600-800-400-30 536 -> 525 us).  Other remainders, or rows that do not start on 16
-    // bytes, element by element.
-    if (nv == 32) return epi_staged<EPI, true>(v, col0, 4, e, wbuf, row0, nrows, lane);
-    if ((nv & 7) == 0 && (((uintptr_t)e.out | (uintptr_t)e.zout | (uintptr_t)e.z | (uintptr_t)e.bias |
-                           (2 * e.ldo) | (EPI == 2 ? 2 * e.ldz : 0)) & 15) == 0)
-      return epi_staged<EPI, false>(v, col0, nv >> 3, e, wbuf, row0, nrows, lane);
+    // 64-1600-800-400-30 536 -> 525 us).  Other remainders, and rows that do not start on 16 bytes, element
+    // by element.
+    if (e.vec && nv == 32) return epi_staged<EPI, true>(v, col0, 4, e, wbuf, row0, nrows, lane);
+    if (e.vec && (nv & 7) == 0) return epi_staged<EPI, false>(v, col0, nv >> 3, e, wbuf, row0, nrows, lane);
   }
   if (row - row0 >= nrows) return;
   // every loop below is unrolled over the 32 columns with the ragged bound as a predicate: an
@@ -249,31 +247,17 @@ __device__ __forceinline__ void epi_chunk(float (&v)[32], int row, int col0, int
     // hidden layer forward: out = bf16(GELU(acc + b)); optional pre-activation copy
     bf16* o = (bf16*)e.out + (size_t)row * e.ldo + col0;
     bf16* zo = e.zout ? e.zout + (size_t)row * e.ldo + col0 : nullptr;
-    if (nv == 32) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        __align__(16) bf16 t[8], u[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          t[i] = __float2bfloat16_rn(gelu_f(v[8 * q + i]));
-          u[i] = __float2bfloat16_rn(v[8 * q + i]);
-        }
-        *(uint4*)(o + 8 * q) = *(const uint4*)t;
-        if (zo) *(uint4*)(zo + 8 * q) = *(const uint4*)u;
-      }
-    } else {
-#pragma unroll
-      for (int i = 0; i < 32; ++i) {
-        if (i < nv) {
-          o[i] = __float2bfloat16_rn(gelu_f(v[i]));
-          if (zo) zo[i] = __float2bfloat16_rn(v[i]);
-        }
+    for (int i = 0; i < 32; ++i) {
+      if (i < nv) {
+        o[i] = __float2bfloat16_rn(gelu_f(v[i]));
+        if (zo) zo[i] = __float2bfloat16_rn(v[i]);
       }
     }
   } else if (EPI == 1 || EPI == 3) {
     // output layer (acc + b) or weight gradient (acc), FP32
     float* o = (float*)e.out + (size_t)row * e.ldo + col0;
-    if (nv == 32) {
+    if (e.vec && nv == 32) {
 #pragma unroll
       for (int q = 0; q < 8; ++q) *(float4*)(o + 4 * q) = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
     } else {
@@ -842,6 +826,7 @@ __global__ void __launch_bounds__(256, 1) wgrad_kernel(const __grid_constant__ W
       GemmEpi e{};
       e.out = p.out[l] + (int64_t)gr * M * N;
       e.ldo = N;
+      e.vec = true;   // checked by wgrad_bf16
 #pragma unroll 1
       for (int c0 = (warp >> 2) * 32; c0 < kWgradBN; c0 += 64) {
         if (n0 + c0 >= N) break;
@@ -1013,8 +998,13 @@ static int launch_gemm_t(const bf16* A, int64_t lda, const bf16* B, int64_t ldb,
 // 1: bias -> FP32, 2: * GELU'(z) -> BF16, 3: FP32).  BN (a multiple of 32, at most 256) is
 // chosen from N.
 int gemm_bf16(int epi, const bf16* A, int64_t lda, const bf16* B, int64_t ldb, int M, int N, int K,
-              const GemmEpi& e, int* err, cudaStream_t s) {
+              const GemmEpi& e_in, int* err, cudaStream_t s) {
   if (M <= 0 || N <= 0 || K <= 0) return CHEM_OK;
+  GemmEpi e = e_in;
+  const int per16 = (epi == 0 || epi == 2) ? 8 : 4;   // result elements in 16 bytes
+  e.vec = (((uintptr_t)e.out | (uintptr_t)e.zout | (uintptr_t)e.bias) & 15) == 0 && e.ldo % per16 == 0 &&
+          (epi != 2 || (((uintptr_t)e.z & 15) == 0 && e.ldz % 8 == 0)) &&
+          (e.groups <= 1 || (e.out_goff % per16 == 0 && e.z_goff % 8 == 0 && e.bias_goff % 4 == 0));
   if (e.groups > 1) {
     // TMA column coordinates on 16-byte boundaries; 16-byte vector stores and z loads of
     // full 32-column chunks at every group's offset
@@ -1045,8 +1035,7 @@ int gemm_bf16(int epi, const bf16* A, int64_t lda, const bf16* B, int64_t ldb, i
     }
   }
   // the first layer's forward without a pre-activation copy: the short-K kernel's lean GELU epilogue
-  const bool gelu_x8 = epi == 0 && !e.zout && e.groups <= 1 && K <= 2 * tc::BK && N % 8 == 0 && e.ldo % 8 == 0 &&
-                       (((uintptr_t)e.out | (uintptr_t)e.bias) & 15) == 0;
+  const bool gelu_x8 = epi == 0 && !e.zout && e.groups <= 1 && K <= 2 * tc::BK && N % 8 == 0 && e.vec;
 #define CHEM_GEMM_CASE(BNV)                                                                    \
   if (bn == BNV) {                                                                             \
     switch (epi) {                                                                             \
@@ -1076,6 +1065,7 @@ int wgrad_bf16(const WgradLayer* layers, int n, int R, int* err, cudaStream_t s)
   for (int l = 0; l < n; ++l) {
     const WgradLayer& w = layers[l];
     if ((w.a_col & 7) || (w.b_col & 7)) return set_error(CHEM_E_ARG, "wgrad: group column offsets must be multiples of 8");
+    if ((w.N & 3) || ((uintptr_t)w.out & 15)) return set_error(CHEM_E_ARG, "wgrad: rows of the result must start on 16 bytes");
     // the maps span every group's columns; a tile that runs past a group's units reads the next
     // group's and does not store them
     if ((rc = make_map(&p.ta[l], w.A, R, (int64_t)(w.groups - 1) * w.a_col + w.M, w.lda, 64))) return rc;
