@@ -112,8 +112,8 @@ typedef struct {
  *   stats    NULL, or int32 stats[4 * n]: steps, RHS evaluations, Jacobian evaluations and
  *            LU factorisations per cell (stats[k * n + i]), for work accounting.
  *   workspace device scratch of at least chem_workspace_bytes(mech, n) bytes (the cell work
- *            queue); it must not be used by another call in flight.
- * Returns CHEM_E_WORKSPACE if the workspace is missing or too small. */
+ *            queue), 4-byte aligned; it must not be used by another call in flight.
+ * Returns CHEM_E_WORKSPACE if the workspace is missing, too small or misaligned. */
 int chem_step_di(chem_mech mech, int64_t n, int64_t ld, double dt, double* T, const double* p,
                  double* Y, const int32_t* idx, const chem_di_opts* opts, int32_t* status,
                  int32_t* stats, void* workspace, size_t ws_bytes, chem_stream stream);
@@ -181,7 +181,7 @@ int chem_ann_get_norm(chem_ann ann, float* host_norm);
  * training states (T, p, Y0) and their DI results Y1 (device, SoA, ld-strided). */
 int chem_ann_fit_norm(chem_ann ann, int64_t n, int64_t ld, const double* T, const double* p,
                       const double* Y0, const double* Y1, chem_stream stream);
-/* Normalised BF16 features X [n, 64]; if bcty is not NULL also the raw F(Y) as FP32 [n, K]
+/* Normalised BF16 features X [n, 64] (16-byte aligned, else CHEM_E_ARG); if bcty is not NULL also the raw F(Y) as FP32 [n, K]
  * (needed by the mass term of the loss).  If flags is not NULL, flags[i] receives the range
  * flag of the learned step (1 when a raw feature of cell i lies outside [min - m (max - min),
  * max + m (max - min)] of the training set, m = range_margin >= 0; else 0): the first stage
@@ -276,7 +276,7 @@ typedef struct {
  * on the tensor cores, the new state (inverse Box-Cox, renormalisation, T from enthalpy
  * conservation by Newton's method) and its checks; flagged cells are integrated by DI
  * (status CHEM_CELL_ANN_FALLBACK when DI succeeded, else DI's code).  Workspace:
- * chem_ann_workspace_bytes(ann, n). */
+ * chem_ann_workspace_bytes(ann, n), 16-byte aligned. */
 int chem_step_ann(chem_mech mech, chem_ann ann, int64_t n, int64_t ld, double dt, double* T,
                   const double* p, double* Y, const int32_t* idx, const chem_ann_opts* opts,
                   int32_t* status, void* workspace, size_t ws_bytes, chem_stream stream);

@@ -1292,6 +1292,7 @@ int chem_ann_features(chem_ann a, int64_t n, int64_t ld, const double* T, const 
   if (rc) return rc;
   if (n < 0 || ld < n || (n > 0 && (!T || !p || !Y || !X))) return set_error(CHEM_E_ARG, "chem_ann_features: bad arguments");
   if (flags && !(range_margin >= 0.0)) return set_error(CHEM_E_ARG, "chem_ann_features: range_margin must be >= 0");
+  if ((uintptr_t)X & 15) return set_error(CHEM_E_ARG, "chem_ann_features: X must be 16-byte aligned");
   if (n == 0) return CHEM_OK;
   features_kernel<<<grid_for(n, kFeatCells), 256, 0, (cudaStream_t)stream>>>(n, ld, T, p, Y, a->n_in, a->norm,
                                                                      (float)range_margin, (bf16*)X, flags, bcty,
@@ -1411,6 +1412,7 @@ int chem_ann_forward(chem_ann a, const void* X, int64_t n, float* U, void* works
   if (n == 0) return CHEM_OK;
   if (!workspace || ws_bytes < chem_ann_workspace_bytes(a, n))
     return set_error(CHEM_E_WORKSPACE, "chem_ann_forward: workspace smaller than chem_ann_workspace_bytes()");
+  if ((uintptr_t)workspace & 15) return set_error(CHEM_E_WORKSPACE, "chem_ann_forward: workspace must be 16-byte aligned");
   const int64_t mc = std::min<int64_t>(n, infer_chunk(a));
   char* w = (char*)workspace;
   bf16* act[kMaxLayers];
@@ -1447,6 +1449,7 @@ int chem_step_ann(chem_mech mech, chem_ann a, int64_t n, int64_t ld, double dt, 
   if (n > (int64_t)0x7fffffff) return set_error(CHEM_E_ARG, "chem_step_ann: too many cells");
   if (!workspace || ws_bytes < chem_ann_workspace_bytes(a, n))
     return set_error(CHEM_E_WORKSPACE, "chem_step_ann: workspace smaller than chem_ann_workspace_bytes()");
+  if ((uintptr_t)workspace & 15) return set_error(CHEM_E_WORKSPACE, "chem_step_ann: workspace must be 16-byte aligned");
   chem_ann_opts o{};
   if (opts) o = *opts;
   ann_fill_defaults(o);

@@ -699,6 +699,7 @@ static int step_di(chem_mech m, int form, int64_t n, int64_t ld, double dt, doub
   if (!T || !p || !Y || !status) return set_error(CHEM_E_ARG, "chem_step_di: null array");
   if (!workspace || ws_bytes < chem_workspace_bytes(m, n))
     return set_error(CHEM_E_WORKSPACE, "chem_step_di: workspace missing or smaller than chem_workspace_bytes()");
+  if ((uintptr_t)workspace & 3) return set_error(CHEM_E_WORKSPACE, "chem_step_di: workspace must be 4-byte aligned");
   chem_di_opts o{};
   if (opts) o = *opts;
   di_fill_defaults(o);
