@@ -27,7 +27,8 @@ struct ThermoSmem {
   float* invW;   // [K]
 };
 
-__host__ __device__ inline size_t thermo_smem_bytes(int K) {
+__host__ __device__ inline size_t thermo_smem_bytes(int K, bool transport) {
+  if (!transport) return (size_t)12 * K * sizeof(double);
   return (size_t)12 * K * sizeof(double) + (size_t)8 * K * sizeof(float) + (size_t)K * K * sizeof(float4) +
          (size_t)K * sizeof(float) + 16;
 }
@@ -46,8 +47,10 @@ __device__ __forceinline__ void mix_coeffs(const double* __restrict__ cr, int K,
   }
 }
 __device__ __forceinline__ void cp_h_of(const double (&A)[6], double T, double& cp, double& h) {
-  cp = kR * (A[0] + T * (A[1] + T * (A[2] + T * (A[3] + T * A[4]))));
-  h = kR * (T * (A[0] + T * (A[1] * 0.5 + T * (A[2] * (1.0 / 3.0) + T * (A[3] * 0.25 + T * A[4] * 0.2)))) + A[5]);
+  // T A4, common to both, is rounded by itself, so that c_p has the same bits whether or not h is wanted
+  const double t4 = __dmul_rn(T, A[4]);
+  cp = kR * (A[0] + T * (A[1] + T * (A[2] + T * __dadd_rn(A[3], t4))));
+  h = kR * (T * (A[0] + T * (A[1] * 0.5 + T * (A[2] * (1.0 / 3.0) + T * fma(A[3], 0.25, __dmul_rn(t4, 0.2))))) + A[5]);
 }
 
 // T from h(T) = ht by Newton's method.  The mixture coefficients belong to a temperature range, not
@@ -82,27 +85,32 @@ __device__ __forceinline__ void solve_T(double& Tc, bool newton, double ht, doub
   }
 }
 
-// mixed precision: one thread per cell
-template <int KC>
+// One thread per cell: the mixed mode, and either mode without transport outputs (TR = false), where c_p and
+// h are the same FP64 sums in both and the kernel holds only them: bound by its loads, where
+// thermo64_kernel's registers and shared memory leave few warps to hide them (FP64 mode, 200,000 cells,
+// thermo64_kernel -> this one: c_p of 12 species 74 -> 44 us, 30 species 117 -> 64, 53 species 220 -> 111; T from
+// h of 30 species 249 -> 171).
+template <int KC, bool TR>
 __global__ void __launch_bounds__(128) thermo_kernel(DevMech m, int64_t n, int64_t ld, const double* T,
                                                      const double* Y, double* cp_out, double* h_out,
                                                      double* mu_out, double* kappa_out, const double* h_in,
                                                      double* T_out) {
   extern __shared__ double tsm[];
   const int K = KC ? KC : m.K;
-  const bool transport = mu_out || kappa_out;
   ThermoSmem S;
   S.c = tsm;
-  S.tr = (float*)(tsm + 12 * K);
-  // float4 table 16-byte aligned after the FP32 fits
-  S.w3 = (float4*)(((uintptr_t)(S.tr + 8 * K) + 15) & ~(uintptr_t)15);
-  S.invW = (float*)(S.w3 + K * K);
+  if constexpr (TR) {
+    S.tr = (float*)(tsm + 12 * K);
+    // float4 table 16-byte aligned after the FP32 fits
+    S.w3 = (float4*)(((uintptr_t)(S.tr + 8 * K) + 15) & ~(uintptr_t)15);
+    S.invW = (float*)(S.w3 + K * K);
+  }
   for (int i = threadIdx.x; i < 12 * K; i += blockDim.x) {
     const int rg = i / (6 * K), q = (i / K) % 6, k = i % K;
     const double* a = m.th + ((size_t)k * 2 + rg) * kThermoStride;
     S.c[i] = __ldg(a + (q < 5 ? q : 10)) * __ldg(m.invW + k);   // cp/R coefficients a1..a5, then a6
   }
-  if (transport) {
+  if constexpr (TR) {
     for (int i = threadIdx.x; i < 8 * K; i += blockDim.x) S.tr[i] = (float)__ldg(m.tr + (size_t)(i % K) * 8 + i / K);
     for (int i = threadIdx.x; i < K * K; i += blockDim.x) {
       const double A = __ldg(m.wA + i), B = __ldg(m.wB + i);
@@ -118,7 +126,7 @@ __global__ void __launch_bounds__(128) thermo_kernel(DevMech m, int64_t n, int64
 #pragma unroll
     for (int k = 0; k < (KC ? KC : K); ++k) {
       yv[k] = Y[(size_t)k * ld + i];
-      sYW = fma(yv[k], __ldg(m.invW + k), sYW);
+      if (TR) sYW = fma(yv[k], __ldg(m.invW + k), sYW);
     }
     double Tc = T[i], cp, h, A[6];
     solve_T<false>(Tc, h_in != nullptr, h_in ? h_in[i] : 0.0, m.Tmid,
@@ -126,7 +134,7 @@ __global__ void __launch_bounds__(128) thermo_kernel(DevMech m, int64_t n, int64
     if (h_in) T_out[i] = Tc;
     if (cp_out) cp_out[i] = cp;
     if (h_out) h_out[i] = h;
-    if (!transport) continue;
+    if constexpr (!TR) continue;
     // FP32 transport.  Wilke's denominator D_k = sum_j X_j A_kj (1 + s_k B_kj / s_j)^2 with
     // s = sqrt(mu) expands into three sums over j with per-cell vectors X_j, X_j / s_j and
     // X_j / s_j^2: D_k = sum A X + 2 s_k sum (A B) (X / s) + s_k^2 sum (A B^2)(X / s^2),
@@ -259,7 +267,6 @@ __global__ void __launch_bounds__(128, JC <= 16 ? 4 : 2) thermo64_kernel(DevMech
   using Cf = Thermo64Cfg<JC, SPLIT>;
   extern __shared__ __align__(16) uint8_t tsm8[];
   const int K = m.K, nt = blockDim.x, tid = threadIdx.x;
-  const bool transport = mu_out || kappa_out;
   double* fx = (double*)tsm8;                       // [2][KP][6] NASA-7 a1..a5, a6
   int2* ct = (int2*)(tsm8 + Cf::FX);                // [KP][SPLIT][JE]
   double* trs = (double*)(tsm8 + Cf::FX + Cf::CT);  // [KP][11]
@@ -323,114 +330,112 @@ __global__ void __launch_bounds__(128, JC <= 16 ? 4 : 2) thermo64_kernel(DevMech
     };
     solve_T<SPLIT == 2>(Tc, h_in != nullptr, h_in ? h_in[i] : 0.0, m.Tmid, coeffs, A, cp, h);
     double l1 = 0.0, l2 = 0.0, mu = 0.0;
-    if (transport) {
-      const double L = log_t_fix(Tc, m.flogtab);
+    const double L = log_t_fix(Tc, m.flogtab);
 #pragma unroll
-      for (int j = 0; j < JC; ++j) ps[j * nt + tid] = v[j];
-      int Ep = 0, Eq = 0, Er = 0, ex = 0;
-      // not unrolled: the three exponentials per species would not fit the instruction cache
+    for (int j = 0; j < JC; ++j) ps[j * nt + tid] = v[j];
+    int Ep = 0, Eq = 0, Er = 0, ex = 0;
+    // not unrolled: the three exponentials per species would not fit the instruction cache
 #pragma unroll 1
+    for (int j = 0; j < JC; ++j) {
+      const int k = half * JC + j;
+      const double* b = trs + 11 * k;
+      const double yw = ps[j * nt + tid];
+      const double xu = b[0] + L * (b[1] + L * (b[2] + L * b[3]));
+      const double xl = b[4] + L * (b[5] + L * (b[6] + L * b[7]));
+      const double u = b[10] * exp2_fix(fix_exp_arg(xu), m.fexptab);
+      const long long fl = fix_exp_arg(xl);
+      l1 = fma(yw, exp2_fix(fl, m.fexptab), l1);
+      l2 = fma(yw, exp2_fix(-fl, m.fexptab), l2);
+      const double p = yw * b[9], q = p * u;
+      us[j * nt + tid] = u;
+      ps[j * nt + tid] = p;
+      Ep = max(Ep, fix_exp(p));
+      Eq = max(Eq, fix_exp(q));
+      Er = max(Er, fix_exp(q * u));
+      ex = max(ex, max(fix_exp(xu), fix_exp(xl)));
+    }
+    plain = plain || ex > 1023 + 8;   // an exponential's argument beyond 512, or not finite
+    if (SPLIT == 2) {
+      Ep = max(Ep, __shfl_xor_sync(0xffffffffu, Ep, 16));
+      Eq = max(Eq, __shfl_xor_sync(0xffffffffu, Eq, 16));
+      Er = max(Er, __shfl_xor_sync(0xffffffffu, Er, 16));
+      l1 += __shfl_xor_sync(0xffffffffu, l1, 16);
+      l2 += __shfl_xor_sync(0xffffffffu, l2, 16);
+      plain = __shfl_xor_sync(0xffffffffu, (int)plain, 16) || plain;
+    }
+    plain = plain || min(Ep, min(Eq, Er)) < kFxExpLo || max(Ep, max(Eq, Er)) > kFxExpHi;
+    if (mu_out) {
+      if (SPLIT == 2) __syncwarp();
+      int2 p2[JC], q2[JC], r2[JC];
+#pragma unroll
       for (int j = 0; j < JC; ++j) {
-        const int k = half * JC + j;
-        const double* b = trs + 11 * k;
-        const double yw = ps[j * nt + tid];
-        const double xu = b[0] + L * (b[1] + L * (b[2] + L * b[3]));
-        const double xl = b[4] + L * (b[5] + L * (b[6] + L * b[7]));
-        const double u = b[10] * exp2_fix(fix_exp_arg(xu), m.fexptab);
-        const long long fl = fix_exp_arg(xl);
-        l1 = fma(yw, exp2_fix(fl, m.fexptab), l1);
-        l2 = fma(yw, exp2_fix(-fl, m.fexptab), l2);
-        const double p = yw * b[9], q = p * u;
-        us[j * nt + tid] = u;
-        ps[j * nt + tid] = p;
-        Ep = max(Ep, fix_exp(p));
-        Eq = max(Eq, fix_exp(q));
-        Er = max(Er, fix_exp(q * u));
-        ex = max(ex, max(fix_exp(xu), fix_exp(xl)));
+        const double p = ps[j * nt + tid], u = us[j * nt + tid], q = p * u;
+        p2[j] = fix_vec(p, Ep);
+        q2[j] = fix_vec(q, Eq);
+        r2[j] = fix_vec(q * u, Er);
       }
-      plain = plain || ex > 1023 + 8;   // an exponential's argument beyond 512, or not finite
-      if (SPLIT == 2) {
-        Ep = max(Ep, __shfl_xor_sync(0xffffffffu, Ep, 16));
-        Eq = max(Eq, __shfl_xor_sync(0xffffffffu, Eq, 16));
-        Er = max(Er, __shfl_xor_sync(0xffffffffu, Er, 16));
-        l1 += __shfl_xor_sync(0xffffffffu, l1, 16);
-        l2 += __shfl_xor_sync(0xffffffffu, l2, 16);
-        plain = __shfl_xor_sync(0xffffffffu, (int)plain, 16) || plain;
-      }
-      plain = plain || min(Ep, min(Eq, Er)) < kFxExpLo || max(Ep, max(Eq, Er)) > kFxExpHi;
-      if (mu_out) {
-        if (SPLIT == 2) __syncwarp();
-        int2 p2[JC], q2[JC], r2[JC];
-#pragma unroll
-        for (int j = 0; j < JC; ++j) {
-          const double p = ps[j * nt + tid], u = us[j * nt + tid], q = p * u;
-          p2[j] = fix_vec(p, Ep);
-          q2[j] = fix_vec(q, Eq);
-          r2[j] = fix_vec(q * u, Er);
-        }
-        const int x0 = -1024 - m.fxC_e;
+      const int x0 = -1024 - m.fxC_e;
 #pragma unroll 1
-        for (int k0 = 0; k0 < K; k0 += SPLIT) {
-          long long P[SPLIT], Q[SPLIT], R[SPLIT];
+      for (int k0 = 0; k0 < K; k0 += SPLIT) {
+        long long P[SPLIT], Q[SPLIT], R[SPLIT];
 #pragma unroll
-          for (int s = 0; s < SPLIT; ++s) {
-            // (SPLIT = 2, odd K: the second row may be the zero row K < KP)
-            const int4* c4 = (const int4*)(ct + ((size_t)(k0 + s) * SPLIT + half) * Cf::JE);
-            long long ph = 0, pl = 0, qh = 0, ql = 0, rh = 0, rl = 0;
+        for (int s = 0; s < SPLIT; ++s) {
+          // (SPLIT = 2, odd K: the second row may be the zero row K < KP)
+          const int4* c4 = (const int4*)(ct + ((size_t)(k0 + s) * SPLIT + half) * Cf::JE);
+          long long ph = 0, pl = 0, qh = 0, ql = 0, rh = 0, rl = 0;
 #pragma unroll
-            for (int j = 0; j < JC; j += 2) {
-              const int4 c = c4[j / 2];
-              mad_wide(ph, c.x, p2[j].x);
-              mad_wide(pl, c.x, p2[j].y);
-              mad_wide(pl, c.y, p2[j].x);
-              mad_wide(qh, c.x, q2[j].x);
-              mad_wide(ql, c.x, q2[j].y);
-              mad_wide(ql, c.y, q2[j].x);
-              mad_wide(rh, c.x, r2[j].x);
-              mad_wide(rl, c.x, r2[j].y);
-              mad_wide(rl, c.y, r2[j].x);
-              if (j + 1 < JC) {
-                mad_wide(ph, c.z, p2[j + 1].x);
-                mad_wide(pl, c.z, p2[j + 1].y);
-                mad_wide(pl, c.w, p2[j + 1].x);
-                mad_wide(qh, c.z, q2[j + 1].x);
-                mad_wide(ql, c.z, q2[j + 1].y);
-                mad_wide(ql, c.w, q2[j + 1].x);
-                mad_wide(rh, c.z, r2[j + 1].x);
-                mad_wide(rl, c.z, r2[j + 1].y);
-                mad_wide(rl, c.w, r2[j + 1].x);
-              }
+          for (int j = 0; j < JC; j += 2) {
+            const int4 c = c4[j / 2];
+            mad_wide(ph, c.x, p2[j].x);
+            mad_wide(pl, c.x, p2[j].y);
+            mad_wide(pl, c.y, p2[j].x);
+            mad_wide(qh, c.x, q2[j].x);
+            mad_wide(ql, c.x, q2[j].y);
+            mad_wide(ql, c.y, q2[j].x);
+            mad_wide(rh, c.x, r2[j].x);
+            mad_wide(rl, c.x, r2[j].y);
+            mad_wide(rl, c.y, r2[j].x);
+            if (j + 1 < JC) {
+              mad_wide(ph, c.z, p2[j + 1].x);
+              mad_wide(pl, c.z, p2[j + 1].y);
+              mad_wide(pl, c.w, p2[j + 1].x);
+              mad_wide(qh, c.z, q2[j + 1].x);
+              mad_wide(ql, c.z, q2[j + 1].y);
+              mad_wide(ql, c.w, q2[j + 1].x);
+              mad_wide(rh, c.z, r2[j + 1].x);
+              mad_wide(rl, c.z, r2[j + 1].y);
+              mad_wide(rl, c.w, r2[j + 1].x);
             }
-            P[s] = fix_fold(ph, pl);
-            Q[s] = fix_fold(qh, ql);
-            R[s] = fix_fold(rh, rl);
           }
-          long long Pk = P[0], Qk = Q[0], Rk = R[0];
-          int k = k0;
-          if (SPLIT == 2) {
-            // the first half's thread finishes row k0, the second's row k0 + 1
-            const int o = half;
-            Pk = P[o ? SPLIT - 1 : 0] + __shfl_xor_sync(0xffffffffu, P[o ? 0 : SPLIT - 1], 16);
-            Qk = Q[o ? SPLIT - 1 : 0] + __shfl_xor_sync(0xffffffffu, Q[o ? 0 : SPLIT - 1], 16);
-            Rk = R[o ? SPLIT - 1 : 0] + __shfl_xor_sync(0xffffffffu, R[o ? 0 : SPLIT - 1], 16);
-            k = k0 + half;
-          }
-          if (k < K) {
-            // u_k and p_k from the thread that owns species k
-            const int own = SPLIT == 1 ? tid : (tid & ~16) | (k >= JC ? 16 : 0);
-            const int at = (SPLIT == 1 ? k : (k >= JC ? k - JC : k)) * nt + own;
-            const double u = us[at];
-            const double S = fma(u, fma(u, fix_to_double(Pk, x0 + Ep), fix_to_double(Qk, x0 + Eq + 1)),
-                                 fix_to_double(Rk, x0 + Er));
-            mu = fma(ps[at], rcp_nr(S), mu);
-          }
+          P[s] = fix_fold(ph, pl);
+          Q[s] = fix_fold(qh, ql);
+          R[s] = fix_fold(rh, rl);
         }
+        long long Pk = P[0], Qk = Q[0], Rk = R[0];
+        int k = k0;
         if (SPLIT == 2) {
-          mu += __shfl_xor_sync(0xffffffffu, mu, 16);
-          __syncwarp();   // the next round overwrites us and ps
+          // the first half's thread finishes row k0, the second's row k0 + 1
+          const int o = half;
+          Pk = P[o ? SPLIT - 1 : 0] + __shfl_xor_sync(0xffffffffu, P[o ? 0 : SPLIT - 1], 16);
+          Qk = Q[o ? SPLIT - 1 : 0] + __shfl_xor_sync(0xffffffffu, Q[o ? 0 : SPLIT - 1], 16);
+          Rk = R[o ? SPLIT - 1 : 0] + __shfl_xor_sync(0xffffffffu, R[o ? 0 : SPLIT - 1], 16);
+          k = k0 + half;
         }
-        mu *= 2.8284271247461903;   // sqrt(8)
+        if (k < K) {
+          // u_k and p_k from the thread that owns species k
+          const int own = SPLIT == 1 ? tid : (tid & ~16) | (k >= JC ? 16 : 0);
+          const int at = (SPLIT == 1 ? k : (k >= JC ? k - JC : k)) * nt + own;
+          const double u = us[at];
+          const double S = fma(u, fma(u, fix_to_double(Pk, x0 + Ep), fix_to_double(Qk, x0 + Eq + 1)),
+                               fix_to_double(Rk, x0 + Er));
+          mu = fma(ps[at], rcp_nr(S), mu);
+        }
       }
+      if (SPLIT == 2) {
+        mu += __shfl_xor_sync(0xffffffffu, mu, 16);
+        __syncwarp();   // the next round overwrites us and ps
+      }
+      mu *= 2.8284271247461903;   // sqrt(8)
     }
     if (!have || half != 0) continue;
     if (plain) {
@@ -452,15 +457,15 @@ static int thermo_sms() {
   return sms;
 }
 
-template <int KC>
-static int launch_thermo_mixed(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* Y, double* cp,
-                               double* h, double* mu, double* kappa, const double* h_in, double* T_out, cudaStream_t s) {
-  const size_t smem = thermo_smem_bytes(m.K);
-  int rc = cuda_check(cudaFuncSetAttribute(thermo_kernel<KC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+template <int KC, bool TR>
+static int launch_thermo_cell(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* Y, double* cp,
+                              double* h, double* mu, double* kappa, const double* h_in, double* T_out, cudaStream_t s) {
+  const size_t smem = thermo_smem_bytes(m.K, TR);
+  int rc = cuda_check(cudaFuncSetAttribute(thermo_kernel<KC, TR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
                       "thermo smem attribute");
   if (rc) return rc;
   const int64_t blocks = std::min<int64_t>((n + 127) / 128, (int64_t)thermo_sms() * 8);
-  thermo_kernel<KC><<<(int)blocks, 128, smem, s>>>(m, n, ld, T, Y, cp, h, mu, kappa, h_in, T_out);
+  thermo_kernel<KC, TR><<<(int)blocks, 128, smem, s>>>(m, n, ld, T, Y, cp, h, mu, kappa, h_in, T_out);
   return cuda_check(cudaGetLastError(), "thermo_kernel launch");
 }
 
@@ -483,14 +488,19 @@ static int launch_thermo64(const DevMech& m, int64_t n, int64_t ld, const double
 int launch_thermo(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* Y,
                   double* cp, double* h, double* mu, double* kappa, const double* h_in,
                   double* T_out, int mixed, cudaStream_t s) {
-  if (mixed) {
-    // species counts of the shipped workloads get fully unrolled kernels; others run the
-    // generic loop
-    if (m.K == 9) return launch_thermo_mixed<9>(m, n, ld, T, Y, cp, h, mu, kappa, h_in, T_out, s);
-    if (m.K == 30) return launch_thermo_mixed<30>(m, n, ld, T, Y, cp, h, mu, kappa, h_in, T_out, s);
-    if (m.K == 53) return launch_thermo_mixed<53>(m, n, ld, T, Y, cp, h, mu, kappa, h_in, T_out, s);
-    return launch_thermo_mixed<0>(m, n, ld, T, Y, cp, h, mu, kappa, h_in, T_out, s);
+  // Without transport outputs both modes are the same FP64 sums, by a thread per cell.  Species counts
+  // of the shipped workloads get fully unrolled kernels; others run the generic loop
+  const bool transport = mu || kappa;
+#define CHEM_THERMO_CELL(KC)                                                                                   \
+  return transport ? launch_thermo_cell<KC, true>(m, n, ld, T, Y, cp, h, mu, kappa, h_in, T_out, s)            \
+                   : launch_thermo_cell<KC, false>(m, n, ld, T, Y, cp, h, mu, kappa, h_in, T_out, s)
+  if (mixed || !transport) {
+    if (m.K == 9) CHEM_THERMO_CELL(9);
+    if (m.K == 30) CHEM_THERMO_CELL(30);
+    if (m.K == 53) CHEM_THERMO_CELL(53);
+    CHEM_THERMO_CELL(0);
   }
+#undef CHEM_THERMO_CELL
   // the narrowest instantiation that holds the species (the rest of its slots are zeros)
 #define CHEM_THERMO64(JC, SPLIT) \
   if (m.K <= JC * SPLIT) return launch_thermo64<JC, SPLIT>(m, n, ld, T, Y, cp, h, mu, kappa, h_in, T_out, s);
