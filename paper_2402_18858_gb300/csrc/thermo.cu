@@ -90,7 +90,10 @@ __device__ __forceinline__ void solve_T(double& Tc, bool newton, double ht, doub
 // thermo64_kernel's registers and shared memory leave few warps to hide them (FP64 mode, 200,000 cells,
 // thermo64_kernel -> this one: c_p of 12 species 74 -> 44 us, 30 species 117 -> 64, 53 species 220 -> 111; T from
 // h of 30 species 249 -> 171).
-template <int KC, bool TR>
+// FROM_H: T from h first (decided at run time without an unrolled species loop, where the split lost 17 %);
+// unrolled, the solve in the same kernel cost calls without it 3 % (53 species, all outputs of 200,000 cells 375
+// -> 361 us).
+template <int KC, bool TR, bool FROM_H>
 __global__ void __launch_bounds__(128) thermo_kernel(DevMech m, int64_t n, int64_t ld, const double* T,
                                                      const double* Y, double* cp_out, double* h_out,
                                                      double* mu_out, double* kappa_out, const double* h_in,
@@ -129,9 +132,10 @@ __global__ void __launch_bounds__(128) thermo_kernel(DevMech m, int64_t n, int64
       if (TR) sYW = fma(yv[k], __ldg(m.invW + k), sYW);
     }
     double Tc = T[i], cp, h, A[6];
-    solve_T<false>(Tc, h_in != nullptr, h_in ? h_in[i] : 0.0, m.Tmid,
+    const bool newton = KC ? FROM_H : h_in != nullptr;
+    solve_T<false>(Tc, newton, newton ? h_in[i] : 0.0, m.Tmid,
                    [&](bool hi, double (&a)[6]) { mix_coeffs<KC>(S.c + (hi ? 6 * K : 0), K, yv, a); }, A, cp, h);
-    if (h_in) T_out[i] = Tc;
+    if (newton) T_out[i] = Tc;
     if (cp_out) cp_out[i] = cp;
     if (h_out) h_out[i] = h;
     if constexpr (!TR) continue;
@@ -457,15 +461,15 @@ static int thermo_sms() {
   return sms;
 }
 
-template <int KC, bool TR>
+template <int KC, bool TR, bool FROM_H>
 static int launch_thermo_cell(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* Y, double* cp,
                               double* h, double* mu, double* kappa, const double* h_in, double* T_out, cudaStream_t s) {
   const size_t smem = thermo_smem_bytes(m.K, TR);
-  int rc = cuda_check(cudaFuncSetAttribute(thermo_kernel<KC, TR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+  int rc = cuda_check(cudaFuncSetAttribute(thermo_kernel<KC, TR, FROM_H>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
                       "thermo smem attribute");
   if (rc) return rc;
   const int64_t blocks = std::min<int64_t>((n + 127) / 128, (int64_t)thermo_sms() * 8);
-  thermo_kernel<KC, TR><<<(int)blocks, 128, smem, s>>>(m, n, ld, T, Y, cp, h, mu, kappa, h_in, T_out);
+  thermo_kernel<KC, TR, FROM_H><<<(int)blocks, 128, smem, s>>>(m, n, ld, T, Y, cp, h, mu, kappa, h_in, T_out);
   return cuda_check(cudaGetLastError(), "thermo_kernel launch");
 }
 
@@ -491,9 +495,10 @@ int launch_thermo(const DevMech& m, int64_t n, int64_t ld, const double* T, cons
   // Without transport outputs both modes are the same FP64 sums, by a thread per cell.  Species counts
   // of the shipped workloads get fully unrolled kernels; others run the generic loop
   const bool transport = mu || kappa;
-#define CHEM_THERMO_CELL(KC)                                                                                   \
-  return transport ? launch_thermo_cell<KC, true>(m, n, ld, T, Y, cp, h, mu, kappa, h_in, T_out, s)            \
-                   : launch_thermo_cell<KC, false>(m, n, ld, T, Y, cp, h, mu, kappa, h_in, T_out, s)
+#define CHEM_THERMO_CELL(KC)                                                                                        \
+  return (transport ? h_in && KC ? launch_thermo_cell<KC, true, KC != 0> : launch_thermo_cell<KC, true, false>         \
+                    : h_in && KC ? launch_thermo_cell<KC, false, KC != 0> : launch_thermo_cell<KC, false, false>)(     \
+      m, n, ld, T, Y, cp, h, mu, kappa, h_in, T_out, s)
   if (mixed || !transport) {
     if (m.K == 9) CHEM_THERMO_CELL(9);
     if (m.K == 30) CHEM_THERMO_CELL(30);
