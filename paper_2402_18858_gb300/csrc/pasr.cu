@@ -28,11 +28,16 @@ namespace chem {
 // Y1 and Y0 arrive by asynchronous copies into a ring of kRing chunks of kChunk species per thread:
 // with plain loads the compiler placed each load before its use, one latency after the other (25 to
 // 39 thousand cycles per cell of a warp, 2.7 to 3.4 TB/s).  A thread copies and reads only its own
-// cells' slots, so no barrier is involved and any alignment of the rows (8 bytes) will do.  Two chunks
-// of 10 at four blocks per SM measured best (177 us against 180 to 208 us for 3 to 5 chunks of 3 to 10
-// species at three to five blocks).
+// cells' slots, so no barrier is involved and any alignment of the rows (8 bytes) will do.  The species'
+// differences stay in registers, so there is a kernel for each number of chunks (NB), and one more for a
+// last chunk that is whole (WHOLE: no guards; 30 species, 900,000 cells 164 -> 160 us).  900,000 cells,
+// thread-local arrays and plain loads -> ring: 12 species 109 -> 93 us, 20 species 154 -> 124, 36 species 244 ->
+// 185, 44 species 287 -> 226, 62 species 392 -> 362.
 constexpr int kChunk = 10, kRing = 2, kThreads = 128;
 constexpr int kSlots = 2 * kChunk + 4;   // the cell's rho, k, eps and nu come with its last chunk
+// blocks per SM by chunks, as the registers for the differences allow (six chunks: two blocks 305 us, three
+// 264 us at 900,000 cells of 53 species; four chunks: three blocks 185 us, four 189 us at 36 species)
+constexpr int kBlocks[8] = {0, 4, 4, 4, 3, 3, 3, 2};
 
 __device__ __forceinline__ void copy_async8(double* smem_dst, const double* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned int)__cvta_generic_to_shared(smem_dst)), "l"(src)
@@ -91,19 +96,18 @@ __device__ __forceinline__ void slowest_step(double y1, double dk, long long ymi
   b.dk = take ? dk : b.dk;
 }
 
-template <int KC>
-__global__ void __launch_bounds__(kThreads, KC <= 32 ? 4 : 2) pasr_kernel(int Kr, int64_t n, int64_t ld, double dt, double inv_dt,
+template <int NB, bool WHOLE>
+__global__ void __launch_bounds__(kThreads, kBlocks[NB]) pasr_kernel(int Kr, int64_t n, int64_t ld, double dt, double inv_dt,
                                                    const double* __restrict__ rho, const double* __restrict__ Y0,
                                                    const double* __restrict__ Y1, const double* __restrict__ ksgs,
                                                    const double* __restrict__ eps, const double* __restrict__ nu,
                                                    long long ymin_bits, double r_min, double* __restrict__ omega,
                                                    double* __restrict__ kappa) {
-  const int K = KC ? KC : Kr;
+  const int K = WHOLE ? NB * kChunk : Kr;
   const float r_minf = __double2float_rn(r_min);
   const float r_hi = r_minf * (1.0f + 0x1p-20f), r_lo = r_minf * (1.0f - 0x1p-20f);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  constexpr int NB = KC ? (KC + kChunk - 1) / kChunk : 1;   // chunks per cell
   extern __shared__ double ring[];                          // [kRing][kSlots][kThreads]
   double* mine = ring + threadIdx.x;
   int64_t fi = first;    // the cell and chunk fetched next
@@ -114,7 +118,7 @@ __global__ void __launch_bounds__(kThreads, KC <= 32 ? 4 : 2) pasr_kernel(int Kr
 #pragma unroll
       for (int u = 0; u < kChunk; ++u) {
         const int k = fc * kChunk + u;
-        if (k < KC) {
+        if (k < K) {
           copy_async8(dst + 2 * u * kThreads, Y1 + (size_t)k * ld + fi);
           copy_async8(dst + (2 * u + 1) * kThreads, Y0 + (size_t)k * ld + fi);
         }
@@ -134,48 +138,33 @@ __global__ void __launch_bounds__(kThreads, KC <= 32 ? 4 : 2) pasr_kernel(int Kr
       fi += stride;
     }
   };
-  if constexpr (KC > 0) {
 #pragma unroll
-    for (int q = 0; q < kRing - 1; ++q) fetch();
-  }
+  for (int q = 0; q < kRing - 1; ++q) fetch();
   for (int64_t i = first; i < n; i += stride) {
-    double d[KC ? KC : CHEM_MAX_SPECIES];
+    double d[NB * kChunk];
     Slowest b{0.0f, 1.0f, 0.0, 0.0};
     bool unsure = false;
     const double* last = nullptr;   // rho, k, eps, nu of the cell
-    if constexpr (KC > 0) {
 #pragma unroll
-      for (int c = 0; c < NB; ++c) {
-        fetch();
-        copy_wait<kRing - 1>();   // all but the kRing - 1 newest groups: this chunk is here
-        const double* src = mine + (size_t)slot * kSlots * kThreads;
-        slot = slot + 1 == kRing ? 0 : slot + 1;
+    for (int c = 0; c < NB; ++c) {
+      fetch();
+      copy_wait<kRing - 1>();   // all but the kRing - 1 newest groups: this chunk is here
+      const double* src = mine + (size_t)slot * kSlots * kThreads;
+      slot = slot + 1 == kRing ? 0 : slot + 1;
 #pragma unroll
-        for (int u = 0; u < kChunk; ++u)
-          if (c * kChunk + u < KC) {
-            const double y1 = src[2 * u * kThreads], dk = y1 - src[(2 * u + 1) * kThreads];
-            d[c * kChunk + u] = dk;
-            slowest_step(y1, dk, ymin_bits, r_hi, r_lo, b, unsure);
-          }
-        last = src + 2 * kChunk * kThreads;
-      }
-    } else {
-      for (int k = 0; k < K; ++k) {
-        const double y1 = Y1[(size_t)k * ld + i];
-        d[k] = y1 - Y0[(size_t)k * ld + i];
-        slowest_step(y1, d[k], ymin_bits, r_hi, r_lo, b, unsure);
-      }
+      for (int u = 0; u < kChunk; ++u)
+        if (c < NB - 1 || c * kChunk + u < K) {
+          const double y1 = src[2 * u * kThreads], dk = y1 - src[(2 * u + 1) * kThreads];
+          d[c * kChunk + u] = dk;
+          slowest_step(y1, dk, ymin_bits, r_hi, r_lo, b, unsure);
+        }
+      last = src + 2 * kChunk * kThreads;
     }
     if (unsure) b = slowest_exact(K, i, ld, Y0, Y1, ymin_bits, r_min);
     // dk > 0 for every candidate, 0 when there is none
     const double tau_c = __double_as_longlong(b.dk) > 0 ? dt * b.y1 * rcp_nr(b.dk) : 0.0;
     float tau_mix = 0.0f;
-    double kk, ee, nn, rr;
-    if constexpr (KC > 0) {
-      rr = last[0], kk = last[kThreads], ee = last[2 * kThreads], nn = last[3 * kThreads];
-    } else {
-      rr = rho[i], kk = ksgs[i], ee = eps[i], nn = nu[i];
-    }
+    const double rr = last[0], kk = last[kThreads], ee = last[2 * kThreads], nn = last[3 * kThreads];
     if (__double_as_longlong(kk) > 0 && __double_as_longlong(ee) > 0) {
       const float ie = __frcp_rn(__double2float_rn(ee));
       tau_mix = sqrtf(sqrtf(__double2float_rn(nn) * ie) * (__double2float_rn(kk) * ie));
@@ -185,7 +174,8 @@ __global__ void __launch_bounds__(kThreads, KC <= 32 ? 4 : 2) pasr_kernel(int Kr
     if (kappa) kappa[i] = kap;
     const double s = kap * rr * inv_dt;
 #pragma unroll
-    for (int k = 0; k < (KC ? KC : K); ++k) omega[(size_t)k * ld + i] = s * d[k];
+    for (int k = 0; k < NB * kChunk; ++k)
+      if (k < (NB - 1) * kChunk || k < K) omega[(size_t)k * ld + i] = s * d[k];
   }
 }
 
@@ -195,27 +185,30 @@ int launch_pasr(const DevMech& m, int64_t n, int64_t ld, double dt, const double
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int blocks = (int)std::min<int64_t>((n + kThreads - 1) / kThreads, (int64_t)sms * (m.K <= 32 ? 4 : 2));
   const size_t smem = (size_t)kRing * kSlots * kThreads * sizeof(double);   // 48 KB
   long long yb = 0;
   std::memcpy(&yb, &y_min, sizeof yb);
   const double inv_dt = 1.0 / dt;
-#define CHEM_PASR_K(KV)                                                                                 \
-  if (m.K == KV) {                                                                                      \
-    int rc = cuda_check(cudaFuncSetAttribute(pasr_kernel<KV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), \
-                        "pasr smem attribute");                                                          \
-    if (rc) return rc;                                                                                  \
-    pasr_kernel<KV><<<blocks, kThreads, smem, s>>>(m.K, n, ld, dt, inv_dt, rho, Y0, Y1, ksgs, eps, nu, yb, r_min, \
-                                           omega, kappa);                                                   \
-    return cuda_check(cudaGetLastError(), "pasr_kernel launch");                                        \
+  const int chunks = (m.K + kChunk - 1) / kChunk;
+#define CHEM_PASR_CHUNKS(NB)                                                                                 \
+  if (chunks == NB) {                                                                                        \
+    auto kern = m.K % kChunk ? pasr_kernel<NB, false> : pasr_kernel<NB, true>;                               \
+    int rc = cuda_check(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),  \
+                        "pasr smem attribute");                                                              \
+    if (rc) return rc;                                                                                       \
+    const int blocks = (int)std::min<int64_t>((n + kThreads - 1) / kThreads, (int64_t)sms * kBlocks[NB]);    \
+    kern<<<blocks, kThreads, smem, s>>>(m.K, n, ld, dt, inv_dt, rho, Y0, Y1, ksgs, eps, nu, yb, r_min, omega, kappa); \
+    return cuda_check(cudaGetLastError(), "pasr_kernel launch");                                             \
   }
-  CHEM_PASR_K(9)
-  CHEM_PASR_K(30)
-  CHEM_PASR_K(53)
-#undef CHEM_PASR_K
-  pasr_kernel<0><<<(int)std::min<int64_t>((n + kThreads - 1) / kThreads, (int64_t)sms * 16), kThreads, 0, s>>>(m.K, n, ld, dt, inv_dt, rho, Y0, Y1, ksgs, eps, nu, yb, r_min, omega,
-                                        kappa);
-  return cuda_check(cudaGetLastError(), "pasr_kernel launch");
+  CHEM_PASR_CHUNKS(1)
+  CHEM_PASR_CHUNKS(2)
+  CHEM_PASR_CHUNKS(3)
+  CHEM_PASR_CHUNKS(4)
+  CHEM_PASR_CHUNKS(5)
+  CHEM_PASR_CHUNKS(6)
+  CHEM_PASR_CHUNKS(7)
+#undef CHEM_PASR_CHUNKS
+  return set_error(CHEM_E_UNSUPPORTED, "chem_pasr_source: too many species");
 }
 
 }  // namespace chem
