@@ -105,7 +105,9 @@ __global__ void __launch_bounds__(kThreads, kBlocks[NB]) pasr_kernel(int Kr, int
                                                    double* __restrict__ kappa) {
   const int K = WHOLE ? NB * kChunk : Kr;
   const float r_minf = __double2float_rn(r_min);
-  const float r_hi = r_minf * (1.0f + 0x1p-20f), r_lo = r_minf * (1.0f - 0x1p-20f);
+  // With r_min = 0 every gain is above the threshold, r_hi y1 = 0, and any r_lo > 0 lets that settle it
+  // (0 did not: every cell went through slowest_exact, 30 species, 900,000 cells 328 us).
+  const float r_hi = r_minf * (1.0f + 0x1p-20f), r_lo = r_min == 0.0 ? 1.0f : r_minf * (1.0f - 0x1p-20f);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   extern __shared__ double ring[];                          // [kRing][kSlots][kThreads]
