@@ -13,6 +13,7 @@
 #include <mutex>
 
 #include "gemm_tc.cuh"
+#include "per_device.h"
 #include "internal.h"
 
 namespace chem {
@@ -883,6 +884,27 @@ static int make_map(CUtensorMap* map, const void* base, int64_t rows, int64_t co
   return CHEM_OK;
 }
 
+static int current_device() {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  return dev;
+}
+static int sm_count(int dev) {
+  int sms = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return std::max(sms, 1);
+}
+// allow a kernel its dynamic shared memory, once per device
+template <typename Kern>
+static int allow_smem(PerDevice& done, int dev, Kern kern, size_t bytes, const char* what) {
+  int rc = CHEM_OK;
+  done.get(dev, [&] {
+    rc = cuda_check(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes), what);
+    return rc ? 0 : 1;
+  });
+  return rc;
+}
+
 template <int BN, int EPI>
 static int launch_pair_t(const bf16* A, int64_t lda, const bf16* B, int64_t ldb, int M, int N, int K,
                          const GemmEpi& e, int* err, cudaStream_t s) {
@@ -893,8 +915,8 @@ static int launch_pair_t(const bf16* A, int64_t lda, const bf16* B, int64_t ldb,
   // the maps span every group's operand, as for the single-CTA kernels
   if ((rc = make_map(&ta, A, M + (int64_t)(G - 1) * e.a_row, K + (int64_t)(G - 1) * e.a_col, lda, tc::BM))) return rc;
   if ((rc = make_map(&tb, B, N + (int64_t)(G - 1) * e.b_row, K + (int64_t)(G - 1) * e.b_col, ldb, BN / 2))) return rc;
-  static int max_clusters = 0;
-  static bool configured = false;
+  static PerDevice limit, clusters;
+  const int dev = current_device();
   const int nkb = (K + P::KSUB * tc::BK - 1) / (P::KSUB * tc::BK);
   const int S = nkb < P::STAGES ? nkb : P::STAGES;
   const size_t smem = 1024 + (size_t)S * (P::A_BYTES + P::B_BYTES) + (2 * (size_t)S + 4) * 8 + 16 + 128 +
@@ -910,20 +932,17 @@ static int launch_pair_t(const bf16* A, int64_t lda, const bf16* B, int64_t ldb,
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (!configured) {
-    if ((rc = cuda_check(cudaFuncSetAttribute(gemm_bf16_pair<BN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)P::SMEM), "gemm pair smem attribute")))
-      return rc;
+  if ((rc = allow_smem(limit, dev, gemm_bf16_pair<BN, EPI>, P::SMEM, "gemm pair smem attribute"))) return rc;
+  const int max_clusters = clusters.get(dev, [&] {
     cudaLaunchConfig_t q = cfg;
     q.dynamicSmemBytes = P::SMEM;
     q.gridDim = dim3(2, 1, 1);
     int nc = 0;
-    if ((rc = cuda_check(cudaOccupancyMaxActiveClusters(&nc, gemm_bf16_pair<BN, EPI>, &q), "gemm pair occupancy")))
-      return rc;
-    if (nc <= 0) return set_error(CHEM_E_UNSUPPORTED, "gemm: no CTA pair fits on the device");
-    max_clusters = nc;
-    configured = true;
-  }
+    rc = cuda_check(cudaOccupancyMaxActiveClusters(&nc, gemm_bf16_pair<BN, EPI>, &q), "gemm pair occupancy");
+    return rc ? 0 : nc;
+  });
+  if (rc) return rc;
+  if (max_clusters <= 0) return set_error(CHEM_E_UNSUPPORTED, "gemm: no CTA pair fits on the device");
   const int64_t total = (int64_t)((N + BN - 1) / BN) * ((M + 2 * tc::BM - 1) / (2 * tc::BM)) * G;
   if (total > 0x7fffffff) return set_error(CHEM_E_ARG, "gemm: too many tiles in one call");
   const int ncl = (int)std::min<int64_t>(total, (int64_t)max_clusters);
@@ -952,38 +971,21 @@ static int launch_gemm_t(const bf16* A, int64_t lda, const bf16* B, int64_t ldb,
     }
     // long K: persistent warp-specialised kernel, one CTA per SM
     using P = PersistCfg<BN>;
-    static bool pconfigured = false;
-    if (!pconfigured) {
-      if ((rc = cuda_check(cudaFuncSetAttribute(gemm_bf16_persistent<BN, EPI>,
-                                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P::SMEM),
-                           "gemm smem attribute")))
-        return rc;
-      pconfigured = true;
-    }
+    static PerDevice plimit;
+    const int dev = current_device();
+    if ((rc = allow_smem(plimit, dev, gemm_bf16_persistent<BN, EPI>, P::SMEM, "gemm smem attribute"))) return rc;
     const int S = nkb_all < P::STAGES ? nkb_all : P::STAGES;
     const size_t smem = 1024 + (size_t)S * (P::A_BYTES + P::B_BYTES) + (2 * (size_t)S + 4) * 8 + 16 + 128 +
                         8 * (size_t)kEpiWarpBytes;
     const int64_t total = (int64_t)((N + BN - 1) / BN) * ((M + tc::BM - 1) / tc::BM) * G;
     if (total > 0x7fffffff) return set_error(CHEM_E_ARG, "gemm: too many tiles in one call");
-    static int sms = 0;
-    if (!sms) {
-      int dev = 0;
-      cudaGetDevice(&dev);
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-      if (sms <= 0) sms = 1;
-    }
-    const int grid = (int)std::min<int64_t>(total, (int64_t)sms);
+    const int grid = (int)std::min<int64_t>(total, (int64_t)sm_count(dev));
     gemm_bf16_persistent<BN, EPI><<<grid, 320, smem, s>>>(ta, tb, e, M, N, K, S, err);
     return cuda_check(cudaGetLastError(), "gemm_bf16_persistent launch");
   }
   using Cfg = TileCfg<BN>;
-  static bool configured = false;
-  if (!configured) {
-    if ((rc = cuda_check(cudaFuncSetAttribute(gemm_bf16_kernel<BN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)Cfg::SMEM), "gemm smem attribute")))
-      return rc;
-    configured = true;
-  }
+  static PerDevice limit;
+  if ((rc = allow_smem(limit, current_device(), gemm_bf16_kernel<BN, EPI>, Cfg::SMEM, "gemm smem attribute"))) return rc;
   const int nkb = (K + tc::BK - 1) / tc::BK;
   const int S = nkb < Cfg::STAGES ? nkb : Cfg::STAGES;
   const size_t smem = 1024 + (size_t)S * (Cfg::A_BYTES + Cfg::B_BYTES) + (2 * (size_t)S + 2) * 8 + 16 + 128 +
@@ -1082,17 +1084,10 @@ int wgrad_bf16(const WgradLayer* layers, int n, int R, int* err, cudaStream_t s)
   p.tile0[n] = (int)tiles;
   p.layers = n;
   p.nkb = (R + 63) / 64;
-  static bool configured = false;
-  if (!configured) {
-    if ((rc = cuda_check(cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)WgradCfg::SMEM), "wgrad smem attribute")))
-      return rc;
-    configured = true;
-  }
-  int dev = 0, sms = 1;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  wgrad_kernel<<<(int)std::min<int64_t>(tiles, sms), 256, WgradCfg::SMEM, s>>>(p, err);
+  static PerDevice limit;
+  const int dev = current_device();
+  if ((rc = allow_smem(limit, dev, wgrad_kernel, WgradCfg::SMEM, "wgrad smem attribute"))) return rc;
+  wgrad_kernel<<<(int)std::min<int64_t>(tiles, sm_count(dev)), 256, WgradCfg::SMEM, s>>>(p, err);
   return cuda_check(cudaGetLastError(), "wgrad_kernel launch");
 }
 
