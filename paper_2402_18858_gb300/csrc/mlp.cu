@@ -305,6 +305,14 @@ __device__ __forceinline__ void epi_gelu_x8(uint32_t taddr, int col0, int nq, co
   flush_rows_bf16(wbuf, (bf16*)e.out + (size_t)row0 * e.ldo + col0, e.ldo, nrows, nq, lane);
 }
 
+// Before a block gives up its shared memory: wait (bounded like every wait) until the copies of the last
+// slabs 0 .. sent - 1 have landed in the ring of S stages.  After a run without a failed wait they have (the
+// MMAs waited for each); after one they may still be on their way.
+__device__ __forceinline__ void drain(uint64_t* full, int S, int sent, int* err, int site) {
+  for (int e = max(0, sent - S); e < sent; ++e)
+    if (!tc::mbar_wait(&full[e % S], (e / S) & 1, err, site)) break;
+}
+
 // S (1..STAGES, a launch argument) stages in the ring: min(STAGES, K slabs), so that a
 // short K takes less shared memory and more CTAs share an SM
 template <int BN, int EPI>
@@ -393,6 +401,7 @@ __global__ void __launch_bounds__(256, 4) gemm_bf16_kernel(const __grid_constant
       __syncwarp();
     }
   }
+  if (!ok && threadIdx.x == 0) drain(full, S, nkb, err, 4);
   tc::tc_fence_before();
   __syncthreads();
   if (warp == 2) tc::tmem_dealloc(tmem, C::TMEM_COLS);
@@ -481,6 +490,7 @@ __global__ void __launch_bounds__(320, 1) gemm_bf16_persistent(const __grid_cons
         }
         if (stop) break;
       }
+      drain(full, S, g, err, 15);
     }
   } else if (warp == 1) {
     if (lane == 0) {
@@ -653,6 +663,7 @@ __global__ void __launch_bounds__(320, 1) gemm_bf16_pair(const __grid_constant__
         }
         if (stop) break;
       }
+      if (rank == 0) drain(full, S, g, err, 25);   // both CTAs' bytes; the odd one waits at the cluster barrier
     }
   } else if (warp == 1) {
     if (lane == 0 && rank == 0) {
@@ -783,6 +794,7 @@ __global__ void __launch_bounds__(256, 1) wgrad_kernel(const __grid_constant__ W
   tc::tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   int g = 0, it = 0, l = 0;   // slabs and tiles so far (the same in every role), layer
+  int sent = 0;               // slabs whose copies were issued (thread 0)
   for (int t = blockIdx.x; t < p.tile0[p.layers]; t += gridDim.x, ++it, g += p.nkb) {
     while (t >= p.tile0[l + 1]) ++l;
     const int M = p.M[l], N = p.N[l];
@@ -801,6 +813,7 @@ __global__ void __launch_bounds__(256, 1) wgrad_kernel(const __grid_constant__ W
 #pragma unroll
         for (int h = 0; h < kWgradBN / 64; ++h)
           tc::tma_load_2d(sB + s * C::B_BYTES + h * C::BOX, &p.tb[l], &full[s], bx + 64 * h, kb * 64);
+        sent = e + 1;
       }
     } else if (threadIdx.x == 32) {
       constexpr uint32_t idesc = tc::idesc_bf16_f32<tc::BM, kWgradBN, true>();
@@ -842,6 +855,7 @@ __global__ void __launch_bounds__(256, 1) wgrad_kernel(const __grid_constant__ W
     tc::tc_fence_after();
     if (!__syncthreads_and(ok && !gemm_failed(err))) break;
   }
+  if (threadIdx.x == 0) drain(full, C::STAGES, sent, err, 34);
   tc::tc_fence_before();
   __syncthreads();
   if (warp == 2) tc::tmem_dealloc(tmem, kWgradBN);
