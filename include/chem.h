@@ -436,7 +436,7 @@ int chem_selftest_di_form(chem_mech mech, int warps, int64_t n, int64_t ld, doub
                           int32_t* stats, void* workspace, size_t ws_bytes, chem_stream stream);
 
 /* Testing hook: y[i] = exp(x[i]) by the library's own FP64 exponential (the table-driven
- * method the kernels use), for comparison with CUDA's exp.  Device pointers, n >= 0. */
+ * method of the integration kernels), for comparison with CUDA's exp.  Device pointers, n >= 0. */
 int chem_selftest_exp(chem_mech mech, int64_t n, const double* x, double* y, chem_stream stream);
 
 /* Testing hook: y[i] = 2^(x[i]/256) = exp(x[i] ln2/256) by the library's FP64 exponential of
@@ -449,6 +449,11 @@ int chem_selftest_exp256(chem_mech mech, int64_t n, const double* x, double* y, 
  * the kernels use for ln T and the falloff logarithms), for comparison with CUDA's log.  Device
  * pointers, n >= 0. */
 int chem_selftest_log(chem_mech mech, int64_t n, const double* x, double* y, chem_stream stream);
+
+/* Testing hook: the 64-bit fixed-point forms of the same functions, which the rates and the FP64
+ * properties use: which 0: exp(x); 1: 2^(x/256); 2: 2^(-x/256) from the negated fixed-point argument, for
+ * |x| < 261485; 3: log(x).  Device pointers, n >= 0. */
+int chem_selftest_fix(chem_mech mech, int which, int64_t n, const double* x, double* y, chem_stream stream);
 
 /* Testing hook: y[i] = 1/x[i] by the library's own FP64 reciprocal (hardware estimate plus one
  * third-order refinement step, used for every reciprocal of the integration and property

@@ -804,6 +804,14 @@ int chem_selftest_log(chem_mech m, int64_t n, const double* x, double* y, chem_s
   return launch_log_selftest(m->dev, n, x, y, (cudaStream_t)stream);
 }
 
+int chem_selftest_fix(chem_mech m, int which, int64_t n, const double* x, double* y, chem_stream stream) {
+  int rc = check_mech(m);
+  if (rc) return rc;
+  if (which < 0 || which > 3 || n < 0 || (n > 0 && (!x || !y))) return set_error(CHEM_E_ARG, "chem_selftest_fix: bad arguments");
+  if (n == 0) return CHEM_OK;
+  return launch_fix_selftest(m->dev, which, n, x, y, (cudaStream_t)stream);
+}
+
 int chem_selftest_rcp(int64_t n, const double* x, double* y, chem_stream stream) {
   if (n < 0 || (n > 0 && (!x || !y))) return set_error(CHEM_E_ARG, "chem_selftest_rcp: bad arguments");
   if (n == 0) return CHEM_OK;

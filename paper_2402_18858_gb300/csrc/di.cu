@@ -1489,6 +1489,18 @@ __global__ void log_selftest_kernel(const double* __restrict__ tab, int64_t n, c
     y[i] = log_t(x[i], tab);
 }
 
+// the fixed-point forms of rates and properties: exp(x), 2^(x/256), its reciprocal by the negated fixed-point
+// argument (as the right-hand side takes both from one), log(x)
+__global__ void fix_selftest_kernel(DevMech m, int which, int64_t n, const double* x, double* y) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const double v = x[i];
+    if (which == 0) y[i] = exp_t_fix(v, m.fexptab);
+    else if (which == 1) y[i] = exp_s256_fix(v, m.fexptab);
+    else if (which == 2) y[i] = exp2_fix(-fix_s256(v), m.fexptab);
+    else y[i] = log_t_fix(v, m.flogtab);
+  }
+}
+
 __global__ void rcp_selftest_kernel(int64_t n, const double* x, double* y) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     y[i] = rcp_nr(x[i]);
@@ -1501,6 +1513,12 @@ int launch_rcp_selftest(int64_t n, const double* x, double* y, cudaStream_t s) {
   const int64_t blocks = std::min<int64_t>((n + 255) / 256, 4096);
   rcp_selftest_kernel<<<(int)blocks, 256, 0, s>>>(n, x, y);
   return cuda_check(cudaGetLastError(), "rcp_selftest_kernel launch");
+}
+
+int launch_fix_selftest(const DevMech& m, int which, int64_t n, const double* x, double* y, cudaStream_t s) {
+  const int64_t blocks = std::min<int64_t>((n + 255) / 256, 4096);
+  fix_selftest_kernel<<<(int)blocks, 256, 0, s>>>(m, which, n, x, y);
+  return cuda_check(cudaGetLastError(), "fix_selftest_kernel launch");
 }
 
 int launch_exp_selftest(const DevMech& m, int64_t n, const double* x, double* y, cudaStream_t s) {

@@ -248,10 +248,10 @@ __device__ __forceinline__ double log_t(double x, const double* __restrict__ tab
 // and 2 FP64 ones for a logarithm (12 before).  The method is the table-driven one of P. T. P. Tang
 // ("Table-driven implementation of the exponential function in IEEE floating-point arithmetic", ACM
 // TOMS 15, 1989; "... of the logarithm function ...", ACM TOMS 16, 1990): a short table and the
-// Taylor polynomial of a small remainder.  With 63 fraction bits the only rounding that counts is
-// the last one: worst errors over the ranges of use 0.55 ulp (exponentials; 1.2 ulp where the
-// argument is within one table step of 0) and 0.92 ulp (logarithm), against 2 ulp of the FP64
-// forms.  Against those (same inputs): rates of 200,000 30-species cells 2,715 -> 2,132 us, FP64
+// Taylor polynomial of a small remainder.  With 63 fraction bits the only roundings that count are
+// the last one and the cutting of the argument.  Worst errors: 2^(x/256) 0.54 ulp from |x| = 256 on, where the
+// argument is exact, and 1.15 below; exp 1.25 ulp from |x| = 1 on and 2.0 below; logarithm 0.92 ulp; against 2
+// ulp of the FP64 forms.  Against those (same inputs): rates of 200,000 30-species cells 2,715 -> 2,132 us, FP64
 // properties of 1 M cells 7,560 -> 6,489 us.
 // ------------------------------------------------------------------------------------------
 
@@ -483,6 +483,7 @@ size_t di_smem_per_warp(const DevMech& m);
 int launch_rcp_selftest(int64_t n, const double* x, double* y, cudaStream_t s);
 int launch_exp_selftest(const DevMech& m, int64_t n, const double* x, double* y, cudaStream_t s);
 int launch_exp256_selftest(const DevMech& m, int64_t n, const double* x, double* y, cudaStream_t s);
+int launch_fix_selftest(const DevMech& m, int which, int64_t n, const double* x, double* y, cudaStream_t s);
 int launch_log_selftest(const DevMech& m, int64_t n, const double* x, double* y, cudaStream_t s);
 
 // thermo.cu
