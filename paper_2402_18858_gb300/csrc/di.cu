@@ -19,8 +19,9 @@
 // of L1 the mechanism tables come from L2, so they are laid out for contiguous warp loads, the
 // triangular solves issue the loads of four factor columns ahead of the FP64 chain, and 12 warps per SM
 // (3 per sub-partition) are resident.  Same bits; 150 30-species cells (one warp per SM, tables in
-// L1): 22.3 -> 18.0 ms; 3,001 53-species cells: 145.7 -> 138 ms; 12,345 30-species cells: 137.7 ->
-// 134.8 ms (FP64 issue bound).
+// L1): 23.2 -> 18.7 ms (14.7 with teams); 3,001 53-species cells: 148 -> 143 ms (138 with teams);
+// 12,345 30-species cells: 138.9 -> 136 ms (FP64 pipe 78 % busy at 8,202 cells; 9 species 69 %, 53
+// species 57 %).
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -379,7 +380,9 @@ __device__ __forceinline__ double entry_nu(unsigned int e) {
 }
 
 // ------------------------------------------------------------------------------------------
-// Teams: TW warps on one cell (150 cells of 30 species 18.7 -> 14.6 ms, 3001 of 53 species 141 -> 136 ms), for launches with few cells (one warp alone keeps one of the SM's four
+// Teams: TW warps on one cell (150 cells of 30 species 18.7 -> 14.7 ms, 3,001 of 53 species 143 -> 138 ms; the form
+// for two warps above 32 unknowns spills 164 bytes at its 168 registers, and four blocks without spills are
+// slower than five with, 142.7 against 136.1 ms), for launches with few cells (one warp alone keeps one of the SM's four
 // FP64 units busy, and that half of the time: 48 thousand cycles per BDF step, of which 27 in the
 // right-hand side) and for mechanisms whose shared memory leaves few warps per SM.  Warp 0 integrates;
 // the others wait for its right-hand sides and take: warp 1 the falloff reactions with the

@@ -197,12 +197,13 @@ __global__ void __launch_bounds__(128) thermo_kernel(DevMech m, int64_t n, int64
 // entries as two limbs (55 bits relative to the largest of the vector), three 32 x 32 + 64-bit
 // multiply-adds (4 cycles each) per term, exact 64-bit sums, rounded once when they return to FP64.
 // About 25 FP64 operations per species are left (c_p and h sums, transport fits, products,
-// reciprocals).  1 M cells, 30 species: 6.49 -> 2.31 ms (8.96 -> 2.75 ms with T from h); 400,000 cells,
+// reciprocals).  1 M cells, 30 species: 6.49 -> 2.27 ms (8.96 -> 2.75 ms with T from h); 400,000 cells,
 // 53 species: 8.23 -> 2.76 ms.  Errors against 64 bits no larger than the FP64 form's: viscosity
 // 7.3e-16 (7.7e-16), c_p 1.4e-16 (1.5e-16), conductivity 3.2e-16 (4.8e-16).
 //
 // Layout: SPLIT threads per cell (1 for K <= 9, 2 above: two threads with 15 species each need 128
-// registers and hide more latency than one with 30 at 255, 2.48 -> 2.09 ms), thread h of a cell keeping
+// registers, 128 bytes of them spilled, and hide more latency than one with 30 at 255: 2.48 -> 2.09 ms before the
+// limbs were rounded instead of cut), thread h of a cell keeping
 // the limbs of species h JC .. h JC + JC - 1 in registers (JC compile-time: every index is static);
 // rows of C are read as broadcasts from shared memory.  With two threads the halves' sums of a row are
 // exchanged and each finishes every other row.  The exponentials stay in a rolled loop: unrolled over
