@@ -196,6 +196,33 @@ using namespace chem;
 const DevMech& chem::mech_dev(chem_mech m) { return m->dev; }
 
 // Pack the host mechanism into one device allocation and point DevMech at its pieces.
+// tables of the elementary functions, FP64 and fixed point (see internal.h): the same for every mechanism,
+// made at the first load (long double logarithms are software on some hosts, 0.2 ms of every load)
+struct FnTables {
+  std::vector<double> exptab, logtab;
+  std::vector<unsigned long long> fexptab;
+  std::vector<long long> flogtab;
+  FnTables() : exptab(256), logtab(3 * 97), fexptab(256), flogtab(2 * 97) {
+    for (int j = 0; j < 256; ++j) {
+      const long double e = std::exp2((long double)j / 256.0L);
+      exptab[j] = (double)e;
+      fexptab[j] = (unsigned long long)std::round(std::ldexp(e, 63));
+    }
+    for (int j = 96; j <= 192; ++j) {
+      const long double F = (long double)j / 128.0L, G = std::round(1024.0L / F);
+      logtab[3 * (j - 96)] = (double)F;
+      logtab[3 * (j - 96) + 1] = (double)(1.0L / F);
+      logtab[3 * (j - 96) + 2] = (double)std::log(F);
+      flogtab[2 * (j - 96)] = (long long)G;
+      flogtab[2 * (j - 96) + 1] = (long long)std::round(std::ldexp(-std::log(G / 1024.0L), 63));
+    }
+  }
+};
+static const FnTables& fn_tables() {
+  static const FnTables t;
+  return t;
+}
+
 static int upload(const HostMech& hm, chem_mech_s* cm) {
   const int K = (int)hm.species.size(), I = (int)hm.rxn.size();
   // order reactions by kind
@@ -379,23 +406,7 @@ static int upload(const HostMech& hm, chem_mech_s* cm) {
       for (int i = 0; i < 7; ++i) gneg[((size_t)(rg * 4 + i / 2) * KP + k) * 2 + i % 2] = (double)(-c[i] * kExpScale);
     }
   }
-  // tables of the elementary functions, FP64 and fixed point (see internal.h)
-  std::vector<double> exptab(256), logtab(3 * 97);
-  std::vector<unsigned long long> fexptab(256);
-  std::vector<long long> flogtab(2 * 97);
-  for (int j = 0; j < 256; ++j) {
-    const long double e = std::exp2((long double)j / 256.0L);
-    exptab[j] = (double)e;
-    fexptab[j] = (unsigned long long)std::round(std::ldexp(e, 63));
-  }
-  for (int j = 96; j <= 192; ++j) {
-    const long double F = (long double)j / 128.0L, G = std::round(1024.0L / F);
-    logtab[3 * (j - 96)] = (double)F;
-    logtab[3 * (j - 96) + 1] = (double)(1.0L / F);
-    logtab[3 * (j - 96) + 2] = (double)std::log(F);
-    flogtab[2 * (j - 96)] = (long long)G;
-    flogtab[2 * (j - 96) + 1] = (long long)std::round(std::ldexp(-std::log(G / 1024.0L), 63));
-  }
+  const FnTables& fn = fn_tables();
   std::vector<double> rth((size_t)2 * 12 * KP, 0.0);
   for (int rg = 0; rg < 2; ++rg)
     for (int i = 0; i < 11; ++i)
@@ -543,9 +554,9 @@ static int upload(const HostMech& hm, chem_mech_s* cm) {
   size_t ofxt = add(fx_tr.data(), fx_tr.size() * 8);
   size_t oth32 = add(th32.data(), th32.size() * 4), oiw32 = add(invW32.data(), invW32.size() * 4);
   size_t ocw32 = add(compW32.data(), compW32.size() * 4);
-  size_t oexp = add(exptab.data(), exptab.size() * 8), ocw = add(compW.data(), compW.size() * 8);
-  size_t oxa = add(xarg.data(), xarg.size() * 8), olog = add(logtab.data(), logtab.size() * 8);
-  size_t ofexp = add(fexptab.data(), fexptab.size() * 8), oflog = add(flogtab.data(), flogtab.size() * 8);
+  size_t oexp = add(fn.exptab.data(), fn.exptab.size() * 8), ocw = add(compW.data(), compW.size() * 8);
+  size_t oxa = add(xarg.data(), xarg.size() * 8), olog = add(fn.logtab.data(), fn.logtab.size() * 8);
+  size_t ofexp = add(fn.fexptab.data(), fn.fexptab.size() * 8), oflog = add(fn.flogtab.data(), fn.flogtab.size() * 8);
   size_t obal = add(bal.data(), bal.size() * 4), orun = add(run_ptr.data(), run_ptr.size() * 4);
   size_t orsp2 = add(rsp2.data(), rsp2.size() * 4);
   size_t otb[2] = {add(tb_e[0].data(), tb_e[0].size() * 4), add(tb_e[1].data(), tb_e[1].size() * 4)};
